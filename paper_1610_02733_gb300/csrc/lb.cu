@@ -7,8 +7,8 @@
 // force density F = J_acc / tau_LB + g; the post-collision populations are
 // pushed to the neighbours r + c_i in the other buffer.
 //
-// forcing_update_kernel (variant C): after every MD step, the transfer of
-// that step enters the populations through the forcing part of the collision.
+// Variant C: the transfers of the MD steps enter the populations through the
+// forcing part of the collision (apply_transfer), once per LB step.
 //
 // The post-stream moments rho* and j* of the freshly streamed populations
 // (the node field the MD steps of the next LB cycle read and, in variant B,
@@ -31,9 +31,9 @@ struct LbArgs {
     T rho_base;  // deviation storage: sum_i of the stored rest values w_i rho0
     typename Prec<T>::node4 *node;
     typename Prec<T>::node4 *jacc;
-    const uint2 *occw;                     // variant B: active nodes of this cycle
-    const typename Prec<T>::node4 *cact;   // variant B: their compact records
-    const uint2 *occw_new;                 // variant B: active nodes of the next cycle
+    const uint2 *occw;                     // active nodes of this cycle
+    const typename Prec<T>::node4 *cact;   // their compact records
+    const uint2 *occw_new;                 // active nodes of the next cycle
     typename Prec<T>::node4 *cact_new;     // ... whose records the fused moments write
     typename Prec<T>::node4 *cact_new2;    // variant A with a frozen copy: the same records again
     int occ_words;
@@ -85,12 +85,10 @@ __device__ __forceinline__ void node_moments_at(const S *f, typename Prec<T>::no
     pop_moments<St::deviation>(fl, rho_base, rho, rho_m, jx, jy, jz);
     const typename P::node4 rec = guarded_record(rho, jx, jy, jz, fs, range_flag);
     node[r] = rec;
-    if (occw) {
-        const int sl = active_slot(occw[((size_t)y + (size_t)ny * t) * occ_words + (x >> 5)], x);
-        if (sl >= 0) {
-            cact[sl] = rec;
-            if (cact2) cact2[sl] = rec;
-        }
+    const int sl = active_slot(occw[((size_t)y + (size_t)ny * t) * occ_words + (x >> 5)], x);
+    if (sl >= 0) {
+        cact[sl] = rec;
+        if (cact2) cact2[sl] = rec;
     }
 }
 
@@ -111,7 +109,9 @@ constexpr int FUSE_LAG = 2;
 // agree bit for bit, as the paper's algorithmic equivalence requires.
 // Collide node (x, y, z) and push its post-collision populations to the
 // neighbours r + c_i in the other buffer.
-template <typename T, typename S, bool RELAX_FULL, bool GAUSS>
+// C (variant C, a kernel instance of its own): the cycle's transfers enter the
+// populations first, then the collision sees the body force only.
+template <typename T, typename S, bool RELAX_FULL, bool GAUSS, bool C>
 __device__ __forceinline__ void collide_push_node(const LbArgs<T, S> &a, int x, int y, int z,
                                                   unsigned long long step) {
     using P = Prec<T>;
@@ -123,17 +123,17 @@ __device__ __forceinline__ void collide_push_node(const LbArgs<T, S> &a, int x, 
     T rho, rho_m, jx, jy, jz;
     pop_moments<St::deviation>(f, a.rho_base, rho, rho_m, jx, jy, jz);
     T Fx, Fy, Fz;
-    const int sl = a.occw ? active_slot(a.occw[((size_t)y + (size_t)a.ny * z) * a.occ_words + (x >> 5)], x) : -1;
-    if (sl >= 0 || a.variant == LBMD_VARIANT_B) {
+    const int sl = active_slot(a.occw[((size_t)y + (size_t)a.ny * z) * a.occ_words + (x >> 5)], x);
+    if (C || sl >= 0 || a.variant == LBMD_VARIANT_B) {
         // the record j = fix(j*) + sum of fixed-point transfers: the
         // difference is exactly the accumulated transfer J_acc (an active
         // node's record is its compact one -- variant A: the accumulating
-        // copy; B: an inactive node's is the node field)
+        // copy; B and C: an inactive node's is the node field)
         const typename P::node4 n = sl >= 0 ? a.cact[sl] : a.node[r];
         Fx = P::from_fix(P::jx_of(n) - P::to_fix(jx, a.fs), a.fis);
         Fy = P::from_fix(P::jy_of(n) - P::to_fix(jy, a.fs), a.fis);
         Fz = P::from_fix(P::jz_of(n) - P::to_fix(jz, a.fs), a.fis);
-    } else if (a.occw) {
+    } else {
         // variant A, inactive node: J_acc holds what migrants handed over
         // (rarely anything; cleared only where set)
         const typename P::node4 J = a.jacc[r];
@@ -145,14 +145,11 @@ __device__ __forceinline__ void collide_push_node(const LbArgs<T, S> &a, int x, 
             zero.x = zero.y = zero.z = zero.w = 0;
             a.jacc[r] = zero;
         }
-    } else {
-        const typename P::node4 J = a.jacc[r];
-        Fx = P::from_fix(P::jx_of(J), a.fis);
-        Fy = P::from_fix(P::jy_of(J), a.fis);
-        Fz = P::from_fix(P::jz_of(J), a.fis);
-        typename P::node4 zero;
-        zero.x = zero.y = zero.z = zero.w = 0;
-        a.jacc[r] = zero;
+    }
+    if (C && !(Fx == T(0) && Fy == T(0) && Fz == T(0))) {
+        apply_transfer(f, rho, jx, jy, jz, Fx, Fy, Fz, a.gamma_bulk, a.gamma_shear);
+        pop_moments<St::deviation>(f, a.rho_base, rho, rho_m, jx, jy, jz);
+        Fx = Fy = Fz = T(0);
     }
     Fx += a.g[0];
     Fy += a.g[1];
@@ -193,19 +190,20 @@ __device__ __forceinline__ void collide_push_node(const LbArgs<T, S> &a, int x, 
 // despite their spills: FP32 cycle -0.8 %, FP16 / BF16 LB step -6.5 % /
 // -4.3 %; the stochastic-rounding form measured slower at 7, and it and the
 // Gaussian-noise and partial-relaxation forms keep 6 (3 in FP64).
-template <typename T, typename S, bool RELAX_FULL, bool GAUSS>
+template <typename T, typename S, bool RELAX_FULL, bool GAUSS, bool C>
 constexpr int collide_min_blocks() {
-    return sizeof(T) == 8 ? 3 : (RELAX_FULL && !GAUSS && !PopStore<S, T>::stochastic ? 7 : 6);
+    return sizeof(T) == 8 ? 3 : C ? 5 : (RELAX_FULL && !GAUSS && !PopStore<S, T>::stochastic ? 7 : 6);
 }
 
-template <typename T, typename S, bool RELAX_FULL, bool GAUSS>
-__global__ void __launch_bounds__(256, (collide_min_blocks<T, S, RELAX_FULL, GAUSS>())) lb_collide_push(LbArgs<T, S> a) {
+template <typename T, typename S, bool RELAX_FULL, bool GAUSS, bool C>
+__global__ void __launch_bounds__(256, (collide_min_blocks<T, S, RELAX_FULL, GAUSS, C>()))
+    lb_collide_push(LbArgs<T, S> a) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
     // the step counter, read before the fallback kernel advances it; it also
     // tags the blocks that have pushed
     const unsigned long long step = *a.lb_step;
-    if (x < a.nx) collide_push_node<T, S, RELAX_FULL, GAUSS>(a, x, y, z, step);
+    if (x < a.nx) collide_push_node<T, S, RELAX_FULL, GAUSS, C>(a, x, y, z, step);
 
     // fused post-stream moments: publish this block, then compute the
     // moments of the block FUSE_LAG planes back once its neighbourhood is in
@@ -299,64 +297,6 @@ __global__ void __launch_bounds__(256)
                           blockIdx.z);
 }
 
-// Variant C (Sec. 4): the momentum transfer F = J_acc of the MD step just
-// done enters the populations through the forcing part of the collision
-// alone: mass unchanged, momentum + F, stress modes + (1 + gamma) times the
-// symmetric products of u = (j + F/2)/rho and F (as in collide()), ghost
-// modes unchanged; then the node record is recomputed from the populations
-// and J_acc is cleared.  Nodes without a transfer are left as they are.
-template <typename T, typename S>
-__global__ void __launch_bounds__(256) forcing_update_kernel(S *__restrict__ f, typename Prec<T>::node4 *node,
-                                                             typename Prec<T>::node4 *jacc, int64_t N, T rho_base,
-                                                             T gamma_bulk, T gamma_shear, T fix_s, T fix_is,
-                                                             int32_t *range_flag) {
-    using P = Prec<T>;
-    using St = PopStore<S, T>;
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= N) return;
-    const typename P::node4 J = jacc[r];
-    if (P::jx_of(J) == 0 && P::jy_of(J) == 0 && P::jz_of(J) == 0) return;
-    const T Fx = P::from_fix(P::jx_of(J), fix_is), Fy = P::from_fix(P::jy_of(J), fix_is),
-            Fz = P::from_fix(P::jz_of(J), fix_is);
-    T fl[Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) fl[i] = St::arith(f + (int64_t)i * N + r);
-    T rho, rho_m, jx, jy, jz;
-    pop_moments<St::deviation>(fl, rho_base, rho, rho_m, jx, jy, jz);
-    const T ir = T(1) / rho;
-    const T ux = (jx + T(0.5) * Fx) * ir, uy = (jy + T(0.5) * Fy) * ir, uz = (jz + T(0.5) * Fz) * ir;
-    const T uF = ux * Fx + uy * Fy + uz * Fz;
-    T dm[Q];
-#pragma unroll
-    for (int k = 0; k < Q; ++k) dm[k] = T(0);
-    dm[1] = Fx;
-    dm[2] = Fy;
-    dm[3] = Fz;
-    const T fb = T(1) + gamma_bulk, fs = T(1) + gamma_shear;
-    dm[4] = fb * uF;
-    dm[5] = fs * (T(3) * ux * Fx - uF);
-    dm[6] = fs * (uy * Fy - uz * Fz);
-    dm[7] = fs * T(0.5) * (ux * Fy + uy * Fx);
-    dm[8] = fs * T(0.5) * (ux * Fz + uz * Fx);
-    dm[9] = fs * T(0.5) * (uy * Fz + uz * Fy);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        T acc = T(0);
-#pragma unroll
-        for (int k = 1; k <= 9; ++k) {
-            const int e = EMODE(k, i);
-            if (e != 0) acc += T(e) * dm[k] * T(INV_BNORM(k));
-        }
-        fl[i] += T(WEIGHT(i)) * acc;
-        St::store_arith(f + (int64_t)i * N + r, fl[i]);
-    }
-    pop_moments<St::deviation>(fl, rho_base, rho, rho_m, jx, jy, jz);
-    node[r] = guarded_record(rho, jx, jy, jz, fix_s, range_flag);
-    typename P::node4 zero;
-    zero.x = zero.y = zero.z = zero.w = 0;
-    jacc[r] = zero;
-}
-
 template <typename T, typename S>
 __global__ void init_equilibrium_kernel(S *f, int64_t N, T rho0) {
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -374,15 +314,21 @@ static dim3 node_grid(const lbmd_ctx *ctx, dim3 block) {
     return dim3((ctx->p.nx + block.x - 1) / block.x, ctx->p.ny, ctx->p.nz);
 }
 
-// Deviation storage: the density of the stored rest values, sum_i b_i with
-// b_i = w_i rho0 formed in T as the kernels form it (0 for the plain forms,
-// whose arithmetic is on the populations themselves).
-template <typename T, typename S>
-static T rest_density(const lbmd_ctx *ctx) {
-    if (!PopStore<S, T>::deviation) return T(0);
-    double sum = 0.0;
-    for (int i = 0; i < Q; ++i) sum += (double)(T(WEIGHT(i)) * (T)ctx->p.rho0);
-    return (T)sum;
+// Normal variates and variant C are kernel instances of their own, so that
+// the default one keeps its registers; neither combines with the storage
+// forms that lbmd_create refuses them for.
+template <typename T, typename S, bool FULL>
+static void launch_collide(lbmd_ctx *ctx, const LbArgs<T, S> &a, dim3 grid, dim3 block) {
+    const bool gauss = ctx->p.noise == LBMD_NOISE_GAUSS, c = ctx->p.variant == LBMD_VARIANT_C;
+    cudaStream_t st = ctx->stream;
+    if constexpr (!PopStore<S, T>::deviation) {
+        if (gauss && c) return lb_collide_push<T, S, FULL, true, true><<<grid, block, 0, st>>>(a);
+        if (gauss) return lb_collide_push<T, S, FULL, true, false><<<grid, block, 0, st>>>(a);
+    }
+    if constexpr (!PopStore<S, T>::stochastic) {
+        if (c) return lb_collide_push<T, S, FULL, false, true><<<grid, block, 0, st>>>(a);
+    }
+    lb_collide_push<T, S, FULL, false, false><<<grid, block, 0, st>>>(a);
 }
 
 template <typename T, typename S>
@@ -393,11 +339,10 @@ static cudaError_t lb_step_t(lbmd_ctx *ctx) {
     a.rho_base = rest_density<T, S>(ctx);
     a.node = static_cast<typename Prec<T>::node4 *>(ctx->node);
     a.jacc = static_cast<typename Prec<T>::node4 *>(ctx->jacc);
-    const bool B = compact_nodes(ctx);  // variants A and B
-    a.occw = B ? active_words_now(ctx) : nullptr;
-    a.cact = static_cast<const typename Prec<T>::node4 *>(B ? active_records_acc(ctx) : nullptr);
-    a.occw_new = B ? active_words_next(ctx) : nullptr;
-    a.cact_new = static_cast<typename Prec<T>::node4 *>(B ? active_records_next(ctx) : nullptr);
+    a.occw = active_words_now(ctx);
+    a.cact = static_cast<const typename Prec<T>::node4 *>(active_records_acc(ctx));
+    a.occw_new = active_words_next(ctx);
+    a.cact_new = static_cast<typename Prec<T>::node4 *>(active_records_next(ctx));
     a.cact_new2 = static_cast<typename Prec<T>::node4 *>(active_records_copy(ctx, (int)((ctx->lb_step + 1) & 1)));
     a.occ_words = active_words(ctx->p.nx);
     a.blk_done = ctx->blk_done;
@@ -428,22 +373,10 @@ static cudaError_t lb_step_t(lbmd_ctx *ctx) {
     cudaError_t e = cudaMemsetAsync(ctx->lb_missed, 0, sizeof(int32_t), ctx->stream);
     if (e != cudaSuccess) return e;
     const bool full = ctx->co.gamma_bulk == 0.0 && ctx->co.gamma_ghost == 0.0;
-    // normal variates: a kernel instance of its own (FP32 / FP64 storage),
-    // so that the default one keeps its registers
-    if constexpr (!PopStore<S, T>::deviation) {
-        if (ctx->p.noise == LBMD_NOISE_GAUSS) {
-            if (full)
-                lb_collide_push<T, S, true, true><<<grid, block, 0, ctx->stream>>>(a);
-            else
-                lb_collide_push<T, S, false, true><<<grid, block, 0, ctx->stream>>>(a);
-        }
-    }
-    if (ctx->p.noise != LBMD_NOISE_GAUSS) {
-        if (full)
-            lb_collide_push<T, S, true, false><<<grid, block, 0, ctx->stream>>>(a);
-        else
-            lb_collide_push<T, S, false, false><<<grid, block, 0, ctx->stream>>>(a);
-    }
+    if (full)
+        launch_collide<T, S, true>(ctx, a, grid, block);
+    else
+        launch_collide<T, S, false>(ctx, a, grid, block);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // the moments the collide kernel left, on the new populations
     moments_rest_kernel<T, S><<<2 * ctx->sm_count, block, 0, ctx->stream>>>(
@@ -458,24 +391,12 @@ static cudaError_t lb_step_t(lbmd_ctx *ctx) {
 template <typename T, typename S>
 static cudaError_t node_moments_t(lbmd_ctx *ctx) {
     const dim3 block = node_block(ctx), grid = node_grid(ctx, block);
-    const bool B = compact_nodes(ctx);  // variants A and B
     node_moments_kernel<T, S><<<grid, block, 0, ctx->stream>>>(
         static_cast<const S *>(ctx->f[ctx->cur]), static_cast<typename Prec<T>::node4 *>(ctx->node),
-        B ? active_words_now(ctx) : nullptr,
-        static_cast<typename Prec<T>::node4 *>(B ? active_records_now(ctx) : nullptr),
+        active_words_now(ctx), static_cast<typename Prec<T>::node4 *>(active_records_now(ctx)),
         static_cast<typename Prec<T>::node4 *>(active_records_copy(ctx, (int)(ctx->lb_step & 1))),
         active_words(ctx->p.nx), ctx->N, ctx->p.nx, ctx->p.ny, rest_density<T, S>(ctx), (T)ctx->fix.scale,
         ctx->range_flag);
-    return cudaGetLastError();
-}
-
-template <typename T, typename S>
-static cudaError_t forcing_update_t(lbmd_ctx *ctx) {
-    const unsigned blocks = (unsigned)((ctx->N + 255) / 256);
-    forcing_update_kernel<T, S><<<blocks, 256, 0, ctx->stream>>>(
-        static_cast<S *>(ctx->f[ctx->cur]), static_cast<typename Prec<T>::node4 *>(ctx->node),
-        static_cast<typename Prec<T>::node4 *>(ctx->jacc), ctx->N, rest_density<T, S>(ctx), (T)ctx->co.gamma_bulk,
-        (T)ctx->co.gamma_shear, (T)ctx->fix.scale, (T)ctx->fix.inv_scale, ctx->range_flag);
     return cudaGetLastError();
 }
 
@@ -518,5 +439,3 @@ cudaError_t launch_lb_step(lbmd_ctx *ctx) {
 cudaError_t launch_node_moments(lbmd_ctx *ctx, bool) { return LBMD_DISPATCH_POPS(ctx, lbmd::node_moments_t, ctx); }
 
 cudaError_t launch_init_equilibrium(lbmd_ctx *ctx) { return LBMD_DISPATCH_POPS(ctx, lbmd::init_equilibrium_t, ctx); }
-
-cudaError_t launch_forcing_update(lbmd_ctx *ctx) { return LBMD_DISPATCH_POPS(ctx, lbmd::forcing_update_t, ctx); }

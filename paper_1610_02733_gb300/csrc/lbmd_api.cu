@@ -187,7 +187,6 @@ lbmd_status lbmd_create(const lbmd_params *p, lbmd_ctx **out) {
     ctx->cact_cap = std::min<int64_t>(N, 8 * maxp);
     const size_t occ_bytes = (size_t)p->ny * p->nz * (size_t)((p->nx + 31) / 32) * sizeof(uint2);
     const size_t arow_bytes = ((size_t)p->ny * p->nz + 1) * sizeof(int32_t);
-    const bool compact = compact_nodes(ctx);  // variants A and B: compact records of the active nodes
     ctx->node_bytes = node_bytes;
     // the tiled MD step's tables and buffers, where the lattice suits it and
     // the spread mode asks for it
@@ -203,7 +202,7 @@ lbmd_status lbmd_create(const lbmd_params *p, lbmd_ctx **out) {
         {&ctx->f[0], (size_t)19 * N * pop_size(ctx)},
         {&ctx->f[1], (size_t)19 * N * pop_size(ctx)},
         {&ctx->node, (size_t)N * node_bytes},
-        {&ctx->jacc, p->variant != LBMD_VARIANT_B ? (size_t)N * node_bytes : 0},
+        {&ctx->jacc, p->variant == LBMD_VARIANT_A ? (size_t)N * node_bytes : 0},
         {&ctx->pos4[0], (size_t)maxp * 4 * rs},
         {&ctx->pos4[1], (size_t)maxp * 4 * rs},
         {&ctx->vel4[0], (size_t)maxp * 4 * rs},
@@ -222,14 +221,14 @@ lbmd_status lbmd_create(const lbmd_params *p, lbmd_ctx **out) {
         {(void **)&ctx->migrant_count, 2 * sizeof(int32_t)},
         {&ctx->fc4[0], (size_t)maxp * 4 * rs},
         {&ctx->fc4[1], (size_t)maxp * 4 * rs},
-        {&ctx->old4, compact ? (size_t)maxp * 4 * rs : 0},
-        {(void **)&ctx->occw[0], compact ? occ_bytes : 0},
-        {(void **)&ctx->occw[1], compact ? occ_bytes : 0},
-        {&ctx->cact[0], compact ? (size_t)2 * ctx->cact_cap * node_bytes : 0},
-        {&ctx->cact[1], compact ? (size_t)2 * ctx->cact_cap * node_bytes : 0},
-        {(void **)&ctx->arow[0], compact ? arow_bytes : 0},
-        {(void **)&ctx->arow[1], compact ? arow_bytes : 0},
-        {(void **)&ctx->ccw, compact ? occ_bytes / 2 : 0},
+        {&ctx->old4, (size_t)maxp * 4 * rs},
+        {(void **)&ctx->occw[0], occ_bytes},
+        {(void **)&ctx->occw[1], occ_bytes},
+        {&ctx->cact[0], (size_t)2 * ctx->cact_cap * node_bytes},
+        {&ctx->cact[1], (size_t)2 * ctx->cact_cap * node_bytes},
+        {(void **)&ctx->arow[0], arow_bytes},
+        {(void **)&ctx->arow[1], arow_bytes},
+        {(void **)&ctx->ccw, occ_bytes / 2},
         {(void **)&ctx->dev_error, sizeof(int32_t)},
         {&ctx->tile_table[0], table_bytes},
         {&ctx->tile_table[1], table_bytes},

@@ -6,9 +6,9 @@
 //   node        node field, one 16-byte (FP32) / 32-byte (FP64) record per
 //               node: rho* as bits and the momentum density j in fixed point.
 //               Variant A: j* of the last LB update (frozen during the MD
-//               steps).  Variant B: j* plus every transfer since.
-//   jacc        variants A and C: the transfers since the last LB step (C:
-//               since the last MD step), fixed point, 4 words per node.
+//               steps).  Variants B and C: j* plus every transfer since.
+//   jacc        variant A: the transfers to inactive nodes since the last LB
+//               step, fixed point, 4 words per node.
 //   Particles live in "slots".  Once per LB step they are re-ordered by
 //   lattice row (y, z) of their cell, so that the particles a warp handles
 //   touch neighbouring nodes (cache locality of the corner reads and
@@ -216,16 +216,15 @@ inline void *active_records_other(const lbmd_ctx *c) {
 }
 inline uint2 *active_words_next(const lbmd_ctx *c) { return c->occw[(c->lb_step + 1) & 1]; }
 inline void *active_records_next(const lbmd_ctx *c) { return c->cact[(c->lb_step + 1) & 1]; }
-// Variants A and B keep the node records of the active nodes in compact
-// arrays, which the MD steps add their transfers to (variant C updates the
-// populations every MD step instead).  Variant B's MD steps also read them.
+// The node records of the active nodes are kept in compact arrays, which the
+// MD steps add their transfers to.  The MD steps of variants B and C also read
+// them (C differs from B only in how the LB step takes the transfers).
 // Variant A's read the node velocities as the LB step left them: from the
 // node field, which nobody writes between LB steps in A (transfers to
 // inactive nodes go to J_acc), or -- when the node field is too large for the
 // L2 cache, where its scattered reads cost more than a copy -- from the first
 // buffer of the set, the transfers then going to the second buffer, which the
 // moments fill with the same records.
-inline bool compact_nodes(const lbmd_ctx *c) { return c->p.variant != LBMD_VARIANT_C; }
 inline bool a_copy(const lbmd_ctx *c) { return c->p.variant == LBMD_VARIANT_A && c->a_frozen_copy; }
 // the records the MD steps add transfers to (and the LB step reads)
 inline void *active_records_acc(const lbmd_ctx *c) {
@@ -245,11 +244,21 @@ inline void *vel_now(const lbmd_ctx *c) { return c->vel4[c->pv]; }
 // poll: about 67 ms, far above the few microseconds the lag needs).
 constexpr int LBMD_DEFAULT_FUSE_SPIN = 1 << 20;
 
+// Deviation storage: the density of the stored rest values, sum_i b_i with
+// b_i = w_i rho0 formed in T as the kernels form it (0 for the plain forms,
+// whose arithmetic is on the populations themselves).
+template <typename T, typename S>
+inline T rest_density(const lbmd_ctx *ctx) {
+    if (!lbmd::PopStore<S, T>::deviation) return T(0);
+    double sum = 0.0;
+    for (int i = 0; i < lbmd::Q; ++i) sum += (double)(T(lbmd::WEIGHT(i)) * (T)ctx->p.rho0);
+    return (T)sum;
+}
+
 // Launchers, one per kernel family; each enqueues on ctx->stream and returns
 // the launch status.
 cudaError_t launch_lb_step(lbmd_ctx *ctx);
 cudaError_t launch_node_moments(lbmd_ctx *ctx, bool count_step);
-cudaError_t launch_forcing_update(lbmd_ctx *ctx);
 cudaError_t launch_init_equilibrium(lbmd_ctx *ctx);
 cudaError_t launch_md_substep(lbmd_ctx *ctx, int substep);
 cudaError_t launch_bond_forces_only(lbmd_ctx *ctx);

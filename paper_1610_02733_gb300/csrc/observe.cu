@@ -13,6 +13,7 @@
 // block totals, the particle sums in pairs of FP32 values, and FP32 values
 // become doubles through their bit fields (exact, integer pipes).  Doubles
 // are added only per block and in the final reduction.
+#include "lb_core.cuh"
 #include "lbmd_ctx.h"
 #include "lbmd_device.cuh"
 #include "particle_core.cuh"
@@ -140,9 +141,9 @@ struct FluidSums<float> {
     }
 };
 
-// Variant B keeps the records of the active nodes in their compact array
-// during a cycle: a node's current record is found through the active words
-// (occw non-null), so no copy back is needed first.  Every thread issues the
+// The records of the active nodes are in their compact array during a cycle:
+// a node's current record is found through the active words, so no copy back
+// is needed first.  Every thread issues the
 // loads of U nodes before it adds any (memory-level parallelism), and the
 // active-word lookups run one pass ahead of the record loads that depend on
 // them, so a pass waits on one round trip to memory, not two.
@@ -160,7 +161,7 @@ __device__ __forceinline__ void observe_nodes(const typename Prec<T>::node4 *nod
         for (int u = 0; u < U; ++u) {
             const int64_t r = r0 + u * stride;
             x[u] = -1;
-            if (!occw || r >= N) continue;
+            if (r >= N) continue;
             const uint32_t row = fdiv((uint32_t)r, fnx);
             x[u] = (int)((uint32_t)r - row * fnx.d);
             wd[u] = occw[(size_t)row * W + (x[u] >> 5)];
@@ -309,17 +310,16 @@ static cudaError_t observables_t(lbmd_ctx *ctx) {
     const int mass_u = 40 - ctx->fix.e;  // the FP32 mass sum's unit 2^-mass_u
     const double mass_unit = std::ldexp(1.0, -mass_u);
     const auto *vel = static_cast<const typename P::real4 *>(vel_now(ctx));
-    if (ctx->p.variant == LBMD_VARIANT_B)
+    if (ctx->p.variant != LBMD_VARIANT_A)
         observe_kernel<T, LBMD_VARIANT_B><<<B, RED_THREADS, 0, ctx->stream>>>(
             static_cast<const typename P::node4 *>(ctx->node), nullptr, active_words_now(ctx),
             static_cast<const typename P::node4 *>(active_records_now(ctx)), active_words(ctx->p.nx), fnx, ctx->N,
             mass_u, mass_unit, vel, ctx->slot_of, ctx->np, ctx->red_partial, ctx->fix.inv_scale, ctx->range_flag,
             ctx->dev_error, ctx->red_out);
-    else  // variant A: the accumulating records of the active nodes (j* + J_acc), J_acc elsewhere; C: J_acc
+    else  // variant A: the accumulating records of the active nodes (j* + J_acc), J_acc elsewhere
         observe_kernel<T, LBMD_VARIANT_A><<<B, RED_THREADS, 0, ctx->stream>>>(
             static_cast<const typename P::node4 *>(ctx->node), static_cast<const typename P::node4 *>(ctx->jacc),
-            compact_nodes(ctx) ? active_words_now(ctx) : nullptr,
-            static_cast<const typename P::node4 *>(compact_nodes(ctx) ? active_records_acc(ctx) : nullptr),
+            active_words_now(ctx), static_cast<const typename P::node4 *>(active_records_acc(ctx)),
             active_words(ctx->p.nx), fnx, ctx->N, mass_u, mass_unit, vel, ctx->slot_of, ctx->np, ctx->red_partial,
             ctx->fix.inv_scale, ctx->range_flag, ctx->dev_error, ctx->red_out);
     return cudaGetLastError();
@@ -346,6 +346,38 @@ __global__ void pops_to_double_kernel(const S *f, int64_t first, int64_t count, 
     if (t >= count) return;
     const int64_t k = first + t;
     dst[t] = (double)PopStore<S, T>::load(f + k, pop_base<T>(k, N, rho0));
+}
+
+// Variant C inside a cycle: the populations with the transfers of the MD steps
+// done so far, which the LB step would add (lb.cu), added here on the way out;
+// the stored populations stay, so reading them does not change the run.
+template <typename T, typename S>
+__global__ void pops_c_to_double_kernel(const S *f, const typename Prec<T>::node4 *node, const uint2 *occw,
+                                        const typename Prec<T>::node4 *cact, int W, int nx, T rho_base, T gamma_bulk,
+                                        T gamma_shear, T fs, T fis, int64_t first, int64_t count, int64_t N,
+                                        double rho0, double *dst) {
+    using P = Prec<T>;
+    using St = PopStore<S, T>;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= count) return;
+    const int64_t k = first + t, r = k % N;
+    const int i = (int)(k / N), x = (int)(r % nx);
+    T fl[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) fl[q] = St::arith(f + (int64_t)q * N + r);
+    T rho, rho_m, jx, jy, jz;
+    pop_moments<St::deviation>(fl, rho_base, rho, rho_m, jx, jy, jz);
+    const int sl = active_slot(occw[(size_t)(r / nx) * W + (x >> 5)], x);
+    const typename P::node4 n = sl >= 0 ? cact[sl] : node[r];
+    const T Fx = P::from_fix(P::jx_of(n) - P::to_fix(jx, fs), fis), Fy = P::from_fix(P::jy_of(n) - P::to_fix(jy, fs), fis),
+            Fz = P::from_fix(P::jz_of(n) - P::to_fix(jz, fs), fis);
+    if (!(Fx == T(0) && Fy == T(0) && Fz == T(0)))
+        apply_transfer(fl, rho, jx, jy, jz, Fx, Fy, Fz, gamma_bulk, gamma_shear);
+    T v = T(0);
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+        if (q == i) v = fl[q];
+    dst[t] = (double)(St::deviation ? pop_base<T>(k, N, rho0) + v : v);
 }
 
 template <typename T, typename S>
@@ -376,8 +408,11 @@ __global__ void node_to_double_kernel(const typename Prec<T>::node4 *node, const
         dst[4 * t + 3] = (double)P::from_fix(P::jz_of(n), fis);
         return;
     }
-    const int sl = occw ? active_slot(occw[(size_t)(r / nx) * W + ((r % nx) >> 5)], (int)(r % nx)) : -1;
-    if (sl >= 0 && variant == LBMD_VARIANT_A) {
+    const int sl = active_slot(occw[(size_t)(r / nx) * W + ((r % nx) >> 5)], (int)(r % nx));
+    if (variant == LBMD_VARIANT_C) {
+        // the populations count as having taken every transfer (pops_c_to_double_kernel)
+        for (int d = 0; d < 3; ++d) dst[3 * t + d] = 0.0;
+    } else if (sl >= 0 && variant == LBMD_VARIANT_A) {
         // variant A, active node: the accumulating record minus the frozen one
         const typename P::node4 c = cacc[sl];
         dst[3 * t + 0] = (double)P::from_fix(P::jx_of(c) - P::jx_of(n), fis);
@@ -483,6 +518,15 @@ cudaError_t launch_observables(lbmd_ctx *ctx) {
 
 template <typename T, typename S>
 static cudaError_t pops_to_double_t(lbmd_ctx *ctx, int64_t first, int64_t count, double *dst) {
+    if (ctx->p.variant == LBMD_VARIANT_C && ctx->sub_done > 0) {
+        using N4 = typename Prec<T>::node4;
+        pops_c_to_double_kernel<T, S><<<nblocks(count), 256, 0, ctx->stream>>>(
+            static_cast<const S *>(ctx->f[ctx->cur]), static_cast<const N4 *>(ctx->node), active_words_now(ctx),
+            static_cast<const N4 *>(active_records_now(ctx)), active_words(ctx->p.nx), ctx->p.nx,
+            rest_density<T, S>(ctx), (T)ctx->co.gamma_bulk, (T)ctx->co.gamma_shear, (T)ctx->fix.scale,
+            (T)ctx->fix.inv_scale, first, count, ctx->N, ctx->p.rho0, dst);
+        return cudaGetLastError();
+    }
     pops_to_double_kernel<T, S><<<nblocks(count), 256, 0, ctx->stream>>>(
         static_cast<const S *>(ctx->f[ctx->cur]), first, count, ctx->N, ctx->p.rho0, dst);
     return cudaGetLastError();
@@ -500,8 +544,7 @@ static cudaError_t node_to_double_t(lbmd_ctx *ctx, int64_t first, int64_t count,
     using N4 = typename Prec<T>::node4;
     node_to_double_kernel<T, S><<<nblocks(count), 256, 0, ctx->stream>>>(
         static_cast<const N4 *>(ctx->node), static_cast<const N4 *>(ctx->jacc),
-        compact_nodes(ctx) ? active_words_now(ctx) : nullptr,
-        static_cast<const N4 *>(compact_nodes(ctx) ? active_records_acc(ctx) : nullptr), active_words(ctx->p.nx),
+        active_words_now(ctx), static_cast<const N4 *>(active_records_acc(ctx)), active_words(ctx->p.nx),
         ctx->p.nx, static_cast<const S *>(ctx->f[ctx->cur]), ctx->N, (T)ctx->p.rho0, (T)ctx->fix.scale,
         (T)ctx->fix.inv_scale, first, count, dst, transfer_only ? 1 : 0, ctx->p.variant);
     return cudaGetLastError();
@@ -532,7 +575,7 @@ cudaError_t launch_node_field_to_double(lbmd_ctx *ctx, int64_t first, int64_t co
 }
 
 cudaError_t launch_clear_transfer(lbmd_ctx *ctx) {
-    if (ctx->p.variant == LBMD_VARIANT_B) return cudaSuccess;
+    if (ctx->p.variant != LBMD_VARIANT_A) return cudaSuccess;
     if (ctx->p.precision == LBMD_FP64)
         clear_transfer_kernel<double><<<nblocks(ctx->N), 256, 0, ctx->stream>>>(
             static_cast<Prec<double>::node4 *>(ctx->jacc), ctx->N);

@@ -43,8 +43,8 @@ struct PArgs {
     const uint2 *occw;
     typename P::node4 *cact;          // the active nodes' records (variant A with a frozen copy: the frozen ones)
     typename P::node4 *cact_acc;      // ... the ones the transfers go to (the same unless A keeps a frozen copy)
-    typename P::node4 *inactive_acc;  // where transfers to inactive nodes go (A: J_acc, B: the node field)
-    int interp_compact;               // interpolate from cact (B; A with a frozen copy), else the node field
+    typename P::node4 *inactive_acc;  // where transfers to inactive nodes go (A: J_acc, B and C: the node field)
+    int interp_compact;               // interpolate from cact (B, C; A with a frozen copy), else the node field
     int occ_words;
     int32_t *migrant_slot, *migrant_count;  // two lists of np_cap slots, two counters
     int gauss;         // normal variates (Box-Muller) for the random force
@@ -157,28 +157,18 @@ __device__ __forceinline__ void coupling_force(const PArgs<T> &a, int64_t p, con
 }
 
 // Newton's third law for the particle in slot p whose transfer -delta_k dt F
-// belongs to the nodes around position R (cell c): variant C adds it to
-// J_acc at once (forcing_update_kernel then moves it into the populations);
-// variants A and B keep R for the row gather (which adds the transfers to the
-// compact records, cact_acc), and a particle whose cell row
-// is no longer the row bucket it was sorted into is listed as a migrant (two
-// lists alternating with the parity of the MD step).
+// belongs to the nodes around position R: R is kept for the row gather (which
+// adds the transfers to the compact records, cact_acc), and a particle whose
+// cell row is no longer the row bucket it was sorted into is listed as a
+// migrant (two lists alternating with the parity of the MD step).
 template <typename T>
-__device__ __forceinline__ void hand_over(const PArgs<T> &a, int64_t p, const typename Prec<T>::real4 &R,
-                                          const CellXYZ &c, T Fx, T Fy, T Fz) {
+__device__ __forceinline__ void hand_over(const PArgs<T> &a, int64_t p, const typename Prec<T>::real4 &R) {
     using P = Prec<T>;
-    if (a.variant == LBMD_VARIANT_C) {
-        uint32_t idx[8];
-        T delta[8];
-        corners(c, R.x, R.y, R.z, a.nx, a.ny, a.nz, idx, delta);
-        spread_to<T>(a.jacc, idx, delta, Fx * a.neg_scale_dt, Fy * a.neg_scale_dt, Fz * a.neg_scale_dt);
-    } else {
-        a.old4[p] = R;
-        if (a.b_atomic) return;
-        const int32_t srow = a.slot_row[p];
-        if (srow < 0 || (uint32_t)P::cell_of(R) - (uint32_t)srow * (uint32_t)a.nx >= (uint32_t)a.nx) {
-            a.migrant_slot[(int64_t)a.mig_par * a.np_cap + atomicAdd(a.migrant_count + a.mig_par, 1)] = (int32_t)p;
-        }
+    a.old4[p] = R;
+    if (a.b_atomic) return;
+    const int32_t srow = a.slot_row[p];
+    if (srow < 0 || (uint32_t)P::cell_of(R) - (uint32_t)srow * (uint32_t)a.nx >= (uint32_t)a.nx) {
+        a.migrant_slot[(int64_t)a.mig_par * a.np_cap + atomicAdd(a.migrant_count + a.mig_par, 1)] = (int32_t)p;
     }
 }
 

@@ -7,11 +7,9 @@
 //     interpolated fluid velocity (Eq. (4)); Delta P = dt F (Eq. (6));
 //   * velocity Verlet with F held fixed (second half-kick here for ideal
 //     particles, in bond_kick_kernel when bonds exist);
-//   * variant A: the transfer -delta_k Delta P (Eqs. (7), (8)) goes straight
-//     into the accumulator J_acc, which no MD step reads;
-//     variant B: the start-of-step position and F are kept for
-//     spread_rows_kernel, which runs once every particle has read the node
-//     field.
+//   * the start-of-step position and F are kept for spread_rows_kernel, which
+//     adds the transfer -delta_k Delta P (Eqs. (7), (8)) once every particle
+//     has read the nodes.
 // Transfers are added as fixed-point integers with atomics, so the sum does
 // not depend on the order of the particles (bitwise reproducible).
 //
@@ -94,8 +92,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 3) couple_kernel(PAr
     if (BONDS) check_list_skin(a, p, CellXYZ{cx, cy, cz}, fx, fy, fz);
     a.pos4[p] = P::make_pos(fx, fy, fz, cx + (int64_t)a.nx * (cy + (int64_t)a.ny * cz));
     a.vel4[p] = V;
-    if (BONDS || a.variant != LBMD_VARIANT_C) a.fc4[p] = P::make4(Fx, Fy, Fz, T(0));
-    hand_over(a, p, R, c, Fx, Fy, Fz);
+    a.fc4[p] = P::make4(Fx, Fy, Fz, T(0));
+    hand_over(a, p, R);
 }
 
 // One MD step, coupling force from the half-step velocity (integrator
@@ -140,11 +138,11 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 3) couple_half_kerne
     a.pos4[p] = Rn;
     a.vel4[p] = V;
     a.fc4[p] = P::make4(Fx, Fy, Fz, T(0));
-    hand_over(a, p, Rn, cn, Fx, Fy, Fz);
+    hand_over(a, p, Rn);
 }
 
 
-// Variants A and B, atomic-free: one warp per node row (y, z), four rows per block,
+// Atomic-free spreading: one warp per node row (y, z), four rows per block,
 // rows in reverse order (the couple kernel touched the high rows last).  The
 // row's nodes get transfers only from particles in the four cell rows
 // (y - oy, z - oz), oy, oz in {0, 1}; with the particles bucketed by cell
@@ -153,7 +151,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 3) couple_half_kerne
 // Eq. (5)) as fixed-point integers in shared memory, one entry per active
 // node of the row; then it updates the row's compact records with plain
 // loads and stores (no other warp writes them).  A contribution to an inactive node goes with atomics to the
-// node field (B) or J_acc (A).  Particles that left their bucket's row are
+// node field (B, C) or J_acc (A).  Particles that left their bucket's row are
 // skipped here and spread by migrant_spread_kernel.
 constexpr int GATHER_WARPS = 4;  // warps per block (fewer for very long rows)
 
@@ -940,7 +938,7 @@ static PArgs<T> make_pargs(lbmd_ctx *ctx, int substep) {
     a.occw = active_words_now(ctx);
     a.cact = static_cast<typename P::node4 *>(active_records_now(ctx));
     a.cact_acc = static_cast<typename P::node4 *>(active_records_acc(ctx));
-    a.interp_compact = ctx->p.variant == LBMD_VARIANT_B || a_copy(ctx) ? 1 : 0;
+    a.interp_compact = ctx->p.variant != LBMD_VARIANT_A || a_copy(ctx) ? 1 : 0;
     a.inactive_acc = ctx->p.variant == LBMD_VARIANT_A ? a.jacc : a.node;
     a.occ_words = active_words(ctx->p.nx);
     return a;
@@ -952,10 +950,9 @@ static cudaError_t md_substep_t(lbmd_ctx *ctx, int substep) {
     PArgs<T> a = make_pargs<T>(ctx, substep);
     const unsigned blocks = (unsigned)((ctx->np + 255) / 256);
     const bool cons = has_cons(ctx);
-    const bool B = compact_nodes(ctx);  // variants A and B: spreading into the compact records
-    const bool atomic = B && (ctx->p.spread == LBMD_SPREAD_ATOMIC ||
-                              (ctx->p.spread == LBMD_SPREAD_AUTO &&
-                               ctx->np < (int64_t)LBMD_SPREAD_ATOMIC_PER_ROW * ctx->p.ny * ctx->p.nz));
+    const bool atomic = ctx->p.spread == LBMD_SPREAD_ATOMIC ||
+                        (ctx->p.spread == LBMD_SPREAD_AUTO &&
+                         ctx->np < (int64_t)LBMD_SPREAD_ATOMIC_PER_ROW * ctx->p.ny * ctx->p.nz);
     a.b_atomic = atomic ? 1 : 0;
     a.kick_spreads = atomic && cons ? 1 : 0;
     // the tiled step only on request: at the benchmark density it measured
@@ -991,24 +988,20 @@ static cudaError_t md_substep_t(lbmd_ctx *ctx, int substep) {
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    if (ctx->p.variant == LBMD_VARIANT_C) return launch_forcing_update(ctx);
-    if (B) {
-        if (atomic && cons) {
-            // spread by the bond / pair kernel above
-        } else if (atomic) {
-            const unsigned sb = (unsigned)std::min<int64_t>(ctx->sm_count, (ctx->np + 255) / 256);
-            migrant_spread_kernel<T><<<sb, 256, 0, ctx->stream>>>(a, 1);
-        } else {
-            const int rows = (int)((int64_t)ctx->p.ny * ctx->p.nz);
-            const int gw = ctx->gather_warps;
-            const unsigned gblocks = (unsigned)((rows + gw - 1) / gw);
-            spread_rows_kernel<T><<<gblocks, 32 * gw, gather_smem_bytes<T>(ctx, gw), ctx->stream>>>(a, rows);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            migrant_spread_kernel<T><<<ctx->sm_count, 256, 0, ctx->stream>>>(a, 0);
-        }
-        e = cudaGetLastError();
+    if (atomic && cons) {
+        // spread by the bond / pair kernel above
+    } else if (atomic) {
+        const unsigned sb = (unsigned)std::min<int64_t>(ctx->sm_count, (ctx->np + 255) / 256);
+        migrant_spread_kernel<T><<<sb, 256, 0, ctx->stream>>>(a, 1);
+    } else {
+        const int rows = (int)((int64_t)ctx->p.ny * ctx->p.nz);
+        const int gw = ctx->gather_warps;
+        const unsigned gblocks = (unsigned)((rows + gw - 1) / gw);
+        spread_rows_kernel<T><<<gblocks, 32 * gw, gather_smem_bytes<T>(ctx, gw), ctx->stream>>>(a, rows);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        migrant_spread_kernel<T><<<ctx->sm_count, 256, 0, ctx->stream>>>(a, 0);
     }
-    return e;
+    return cudaGetLastError();
 }
 
 template <typename T>
@@ -1032,7 +1025,7 @@ static cudaError_t sort_t(lbmd_ctx *ctx) {
     const int W = active_words(ctx->p.nx);
     cudaError_t e = cudaMemsetAsync(ctx->row_count, 0, (size_t)rows * sizeof(int32_t), ctx->stream);
     if (e != cudaSuccess) return e;
-    if (ctx->ccw && ctx->np > 0 &&
+    if (ctx->np > 0 &&
         (e = cudaMemsetAsync(ctx->ccw, 0, (size_t)rows * W * sizeof(uint32_t), ctx->stream)) != cudaSuccess)
         return e;
     if (ctx->np > 0) {
@@ -1116,12 +1109,11 @@ static cudaError_t nb_build_t(lbmd_ctx *ctx) {
 }  // namespace lbmd
 
 cudaError_t launch_active_set(lbmd_ctx *ctx) {
-    if (!compact_nodes(ctx)) return cudaSuccess;
     return ctx->p.precision == LBMD_FP64 ? lbmd::active_set_t<double>(ctx) : lbmd::active_set_t<float>(ctx);
 }
 
 cudaError_t launch_active_sync(lbmd_ctx *ctx) {
-    if (ctx->p.variant != LBMD_VARIANT_B) return cudaSuccess;
+    if (ctx->p.variant == LBMD_VARIANT_A) return cudaSuccess;
     return ctx->p.precision == LBMD_FP64 ? lbmd::active_sync_t<double>(ctx) : lbmd::active_sync_t<float>(ctx);
 }
 
