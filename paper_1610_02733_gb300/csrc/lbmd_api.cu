@@ -505,7 +505,7 @@ lbmd_status lbmd_md_substep(lbmd_ctx *ctx) {
     LBMD_TRACE("lbmd_md_substep");
     if (!ctx) return LBMD_ERR_ARG;
     if (ctx->sub_done >= ctx->p.n_sub) return fail(ctx, LBMD_ERR_SEQUENCE, "n_sub MD steps already done");
-    CK(ctx, launch_md_substep(ctx, ctx->sub_done));
+    CK(ctx, launch_md_steps(ctx, ctx->sub_done, 1));
     ctx->sub_done += 1;
     ctx->md_step += 1;
     return LBMD_OK;
@@ -532,9 +532,9 @@ lbmd_status lbmd_run_cycles(lbmd_ctx *ctx, int64_t n) {
             // capture one cycle starting from this state
             cudaGraph_t g = nullptr;
             CK(ctx, cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
-            cudaError_t e = cudaSuccess;
+            cudaError_t e;
             const int cur0 = ctx->cur, pcur0 = ctx->pcur, pv0 = ctx->pv, rec0 = ctx->rec;
-            for (int s = 0; s < ctx->p.n_sub && e == cudaSuccess; ++s) e = launch_md_substep(ctx, s);
+            e = launch_md_steps(ctx, 0, ctx->p.n_sub);
             if (e == cudaSuccess) e = launch_lb_step(ctx);
             // the launchers flipped the buffers during capture: keep the state
             // the cycle leaves, then restore the starting one

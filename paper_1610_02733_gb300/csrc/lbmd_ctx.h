@@ -260,7 +260,7 @@ inline T rest_density(const lbmd_ctx *ctx) {
 cudaError_t launch_lb_step(lbmd_ctx *ctx);
 cudaError_t launch_node_moments(lbmd_ctx *ctx, bool count_step);
 cudaError_t launch_init_equilibrium(lbmd_ctx *ctx);
-cudaError_t launch_md_substep(lbmd_ctx *ctx, int substep);
+cudaError_t launch_md_steps(lbmd_ctx *ctx, int substep, int count);
 cudaError_t launch_bond_forces_only(lbmd_ctx *ctx);
 // conservative forces present (bonds or Lennard-Jones)
 inline bool has_cons(const lbmd_ctx *ctx) { return ctx->nb > 0 || ctx->lj_rc > 0.0; }

@@ -74,6 +74,13 @@ __device__ __forceinline__ void corner_pair(const PArgs<T> &a, uint32_t row, int
 // x and x + 1); every caller sums in this one order with explicit fused
 // multiply-adds, so the paths that fetch the records differently agree bit
 // for bit whatever the compiler would contract.
+template <typename T>
+__device__ __forceinline__ void add_corner(T weight, T rho, T jx, T jy, T jz, T &ux, T &uy, T &uz) {
+    const T w = weight / rho;
+    ux = fma(w, jx, ux);
+    uy = fma(w, jy, uy);
+    uz = fma(w, jz, uz);
+}
 template <typename T, typename Fetch>
 __device__ __forceinline__ void interp_u_from(T fx, T fy, T fz, T fis, T &ux, T &uy, T &uz, Fetch &&fetch) {
     using P = Prec<T>;
@@ -86,12 +93,35 @@ __device__ __forceinline__ void interp_u_from(T fx, T fy, T fz, T fis, T &ux, T 
         typename P::node4 n[2];
         fetch(q, n[0], n[1]);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const T w = (wx[h] * wy[q & 1] * wz[q >> 1]) / P::rho_of(n[h]);
-            ux = fma(w, P::from_fix(P::jx_of(n[h]), fis), ux);
-            uy = fma(w, P::from_fix(P::jy_of(n[h]), fis), uy);
-            uz = fma(w, P::from_fix(P::jz_of(n[h]), fis), uz);
-        }
+        for (int h = 0; h < 2; ++h)
+            add_corner(wx[h] * wy[q & 1] * wz[q >> 1], P::rho_of(n[h]), P::from_fix(P::jx_of(n[h]), fis),
+                       P::from_fix(P::jy_of(n[h]), fis), P::from_fix(P::jz_of(n[h]), fis), ux, uy, uz);
+    }
+}
+// ... and from the corners' densities and momenta held by the caller.
+template <typename T>
+__device__ __forceinline__ void interp_u_cached(T fx, T fy, T fz, const T rho[8], const T jx[8], const T jy[8],
+                                                const T jz[8], T &ux, T &uy, T &uz) {
+    ux = T(0);
+    uy = T(0);
+    uz = T(0);
+    const T wx[2] = {T(1) - fx, fx}, wy[2] = {T(1) - fy, fy}, wz[2] = {T(1) - fz, fz};
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        add_corner(wx[k & 1] * wy[(k >> 1) & 1] * wz[k >> 2], rho[k], jx[k], jy[k], jz[k], ux, uy, uz);
+}
+
+// The records of corners 2q, 2q + 1 of cell c (x1: the node after c.x) in
+// lattice row `row`: compact records of active corners, or the node field.
+template <typename T>
+__device__ __forceinline__ void corner_fetch(const PArgs<T> &a, uint32_t row, const CellXYZ &c, int x1,
+                                             typename Prec<T>::node4 &n0, typename Prec<T>::node4 &n1) {
+    if (a.interp_compact) {  // an active corner's compact record
+        corner_pair(a, row, c.x, x1, n0, n1);
+    } else {
+        const size_t r0 = (size_t)row * (uint32_t)a.nx;
+        n0 = a.node[r0 + c.x];
+        n1 = a.node[r0 + x1];
     }
 }
 
@@ -105,14 +135,18 @@ __device__ __forceinline__ void interp_u(const PArgs<T> &a, const CellXYZ &c, T 
     corner_rows(c, a.ny, a.nz, rows);
     const int x1 = c.x + 1 == a.nx ? 0 : c.x + 1;
     interp_u_from(fx, fy, fz, a.fis, ux, uy, uz, [&](int q, typename P::node4 &n0, typename P::node4 &n1) {
-        if (a.interp_compact) {  // an active corner's compact record
-            corner_pair(a, rows[q], c.x, x1, n0, n1);
-        } else {
-            const size_t r0 = (size_t)rows[q] * (uint32_t)a.nx;
-            n0 = a.node[r0 + c.x];
-            n1 = a.node[r0 + x1];
-        }
+        corner_fetch(a, rows[q], c, x1, n0, n1);
     });
+}
+
+// All 8 corner records of cell c.
+template <typename T>
+__device__ __forceinline__ void corner_records(const PArgs<T> &a, const CellXYZ &c, typename Prec<T>::node4 n[8]) {
+    uint32_t rows[4];
+    corner_rows(c, a.ny, a.nz, rows);
+    const int x1 = c.x + 1 == a.nx ? 0 : c.x + 1;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) corner_fetch(a, rows[q], c, x1, n[2 * q], n[2 * q + 1]);
 }
 
 // Coupling force of Eq. (4) without the conservative part: friction against

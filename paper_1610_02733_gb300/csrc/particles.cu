@@ -34,6 +34,7 @@
 
 #include "lbmd_ctx.h"
 #include "lbmd_device.cuh"
+#include "md_phase.cuh"
 #include "particle_core.cuh"
 #include "particle_step.cuh"
 
@@ -944,15 +945,44 @@ static PArgs<T> make_pargs(lbmd_ctx *ctx, int substep) {
     return a;
 }
 
+// Whether the transfers go to the nodes with atomics (else the row gather).
+static bool spreads_atomic(const lbmd_ctx *ctx) {
+    return ctx->p.spread == LBMD_SPREAD_ATOMIC ||
+           (ctx->p.spread == LBMD_SPREAD_AUTO &&
+            ctx->np < (int64_t)LBMD_SPREAD_ATOMIC_PER_ROW * ctx->p.ny * ctx->p.nz);
+}
+
+// `count` MD steps from `substep` on in one launch, where the system allows it.
+// *done says whether it did.
+template <typename T>
+static cudaError_t md_phase_t(lbmd_ctx *ctx, int substep, int count, bool *done) {
+    *done = true;
+    if (ctx->np == 0) return cudaSuccess;
+    const bool atomic = spreads_atomic(ctx);
+    // Variant A without conservative forces.  A single step of a dense system
+    // keeps the row gather, whose plain stores cost less than one atomic
+    // hand-over per particle; from two steps on the phase has fewer of both.
+    if (ctx->p.variant == LBMD_VARIANT_A && !has_cons(ctx) &&
+        (atomic || (ctx->p.spread == LBMD_SPREAD_AUTO && count > 1))) {
+        const PArgs<T> a = make_pargs<T>(ctx, substep);
+        const unsigned blocks = (unsigned)((ctx->np + 127) / 128);
+        if (ctx->p.integrator == LBMD_INTEGRATOR_HALF_STEP)
+            frozen_phase_kernel<T, true><<<blocks, 128, 0, ctx->stream>>>(a, count);
+        else
+            frozen_phase_kernel<T, false><<<blocks, 128, 0, ctx->stream>>>(a, count);
+        return cudaGetLastError();
+    }
+    *done = false;
+    return cudaSuccess;
+}
+
 template <typename T>
 static cudaError_t md_substep_t(lbmd_ctx *ctx, int substep) {
     if (ctx->np == 0) return cudaSuccess;
     PArgs<T> a = make_pargs<T>(ctx, substep);
     const unsigned blocks = (unsigned)((ctx->np + 255) / 256);
     const bool cons = has_cons(ctx);
-    const bool atomic = ctx->p.spread == LBMD_SPREAD_ATOMIC ||
-                        (ctx->p.spread == LBMD_SPREAD_AUTO &&
-                         ctx->np < (int64_t)LBMD_SPREAD_ATOMIC_PER_ROW * ctx->p.ny * ctx->p.nz);
+    const bool atomic = spreads_atomic(ctx);
     a.b_atomic = atomic ? 1 : 0;
     a.kick_spreads = atomic && cons ? 1 : 0;
     // the tiled step only on request: at the benchmark density it measured
@@ -1117,9 +1147,14 @@ cudaError_t launch_active_sync(lbmd_ctx *ctx) {
     return ctx->p.precision == LBMD_FP64 ? lbmd::active_sync_t<double>(ctx) : lbmd::active_sync_t<float>(ctx);
 }
 
-cudaError_t launch_md_substep(lbmd_ctx *ctx, int substep) {
-    return ctx->p.precision == LBMD_FP64 ? lbmd::md_substep_t<double>(ctx, substep)
-                                         : lbmd::md_substep_t<float>(ctx, substep);
+cudaError_t launch_md_steps(lbmd_ctx *ctx, int substep, int count) {
+    const bool dbl = ctx->p.precision == LBMD_FP64;
+    bool done = false;
+    cudaError_t e = dbl ? lbmd::md_phase_t<double>(ctx, substep, count, &done)
+                        : lbmd::md_phase_t<float>(ctx, substep, count, &done);
+    for (int s = 0; !done && s < count && e == cudaSuccess; ++s)
+        e = dbl ? lbmd::md_substep_t<double>(ctx, substep + s) : lbmd::md_substep_t<float>(ctx, substep + s);
+    return e;
 }
 
 cudaError_t launch_bond_forces_only(lbmd_ctx *ctx) {

@@ -1,0 +1,39 @@
+"""Several MD steps in one launch (GPU): the same bits as one step at a time
+with the row gather, whatever the particles do meanwhile."""
+import numpy as np
+import pytest
+
+from paper_1610_02733_gb300 import inputs, lbmd
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(shape, n, kT_init, steps, **kw):
+    """steps: 'g' one captured cycle, 'e' one cycle call by call."""
+    g = lbmd.LBMD(*shape, kT=1e-3, zeta=1.0, seed=11, max_particles=max(n, 1), **kw)
+    if n:
+        mass = inputs.uniform((n,), 0.8, 2.0, 4)
+        g.add_particles(inputs.uniform_positions(n, shape, 6), inputs.maxwell_velocities(n, kT_init, 6), mass)
+    for s in steps:
+        g.run_cycles(1) if s == "g" else g.cycle(1)
+    out = (g.populations(), g.node_field(), *g.particles())
+    g.close()
+    return out
+
+
+def _same(a, b):
+    for x, y in zip(a, b):
+        assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("integrator", ["start", "half_step"])
+@pytest.mark.parametrize("shape,n,m", [((7, 5, 6), 1, 1), ((40, 6, 5), 129, 4), ((20, 9, 8), 1500, 10)])
+def test_variant_a_phase(precision, integrator, shape, n, m):
+    # slow particles (they stay in their cells) and ones that cross several
+    # cells per cycle; captured cycles, single steps, and both in turn
+    for kT_init in (1e-4, 0.2):
+        kw = dict(variant="A", precision=precision, integrator=integrator, n_sub=m)
+        want = _run(shape, n, kT_init, "eeee", spread="rows", **kw)
+        for steps, spread in (("gggg", "auto"), ("gege", "auto"), ("egge", "atomic")):
+            _same(_run(shape, n, kT_init, steps, spread=spread, **kw), want)
