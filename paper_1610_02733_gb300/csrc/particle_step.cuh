@@ -53,20 +53,6 @@ struct PArgs {
     int64_t np_cap;
 };
 
-// Variant B: the records of corners 2q, 2q+1 (nodes x0 and x0 + 1 of row
-// `row`): compact record of an active node, node field entry otherwise.
-template <typename T>
-__device__ __forceinline__ void corner_pair(const PArgs<T> &a, uint32_t row, int x0, int x1,
-                                            typename Prec<T>::node4 &n0, typename Prec<T>::node4 &n1) {
-    const uint2 *wr = a.occw + (size_t)row * (uint32_t)a.occ_words;
-    const uint2 w0 = wr[x0 >> 5];
-    const uint2 w1 = (x1 >> 5) == (x0 >> 5) ? w0 : wr[x1 >> 5];
-    const int s0 = active_slot(w0, x0), s1 = active_slot(w1, x1);
-    const size_t r0 = (size_t)row * (uint32_t)a.nx;
-    n0 = s0 >= 0 ? a.cact[s0] : a.node[r0 + x0];
-    n1 = s1 >= 0 ? a.cact[s1] : a.node[r0 + x1];
-}
-
 // Fluid velocity at a particle with fractional offsets (fx, fy, fz) in its
 // cell, Eq. (5): corners k = ox + 2 oy + 4 oz = 0..7 with weights
 // delta_k = wx wy wz, u(R) = sum_k delta_k j_k / rho_k.  fetch(q, n0, n1)
@@ -111,22 +97,48 @@ __device__ __forceinline__ void interp_u_cached(T fx, T fy, T fz, const T rho[8]
         add_corner(wx[k & 1] * wy[(k >> 1) & 1] * wz[k >> 2], rho[k], jx[k], jy[k], jz[k], ux, uy, uz);
 }
 
-// The records of corners 2q, 2q + 1 of cell c (x1: the node after c.x) in
-// lattice row `row`: compact records of active corners, or the node field.
+// The records of the 8 corners of cell c, k = ox + 2 oy + 4 oz: the compact
+// record of an active node, the node field entry otherwise (interp_compact 0:
+// always the node field).  All active words are loaded before the first
+// record and all records before the first use, so a thread waits on two
+// round trips to memory and has 8 records in flight; fetching them row by
+// row between the divisions of the interpolation left two.
 template <typename T>
-__device__ __forceinline__ void corner_fetch(const PArgs<T> &a, uint32_t row, const CellXYZ &c, int x1,
-                                             typename Prec<T>::node4 &n0, typename Prec<T>::node4 &n1) {
-    if (a.interp_compact) {  // an active corner's compact record
-        corner_pair(a, row, c.x, x1, n0, n1);
+__device__ __forceinline__ void corner_records(const PArgs<T> &a, const CellXYZ &c, typename Prec<T>::node4 n[8]) {
+    using N4 = typename Prec<T>::node4;
+    uint32_t rows[4];
+    corner_rows(c, a.ny, a.nz, rows);
+    const int x1 = c.x + 1 == a.nx ? 0 : c.x + 1;
+    const N4 *ptr[8];
+    if (a.interp_compact) {
+        uint2 w0[4], w1[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint2 *wr = a.occw + (size_t)rows[q] * (uint32_t)a.occ_words;
+            w0[q] = wr[c.x >> 5];
+            w1[q] = w0[q];
+            if ((x1 >> 5) != (c.x >> 5)) w1[q] = wr[x1 >> 5];
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int s0 = active_slot(w0[q], c.x), s1 = active_slot(w1[q], x1);
+            const size_t r0 = (size_t)rows[q] * (uint32_t)a.nx;
+            ptr[2 * q] = s0 >= 0 ? a.cact + s0 : a.node + (r0 + c.x);
+            ptr[2 * q + 1] = s1 >= 0 ? a.cact + s1 : a.node + (r0 + x1);
+        }
     } else {
-        const size_t r0 = (size_t)row * (uint32_t)a.nx;
-        n0 = a.node[r0 + c.x];
-        n1 = a.node[r0 + x1];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const size_t r0 = (size_t)rows[q] * (uint32_t)a.nx;
+            ptr[2 * q] = a.node + (r0 + c.x);
+            ptr[2 * q + 1] = a.node + (r0 + x1);
+        }
     }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) n[k] = *ptr[k];
 }
 
-// The same for a particle in cell c read from global memory; variant B reads
-// an active corner's compact record.
+// The same for a particle in cell c, its records read from memory.
 template <typename T>
 __device__ __forceinline__ void interp_u(const PArgs<T> &a, const CellXYZ &c, T fx, T fy, T fz, T &ux, T &uy,
                                          T &uz) {
@@ -134,19 +146,12 @@ __device__ __forceinline__ void interp_u(const PArgs<T> &a, const CellXYZ &c, T 
     uint32_t rows[4];
     corner_rows(c, a.ny, a.nz, rows);
     const int x1 = c.x + 1 == a.nx ? 0 : c.x + 1;
+    typename P::node4 nn[8];
+    corner_records(a, c, nn);
     interp_u_from(fx, fy, fz, a.fis, ux, uy, uz, [&](int q, typename P::node4 &n0, typename P::node4 &n1) {
-        corner_fetch(a, rows[q], c, x1, n0, n1);
+        n0 = nn[2 * q];
+        n1 = nn[2 * q + 1];
     });
-}
-
-// All 8 corner records of cell c.
-template <typename T>
-__device__ __forceinline__ void corner_records(const PArgs<T> &a, const CellXYZ &c, typename Prec<T>::node4 n[8]) {
-    uint32_t rows[4];
-    corner_rows(c, a.ny, a.nz, rows);
-    const int x1 = c.x + 1 == a.nx ? 0 : c.x + 1;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) corner_fetch(a, rows[q], c, x1, n[2 * q], n[2 * q + 1]);
 }
 
 // Coupling force of Eq. (4) without the conservative part: friction against

@@ -54,11 +54,16 @@ namespace lbmd {
 // second one here for particles without conservative forces, in the bond /
 // pair kernel otherwise), transfer around the start position.
 // The variant is a run-time flag (one instruction sequence for both
-// variants, as in the LB kernel).  At least 5 blocks of 256 threads per SM
-// (3 in FP64): the corner loads are scattered, so latency hiding needs many
-// warps.
+// variants, as in the LB kernel).  Bound by the latency of the scattered
+// corner loads (16 B records, 33 % of the issue slots busy): 8 records in
+// flight per thread (corner_records) need 64 registers, and 8 blocks of 128
+// threads of them per SM measured faster (42 us at 256^3 nodes and 10^6
+// particles, FP32) than 4 of 256 (44 us), 6 of 128 (45 us) or 5 of 256 with
+// 48 registers (50 us; fetching the records row by row 48 us).
+constexpr int COUPLE_THREADS = 128;
+
 template <typename T, bool BONDS>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 3) couple_kernel(PArgs<T> a) {
+__global__ void __launch_bounds__(COUPLE_THREADS, sizeof(T) == 4 ? 8 : 4) couple_kernel(PArgs<T> a) {
     using P = Prec<T>;
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= a.np) return;
@@ -103,7 +108,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 3) couple_kernel(PAr
 // the new position R', second half-kick (here without conservative forces,
 // in the bond / pair kernel otherwise), transfer around R'.
 template <typename T, bool BONDS>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 3) couple_half_kernel(PArgs<T> a) {
+__global__ void __launch_bounds__(COUPLE_THREADS, sizeof(T) == 4 ? 8 : 4) couple_half_kernel(PArgs<T> a) {
     using P = Prec<T>;
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= a.np) return;
@@ -981,6 +986,7 @@ static cudaError_t md_substep_t(lbmd_ctx *ctx, int substep) {
     if (ctx->np == 0) return cudaSuccess;
     PArgs<T> a = make_pargs<T>(ctx, substep);
     const unsigned blocks = (unsigned)((ctx->np + 255) / 256);
+    const unsigned cblocks = (unsigned)((ctx->np + COUPLE_THREADS - 1) / COUPLE_THREADS);
     const bool cons = has_cons(ctx);
     const bool atomic = spreads_atomic(ctx);
     a.b_atomic = atomic ? 1 : 0;
@@ -1000,13 +1006,13 @@ static cudaError_t md_substep_t(lbmd_ctx *ctx, int substep) {
     }
     if (ctx->p.integrator == LBMD_INTEGRATOR_HALF_STEP) {
         if (cons)
-            couple_half_kernel<T, true><<<blocks, 256, 0, ctx->stream>>>(a);
+            couple_half_kernel<T, true><<<cblocks, COUPLE_THREADS, 0, ctx->stream>>>(a);
         else
-            couple_half_kernel<T, false><<<blocks, 256, 0, ctx->stream>>>(a);
+            couple_half_kernel<T, false><<<cblocks, COUPLE_THREADS, 0, ctx->stream>>>(a);
     } else if (cons) {
-        couple_kernel<T, true><<<blocks, 256, 0, ctx->stream>>>(a);
+        couple_kernel<T, true><<<cblocks, COUPLE_THREADS, 0, ctx->stream>>>(a);
     } else {
-        couple_kernel<T, false><<<blocks, 256, 0, ctx->stream>>>(a);
+        couple_kernel<T, false><<<cblocks, COUPLE_THREADS, 0, ctx->stream>>>(a);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
