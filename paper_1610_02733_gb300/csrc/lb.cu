@@ -19,6 +19,7 @@
 // reach.  node_moments_kernel computes them on their own (creation, replaced
 // populations).
 #include "lb_core.cuh"
+#include "lb_fixed.cuh"
 #include "lbmd_ctx.h"
 #include "lbmd_device.cuh"
 
@@ -53,17 +54,16 @@ struct LbArgs {
     const unsigned long long *lb_step;
     int noisy;
     int variant;
+    FixedArgs fx;  // FP64: the integer form of the collision
 };
 
 // Range guard: a record whose momentum reaches half the fixed-point range
 // raises the context's flag (the integer sums of later transfers could wrap).
 template <typename T>
-__device__ __forceinline__ typename Prec<T>::node4 guarded_record(T rho, T jx, T jy, T jz, T fs,
-                                                                  int32_t *range_flag) {
+__device__ __forceinline__ typename Prec<T>::node4 guarded_record(const NodeSums<T> &s, int32_t *range_flag) {
     using P = Prec<T>;
-    const typename P::fix ix = P::to_fix(jx, fs), iy = P::to_fix(jy, fs), iz = P::to_fix(jz, fs);
-    if (P::beyond_half(ix) | P::beyond_half(iy) | P::beyond_half(iz)) atomicOr(range_flag, 1);
-    return P::pack(rho, ix, iy, iz);
+    if (P::beyond_half(s.ix) | P::beyond_half(s.iy) | P::beyond_half(s.iz)) atomicOr(range_flag, 1);
+    return P::pack(s.rho, s.ix, s.iy, s.iz);
 }
 
 // Post-stream moments rho*, j* (Eqs. (1), (2)) of node (x, y, t): the node
@@ -73,7 +73,7 @@ __device__ __forceinline__ typename Prec<T>::node4 guarded_record(T rho, T jx, T
 template <typename T, typename S>
 __device__ __forceinline__ void node_moments_at(const S *f, typename Prec<T>::node4 *node, const uint2 *occw,
                                                 typename Prec<T>::node4 *cact, typename Prec<T>::node4 *cact2,
-                                                int occ_words, int64_t N, int nx, int ny, T rho_base, T fs,
+                                                int occ_words, int64_t N, int nx, int ny, T rho_base, T fs, int e,
                                                 int32_t *range_flag, int x, int y, int t) {
     using P = Prec<T>;
     using St = PopStore<S, T>;
@@ -81,9 +81,7 @@ __device__ __forceinline__ void node_moments_at(const S *f, typename Prec<T>::no
     T fl[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) fl[i] = St::arith_cg(f + (size_t)i * N + r);
-    T rho, rho_m, jx, jy, jz;
-    pop_moments<St::deviation>(fl, rho_base, rho, rho_m, jx, jy, jz);
-    const typename P::node4 rec = guarded_record(rho, jx, jy, jz, fs, range_flag);
+    const typename P::node4 rec = guarded_record(node_sums<St::deviation>(fl, rho_base, fs, e), range_flag);
     node[r] = rec;
     const int sl = active_slot(occw[((size_t)y + (size_t)ny * t) * occ_words + (x >> 5)], x);
     if (sl >= 0) {
@@ -103,6 +101,137 @@ constexpr int FUSE_LAG = 2;
 // lower it (lbmd_set_moments_wait), down to 0, where every row goes to the
 // fallback kernel.
 
+// The transfer J_acc to node (x, y, z) since the last LB step.  A record's
+// j = fix(j*) + sum of fixed-point transfers: the difference is exactly the
+// accumulated transfer (an active node's record is its compact one -- variant
+// A: the accumulating copy; B and C: an inactive node's is the node field).
+// Variant A, inactive node: J_acc holds what was handed over there (rarely
+// anything; cleared only where set).
+//
+// FP32 arithmetic, as the real force of a node with momentum (jx, jy, jz): the
+// integers are converted at once (kept as integers beside the sums they cost
+// the kernel 8 bytes more of spills and 1.6 % of the cycle).
+template <typename T, typename S, bool C>
+__device__ __forceinline__ void node_force(const LbArgs<T, S> &a, uint32_t r, int x, int y, int z, T jx, T jy, T jz,
+                                           T &Fx, T &Fy, T &Fz) {
+    using P = Prec<T>;
+    const int sl = active_slot(a.occw[((size_t)y + (size_t)a.ny * z) * a.occ_words + (x >> 5)], x);
+    if (C || sl >= 0 || a.variant == LBMD_VARIANT_B) {
+        const typename P::node4 n = sl >= 0 ? a.cact[sl] : a.node[r];
+        Fx = P::from_fix(P::jx_of(n) - P::to_fix(jx, a.fs), a.fis);
+        Fy = P::from_fix(P::jy_of(n) - P::to_fix(jy, a.fs), a.fis);
+        Fz = P::from_fix(P::jz_of(n) - P::to_fix(jz, a.fs), a.fis);
+    } else {
+        const typename P::node4 J = a.jacc[r];
+        Fx = P::from_fix(P::jx_of(J), a.fis);
+        Fy = P::from_fix(P::jy_of(J), a.fis);
+        Fz = P::from_fix(P::jz_of(J), a.fis);
+        if ((P::jx_of(J) | P::jy_of(J) | P::jz_of(J)) != 0) {
+            typename P::node4 zero;
+            zero.x = zero.y = zero.z = zero.w = 0;
+            a.jacc[r] = zero;
+        }
+    }
+}
+
+// FP64: the integers themselves; ix, iy, iz are fix(j*).
+template <bool C>
+__device__ __forceinline__ void node_transfer(const LbArgs<double, double> &a, uint32_t r, int x, int y, int z,
+                                              long long ix, long long iy, long long iz, long long J[3]) {
+    const int sl = active_slot(a.occw[((size_t)y + (size_t)a.ny * z) * a.occ_words + (x >> 5)], x);
+    if (C || sl >= 0 || a.variant == LBMD_VARIANT_B) {
+        const L4 n = sl >= 0 ? a.cact[sl] : a.node[r];
+        J[0] = n.y - ix;
+        J[1] = n.z - iy;
+        J[2] = n.w - iz;
+    } else {
+        const L4 n = a.jacc[r];
+        J[0] = n.y;
+        J[1] = n.z;
+        J[2] = n.w;
+        if ((J[0] | J[1] | J[2]) != 0) a.jacc[r] = L4{0, 0, 0, 0};
+    }
+}
+
+// FP64 form: f -> the post-collision populations, for the transfer J.
+template <bool RELAX_FULL, bool GAUSS, bool C>
+__device__ __forceinline__ void collide_with_transfer(const LbArgs<double, double> &a, double f[Q], NodeSums<double> s,
+                                                      const long long J[3], uint32_t r, uint32_t step) {
+    using P = Prec<double>;
+    double Fx = P::from_fix(J[0], a.fis), Fy = P::from_fix(J[1], a.fis), Fz = P::from_fix(J[2], a.fis);
+    if (C && !(Fx == 0.0 && Fy == 0.0 && Fz == 0.0)) {
+        apply_transfer(f, s.rho, s.jx, s.jy, s.jz, Fx, Fy, Fz, a.gamma_bulk, a.gamma_shear);
+        pop_moments<false>(f, 0.0, s.rho, s.rho_m, s.jx, s.jy, s.jz);
+        Fx = Fy = Fz = 0.0;
+    }
+    collide<double, RELAX_FULL, LbArgs<double, double>, GAUSS>(f, s.rho, s.rho_m, s.jx, s.jy, s.jz, Fx + a.g[0],
+                                                               Fy + a.g[1], Fz + a.g[2], a, a.key0, a.key1, r, step);
+}
+
+// The FP64 form of the collision for a node outside the integer form's range
+// (out of line: kept off the common path); out gets the new populations.
+template <bool GAUSS, bool C>
+__device__ __noinline__ void collide_fp64_out(const LbArgs<double, double> &a, uint32_t r, uint32_t step, long long Jx,
+                                              long long Jy, long long Jz, double *out) {
+    double f[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) f[i] = a.fin[(size_t)i * a.N + r];
+    NodeSums<double> s;
+    pop_moments<false>(f, 0.0, s.rho, s.rho_m, s.jx, s.jy, s.jz);
+    const long long J[3] = {Jx, Jy, Jz};
+    collide_with_transfer<true, GAUSS, C>(a, f, s, J, r, step);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) out[i] = f[i];
+}
+template <bool GAUSS, bool C>
+__device__ __forceinline__ void collide_node_fp64(const LbArgs<double, double> &a, uint32_t r, uint32_t step,
+                                                  const long long J[3], double f[Q]) {
+    double out[Q];
+    collide_fp64_out<GAUSS, C>(a, r, step, J[0], J[1], J[2], out);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) f[i] = out[i];
+}
+
+// The noise numbers of a node's 15 modes for collide_fixed, as collide() draws
+// them.
+template <bool GAUSS>
+struct FluidNoise {
+    uint32_t w[8];
+    __device__ __forceinline__ FluidNoise(const LbArgs<double, double> &a, uint32_t node, uint32_t step) {
+        if (!a.noisy) return;
+#pragma unroll
+        for (uint32_t q = 0; q < 2; ++q) {
+            const U4 v = philox4x32_10(U4{node, step, 0u, q}, a.key0, a.key1);
+            w[4 * q] = v.x;
+            w[4 * q + 1] = v.y;
+            w[4 * q + 2] = v.z;
+            w[4 * q + 3] = v.w;
+        }
+    }
+    __device__ __forceinline__ uint32_t bits(int k) const {
+        const int t = k - 4;
+        return (t & 1) ? w[t >> 1] >> 16 : w[t >> 1] & 0xffffu;
+    }
+    __device__ __forceinline__ double normal(int) const { return 0.0; }
+};
+template <>
+struct FluidNoise<true> {
+    double g[16];
+    __device__ __forceinline__ FluidNoise(const LbArgs<double, double> &a, uint32_t node, uint32_t step) {
+        if (!a.noisy) return;
+#pragma unroll
+        for (uint32_t q = 0; q < 4; ++q) {
+            const U4 v = philox4x32_10(U4{node, step, 0u, q}, a.key0, a.key1);
+            box_muller(v.x, v.y, g[4 * q], g[4 * q + 1]);
+            box_muller(v.z, v.w, g[4 * q + 2], g[4 * q + 3]);
+        }
+#pragma unroll
+        for (int k = 4; k < Q; ++k) g[k - 4] *= a.ampg[k];
+    }
+    __device__ __forceinline__ uint32_t bits(int) const { return 0u; }
+    __device__ __forceinline__ double normal(int k) const { return g[k - 4]; }
+};
+
 // One thread per node; grid (ceil(nx / blockDim.x), ny, nz).  The variant is
 // a run-time (warp-uniform) flag rather than a template parameter: both
 // variants then execute one compiled instruction sequence, so at m = 1 they
@@ -120,42 +249,41 @@ __device__ __forceinline__ void collide_push_node(const LbArgs<T, S> &a, int x, 
     T f[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) f[i] = St::arith(a.fin + (size_t)i * a.N + r);
-    T rho, rho_m, jx, jy, jz;
-    pop_moments<St::deviation>(f, a.rho_base, rho, rho_m, jx, jy, jz);
-    T Fx, Fy, Fz;
-    const int sl = active_slot(a.occw[((size_t)y + (size_t)a.ny * z) * a.occ_words + (x >> 5)], x);
-    if (C || sl >= 0 || a.variant == LBMD_VARIANT_B) {
-        // the record j = fix(j*) + sum of fixed-point transfers: the
-        // difference is exactly the accumulated transfer J_acc (an active
-        // node's record is its compact one -- variant A: the accumulating
-        // copy; B and C: an inactive node's is the node field)
-        const typename P::node4 n = sl >= 0 ? a.cact[sl] : a.node[r];
-        Fx = P::from_fix(P::jx_of(n) - P::to_fix(jx, a.fs), a.fis);
-        Fy = P::from_fix(P::jy_of(n) - P::to_fix(jy, a.fs), a.fis);
-        Fz = P::from_fix(P::jz_of(n) - P::to_fix(jz, a.fs), a.fis);
-    } else {
-        // variant A, inactive node: J_acc holds what migrants handed over
-        // (rarely anything; cleared only where set)
-        const typename P::node4 J = a.jacc[r];
-        Fx = P::from_fix(P::jx_of(J), a.fis);
-        Fy = P::from_fix(P::jy_of(J), a.fis);
-        Fz = P::from_fix(P::jz_of(J), a.fis);
-        if ((P::jx_of(J) | P::jy_of(J) | P::jz_of(J)) != 0) {
-            typename P::node4 zero;
-            zero.x = zero.y = zero.z = zero.w = 0;
-            a.jacc[r] = zero;
+    if constexpr (sizeof(T) == 8) {
+        typename P::fix J[3];
+        bool done = RELAX_FULL && a.fx.usable && in_fixed_range(f, a.fx.e);
+        if (RELAX_FULL && done) {
+            FixedMoments o;
+            fixed_moments(f, a.fx.e, o);
+            node_transfer<C>(a, r, x, y, z, record_momentum(o.j[0]), record_momentum(o.j[1]), record_momentum(o.j[2]),
+                             J);
+            const FluidNoise<GAUSS> noise(a, r, (uint32_t)step);
+            done = collide_fixed<C, GAUSS>(o, J, a.gamma_shear, a.g, a.fx, a.noisy != 0, noise, f);
+            if (!done) collide_node_fp64<GAUSS, C>(a, r, (uint32_t)step, J, f);
+        } else {
+            const NodeSums<T> s = node_sums<false>(f, T(0), a.fs, a.fx.e);
+            node_transfer<C>(a, r, x, y, z, s.ix, s.iy, s.iz, J);
+            if (RELAX_FULL)
+                collide_node_fp64<GAUSS, C>(a, r, (uint32_t)step, J, f);
+            else
+                collide_with_transfer<RELAX_FULL, GAUSS, C>(a, f, s, J, r, (uint32_t)step);
         }
-    }
-    if (C && !(Fx == T(0) && Fy == T(0) && Fz == T(0))) {
-        apply_transfer(f, rho, jx, jy, jz, Fx, Fy, Fz, a.gamma_bulk, a.gamma_shear);
+    } else {
+        T rho, rho_m, jx, jy, jz;
         pop_moments<St::deviation>(f, a.rho_base, rho, rho_m, jx, jy, jz);
-        Fx = Fy = Fz = T(0);
+        T Fx, Fy, Fz;
+        node_force<T, S, C>(a, r, x, y, z, jx, jy, jz, Fx, Fy, Fz);
+        if (C && !(Fx == T(0) && Fy == T(0) && Fz == T(0))) {
+            apply_transfer(f, rho, jx, jy, jz, Fx, Fy, Fz, a.gamma_bulk, a.gamma_shear);
+            pop_moments<St::deviation>(f, a.rho_base, rho, rho_m, jx, jy, jz);
+            Fx = Fy = Fz = T(0);
+        }
+        Fx += a.g[0];
+        Fy += a.g[1];
+        Fz += a.g[2];
+        collide<T, RELAX_FULL, LbArgs<T, S>, GAUSS>(f, rho, rho_m, jx, jy, jz, Fx, Fy, Fz, a, a.key0, a.key1, r,
+                                                    (uint32_t)step);
     }
-    Fx += a.g[0];
-    Fy += a.g[1];
-    Fz += a.g[2];
-    collide<T, RELAX_FULL, LbArgs<T, S>, GAUSS>(f, rho, rho_m, jx, jy, jz, Fx, Fy, Fz, a, a.key0, a.key1, r,
-                                                (uint32_t)step);
 
     const int xm = x == 0 ? a.nx - 1 : x - 1, xp = x == a.nx - 1 ? 0 : x + 1;
     const int ym = y == 0 ? a.ny - 1 : y - 1, yp = y == a.ny - 1 ? 0 : y + 1;
@@ -192,12 +320,12 @@ __device__ __forceinline__ void collide_push_node(const LbArgs<T, S> &a, int x, 
 // Gaussian-noise and partial-relaxation forms keep 6 (3 in FP64).
 template <typename T, typename S, bool RELAX_FULL, bool GAUSS, bool C>
 constexpr int collide_min_blocks() {
-    return sizeof(T) == 8 ? 3 : C ? 5 : (RELAX_FULL && !GAUSS && !PopStore<S, T>::stochastic ? 7 : 6);
+    return sizeof(T) == 8 ? (RELAX_FULL ? 2 : 3) : C ? 5 : (RELAX_FULL && !GAUSS && !PopStore<S, T>::stochastic ? 7 : 6);
 }
 
 template <typename T, typename S, bool RELAX_FULL, bool GAUSS, bool C>
 __global__ void __launch_bounds__(256, (collide_min_blocks<T, S, RELAX_FULL, GAUSS, C>()))
-    lb_collide_push(LbArgs<T, S> a) {
+    lb_collide_push(const __grid_constant__ LbArgs<T, S> a) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
     // the step counter, read before the fallback kernel advances it; it also
@@ -246,7 +374,7 @@ __global__ void __launch_bounds__(256, (collide_min_blocks<T, S, RELAX_FULL, GAU
     }
     if (x < a.nx)
         node_moments_at<T, S>(a.fout, a.node, a.occw_new, a.cact_new, a.cact_new2, a.occ_words, a.N, a.nx, a.ny,
-                              a.rho_base, a.fs, a.range_flag, x, y, t);
+                              a.rho_base, a.fs, a.fx.e, a.range_flag, x, y, t);
 }
 
 // The moments the collide kernel left: node rows of plane 0 and of the last
@@ -256,7 +384,8 @@ template <typename T, typename S>
 __global__ void __launch_bounds__(256)
     moments_rest_kernel(const S *__restrict__ f, typename Prec<T>::node4 *node, const uint2 *occw,
                         typename Prec<T>::node4 *cact, typename Prec<T>::node4 *cact2, int occ_words, int64_t N,
-                        int nx, int ny, int nz, T rho_base, T fs, int32_t *range_flag, const int32_t *missed, const int32_t *missed_list,
+                        int nx, int ny, int nz, T rho_base, T fs, int e, int32_t *range_flag, const int32_t *missed,
+                        const int32_t *missed_list,
                         unsigned long long *missed_total, unsigned long long *lb_step) {
     const int gx = (nx + (int)blockDim.x - 1) / (int)blockDim.x;
     const int rows = gx * ny;
@@ -277,7 +406,7 @@ __global__ void __launch_bounds__(256)
         const int xb = b % gx, rest = b / gx, y = rest % ny, t = rest / ny;
         const int x = xb * (int)blockDim.x + (int)threadIdx.x;
         if (x < nx)
-            node_moments_at<T, S>(f, node, occw, cact, cact2, occ_words, N, nx, ny, rho_base, fs, range_flag, x, y,
+            node_moments_at<T, S>(f, node, occw, cact, cact2, occ_words, N, nx, ny, rho_base, fs, e, range_flag, x, y,
                                   t);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -290,10 +419,10 @@ template <typename T, typename S>
 __global__ void __launch_bounds__(256)
     node_moments_kernel(const S *__restrict__ f, typename Prec<T>::node4 *node, const uint2 *occw,
                         typename Prec<T>::node4 *cact, typename Prec<T>::node4 *cact2, int occ_words, int64_t N,
-                        int nx, int ny, T rho_base, T fs, int32_t *range_flag) {
+                        int nx, int ny, T rho_base, T fs, int e, int32_t *range_flag) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= nx) return;
-    node_moments_at<T, S>(f, node, occw, cact, cact2, occ_words, N, nx, ny, rho_base, fs, range_flag, x, blockIdx.y,
+    node_moments_at<T, S>(f, node, occw, cact, cact2, occ_words, N, nx, ny, rho_base, fs, e, range_flag, x, blockIdx.y,
                           blockIdx.z);
 }
 
@@ -368,6 +497,7 @@ static cudaError_t lb_step_t(lbmd_ctx *ctx) {
     a.key1 = (uint32_t)(ctx->p.seed >> 32);
     a.lb_step = ctx->d_lb_step;
     a.noisy = ctx->co.noisy;
+    a.fx = fixed_constants(ctx->fix.e, ctx->co.noise_amp, ctx->co.body_force);
     a.variant = ctx->p.variant;
     const dim3 block = node_block(ctx), grid = node_grid(ctx, block);
     cudaError_t e = cudaMemsetAsync(ctx->lb_missed, 0, sizeof(int32_t), ctx->stream);
@@ -382,7 +512,7 @@ static cudaError_t lb_step_t(lbmd_ctx *ctx) {
     moments_rest_kernel<T, S><<<2 * ctx->sm_count, block, 0, ctx->stream>>>(
         a.fout, a.node, a.occw_new, a.cact_new, a.cact_new2, a.occ_words, ctx->N, ctx->p.nx, ctx->p.ny, ctx->p.nz,
         a.rho_base,
-        a.fs, ctx->range_flag, ctx->lb_missed, ctx->missed_list, ctx->missed_total, ctx->d_lb_step);
+        a.fs, ctx->fix.e, ctx->range_flag, ctx->lb_missed, ctx->missed_list, ctx->missed_total, ctx->d_lb_step);
     return cudaGetLastError();
 }
 
@@ -396,7 +526,7 @@ static cudaError_t node_moments_t(lbmd_ctx *ctx) {
         active_words_now(ctx), static_cast<typename Prec<T>::node4 *>(active_records_now(ctx)),
         static_cast<typename Prec<T>::node4 *>(active_records_copy(ctx, (int)(ctx->lb_step & 1))),
         active_words(ctx->p.nx), ctx->N, ctx->p.nx, ctx->p.ny, rest_density<T, S>(ctx), (T)ctx->fix.scale,
-        ctx->range_flag);
+        ctx->fix.e, ctx->range_flag);
     return cudaGetLastError();
 }
 

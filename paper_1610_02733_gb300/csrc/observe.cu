@@ -14,6 +14,7 @@
 // become doubles through their bit fields (exact, integer pipes).  Doubles
 // are added only per block and in the final reduction.
 #include "lb_core.cuh"
+#include "lb_fixed.cuh"
 #include "lbmd_ctx.h"
 #include "lbmd_device.cuh"
 #include "particle_core.cuh"
@@ -354,7 +355,7 @@ __global__ void pops_to_double_kernel(const S *f, int64_t first, int64_t count, 
 template <typename T, typename S>
 __global__ void pops_c_to_double_kernel(const S *f, const typename Prec<T>::node4 *node, const uint2 *occw,
                                         const typename Prec<T>::node4 *cact, int W, int nx, T rho_base, T gamma_bulk,
-                                        T gamma_shear, T fs, T fis, int64_t first, int64_t count, int64_t N,
+                                        T gamma_shear, T fs, T fis, int e, int64_t first, int64_t count, int64_t N,
                                         double rho0, double *dst) {
     using P = Prec<T>;
     using St = PopStore<S, T>;
@@ -365,14 +366,13 @@ __global__ void pops_c_to_double_kernel(const S *f, const typename Prec<T>::node
     T fl[Q];
 #pragma unroll
     for (int q = 0; q < Q; ++q) fl[q] = St::arith(f + (int64_t)q * N + r);
-    T rho, rho_m, jx, jy, jz;
-    pop_moments<St::deviation>(fl, rho_base, rho, rho_m, jx, jy, jz);
+    const NodeSums<T> s = node_sums<St::deviation>(fl, rho_base, fs, e);
     const int sl = active_slot(occw[(size_t)(r / nx) * W + (x >> 5)], x);
     const typename P::node4 n = sl >= 0 ? cact[sl] : node[r];
-    const T Fx = P::from_fix(P::jx_of(n) - P::to_fix(jx, fs), fis), Fy = P::from_fix(P::jy_of(n) - P::to_fix(jy, fs), fis),
-            Fz = P::from_fix(P::jz_of(n) - P::to_fix(jz, fs), fis);
+    const T Fx = P::from_fix(P::jx_of(n) - s.ix, fis), Fy = P::from_fix(P::jy_of(n) - s.iy, fis),
+            Fz = P::from_fix(P::jz_of(n) - s.iz, fis);
     if (!(Fx == T(0) && Fy == T(0) && Fz == T(0)))
-        apply_transfer(fl, rho, jx, jy, jz, Fx, Fy, Fz, gamma_bulk, gamma_shear);
+        apply_transfer(fl, s.rho, s.jx, s.jy, s.jz, Fx, Fy, Fz, gamma_bulk, gamma_shear);
     T v = T(0);
 #pragma unroll
     for (int q = 0; q < Q; ++q)
@@ -394,7 +394,7 @@ __global__ void pops_from_double_kernel(S *f, int64_t first, int64_t count, int6
 template <typename T, typename S>
 __global__ void node_to_double_kernel(const typename Prec<T>::node4 *node, const typename Prec<T>::node4 *jacc,
                                       const uint2 *occw, const typename Prec<T>::node4 *cacc, int W, int nx,
-                                      const S *f, int64_t N, T rho0, T fs, T fis, int64_t first, int64_t count,
+                                      const S *f, int64_t N, T rho0, T fs, T fis, int e, int64_t first, int64_t count,
                                       double *dst, int transfer_only, int variant) {
     using P = Prec<T>;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -427,11 +427,10 @@ __global__ void node_to_double_kernel(const typename Prec<T>::node4 *node, const
         T fl[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i) fl[i] = PopStore<S, T>::load(f + (int64_t)i * N + r, T(WEIGHT(i)) * rho0);
-        T rho, jx, jy, jz;
-        node_moments(fl, rho, jx, jy, jz);
-        dst[3 * t + 0] = (double)P::from_fix(P::jx_of(n) - P::to_fix(jx, fs), fis);
-        dst[3 * t + 1] = (double)P::from_fix(P::jy_of(n) - P::to_fix(jy, fs), fis);
-        dst[3 * t + 2] = (double)P::from_fix(P::jz_of(n) - P::to_fix(jz, fs), fis);
+        const NodeSums<T> s = node_sums<false>(fl, T(0), fs, e);
+        dst[3 * t + 0] = (double)P::from_fix(P::jx_of(n) - s.ix, fis);
+        dst[3 * t + 1] = (double)P::from_fix(P::jy_of(n) - s.iy, fis);
+        dst[3 * t + 2] = (double)P::from_fix(P::jz_of(n) - s.iz, fis);
     }
 }
 
@@ -524,7 +523,7 @@ static cudaError_t pops_to_double_t(lbmd_ctx *ctx, int64_t first, int64_t count,
             static_cast<const S *>(ctx->f[ctx->cur]), static_cast<const N4 *>(ctx->node), active_words_now(ctx),
             static_cast<const N4 *>(active_records_now(ctx)), active_words(ctx->p.nx), ctx->p.nx,
             rest_density<T, S>(ctx), (T)ctx->co.gamma_bulk, (T)ctx->co.gamma_shear, (T)ctx->fix.scale,
-            (T)ctx->fix.inv_scale, first, count, ctx->N, ctx->p.rho0, dst);
+            (T)ctx->fix.inv_scale, ctx->fix.e, first, count, ctx->N, ctx->p.rho0, dst);
         return cudaGetLastError();
     }
     pops_to_double_kernel<T, S><<<nblocks(count), 256, 0, ctx->stream>>>(
@@ -546,7 +545,7 @@ static cudaError_t node_to_double_t(lbmd_ctx *ctx, int64_t first, int64_t count,
         static_cast<const N4 *>(ctx->node), static_cast<const N4 *>(ctx->jacc),
         active_words_now(ctx), static_cast<const N4 *>(active_records_acc(ctx)), active_words(ctx->p.nx),
         ctx->p.nx, static_cast<const S *>(ctx->f[ctx->cur]), ctx->N, (T)ctx->p.rho0, (T)ctx->fix.scale,
-        (T)ctx->fix.inv_scale, first, count, dst, transfer_only ? 1 : 0, ctx->p.variant);
+        (T)ctx->fix.inv_scale, ctx->fix.e, first, count, dst, transfer_only ? 1 : 0, ctx->p.variant);
     return cudaGetLastError();
 }
 
