@@ -71,58 +71,6 @@ __host__ __device__ __forceinline__ long long mul_hi64(long long a, long long b)
     return (long long)(((__int128)a * b) >> 64);
 #endif
 }
-__host__ __device__ __forceinline__ int clz64(unsigned long long v) {
-#ifdef __CUDA_ARCH__
-    return __clzll((long long)v);
-#else
-    return v ? __builtin_clzll(v) : 64;
-#endif
-}
-__host__ __device__ __forceinline__ unsigned long long bits_of(double v) {
-#ifdef __CUDA_ARCH__
-    return (unsigned long long)__double_as_longlong(v);
-#else
-    unsigned long long u;
-    memcpy(&u, &v, 8);
-    return u;
-#endif
-}
-__host__ __device__ __forceinline__ double double_of(unsigned long long u) {
-#ifdef __CUDA_ARCH__
-    return __longlong_as_double((long long)u);
-#else
-    double v;
-    memcpy(&v, &u, 8);
-    return v;
-#endif
-}
-
-// v rounded to units of 2^-scale (half away from zero), for |v| < 2^(62 - scale)
-// (anything for a larger one); the binary64 fields are shifted as integers.
-__host__ __device__ __forceinline__ long long to_fixed(double v, int scale) {
-    const unsigned long long u = bits_of(v);
-    const int ex = (int)((u >> 52) & 0x7ffu);
-    const unsigned long long m = ((u << 10) & 0x3fffffffffffffffull) | 0x4000000000000000ull;  // 2^62 <= m < 2^63
-    int r = 1023 + 62 - scale - ex;  // v = m 2^(ex - 1023 - 62)
-    r = r > 64 ? 64 : r < 1 ? 1 : r;  // below half a unit: m >> 63 = 0
-    const unsigned long long q = ((m >> (r - 1)) + 1ull) >> 1;
-    const long long s = (long long)u >> 63;
-    return (long long)(q ^ (unsigned long long)s) - s;
-}
-
-// the integer v times 2^-scale, rounded to nearest even
-__host__ __device__ __forceinline__ double from_fixed(long long v, int scale) {
-    const long long s = v >> 63;
-    const unsigned long long a = (unsigned long long)((v ^ s) - s);
-    const int lz = clz64(a) & 63;
-    const unsigned long long m = a << lz;
-    const unsigned long long q = m >> 11;
-    const unsigned up = ((unsigned)(m & 0x7ffu) + (unsigned)(q & 1ull)) > 0x400u ? 1u : 0u;
-    unsigned long long u = ((unsigned long long)(unsigned)(1023 + 63 - lz - scale - 1) << 52) + q + up;
-    u = a ? u : 0ull;
-    return double_of(u | ((unsigned long long)s & 0x8000000000000000ull));
-}
-
 // Whether all populations are below 2^(e - 1): one compare on the largest
 // exponent field (NaN and infinity have the largest).
 __host__ __device__ __forceinline__ bool in_fixed_range(const double f[Q], int e) {

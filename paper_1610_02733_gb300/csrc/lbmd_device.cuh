@@ -19,6 +19,7 @@
 #pragma once
 
 #include <cstdint>
+#include <cstring>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -81,6 +82,64 @@ __host__ __device__ constexpr double BNORM(int k) {
 }
 
 // ---------------------------------------------------------------------------
+// FP64 <-> 64-bit integers through the binary64 fields.  The FP64 pipes of
+// this GPU, which also make the hardware conversions, issue 2 operations per
+// SM and clock against 64 or more integer ones, so a dozen integer
+// instructions cost less than one conversion.
+// ---------------------------------------------------------------------------
+__host__ __device__ __forceinline__ int clz64(unsigned long long v) {
+#ifdef __CUDA_ARCH__
+    return __clzll((long long)v);
+#else
+    return v ? __builtin_clzll(v) : 64;
+#endif
+}
+__host__ __device__ __forceinline__ unsigned long long bits_of(double v) {
+#ifdef __CUDA_ARCH__
+    return (unsigned long long)__double_as_longlong(v);
+#else
+    unsigned long long u;
+    memcpy(&u, &v, 8);
+    return u;
+#endif
+}
+__host__ __device__ __forceinline__ double double_of(unsigned long long u) {
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((long long)u);
+#else
+    double v;
+    memcpy(&v, &u, 8);
+    return v;
+#endif
+}
+
+// v rounded to units of 2^-scale (half away from zero), for |v| < 2^(62 - scale)
+// (anything for a larger one); the binary64 fields are shifted as integers.
+__host__ __device__ __forceinline__ long long to_fixed(double v, int scale) {
+    const unsigned long long u = bits_of(v);
+    const int ex = (int)((u >> 52) & 0x7ffu);
+    const unsigned long long m = ((u << 10) & 0x3fffffffffffffffull) | 0x4000000000000000ull;  // 2^62 <= m < 2^63
+    int r = 1023 + 62 - scale - ex;  // v = m 2^(ex - 1023 - 62)
+    r = r > 64 ? 64 : r < 1 ? 1 : r;  // below half a unit: m >> 63 = 0
+    const unsigned long long q = ((m >> (r - 1)) + 1ull) >> 1;
+    const long long s = (long long)u >> 63;
+    return (long long)(q ^ (unsigned long long)s) - s;
+}
+
+// the integer v times 2^-scale, rounded to nearest even
+__host__ __device__ __forceinline__ double from_fixed(long long v, int scale) {
+    const long long s = v >> 63;
+    const unsigned long long a = (unsigned long long)((v ^ s) - s);
+    const int lz = clz64(a) & 63;
+    const unsigned long long m = a << lz;
+    const unsigned long long q = m >> 11;
+    const unsigned up = ((unsigned)(m & 0x7ffu) + (unsigned)(q & 1ull)) > 0x400u ? 1u : 0u;
+    unsigned long long u = ((unsigned long long)(unsigned)(1023 + 63 - lz - scale - 1) << 52) + q + up;
+    u = a ? u : 0ull;
+    return double_of(u | ((unsigned long long)s & 0x8000000000000000ull));
+}
+
+// ---------------------------------------------------------------------------
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): 10 rounds of the
 // multiply-xor bijection with Weyl-sequence key updates.
 // ---------------------------------------------------------------------------
@@ -106,7 +165,7 @@ __device__ __forceinline__ U4 philox4x32_10(U4 c, uint32_t k0, uint32_t k1) {
 // sqrt(12) ((x + 1/2) 2^-32 - 1/2).  The FP64 form is exact; the FP32 form
 // centres first, (x - 2^31 + 1/2) 2^-32, so only one rounding remains.
 __device__ __forceinline__ double unit_uniform_d(uint32_t x) {
-    return 3.4641016151377544 * (((double)x + 0.5) * 2.3283064365386963e-10 - 0.5);
+    return 3.4641016151377544 * from_fixed(2ll * (long long)x + 1ll - (1ll << 32), 33);
 }
 __device__ __forceinline__ float unit_uniform_f(uint32_t x) {
     const float centred = (float)(int32_t)(x ^ 0x80000000u) + 0.5f;
@@ -228,9 +287,22 @@ struct Prec<double> {
     using fix = long long;
     using node4 = L4;
     static constexpr int SCALE_LOG2 = 56;  // scale at rho0 <= 1: 2^56
-    __device__ static __forceinline__ fix to_fix(double v, double s) { return __double2ll_rn(v * s); }
-    __device__ static __forceinline__ fix to_fix_neg(double d, double ps) { return __double2ll_rn(d * ps); }
-    __device__ static __forceinline__ double from_fix(fix v, double inv_s) { return (double)v * inv_s; }
+    // rounded to nearest; 2^62 and more, and NaN, by the hardware conversion
+    // (volatile: kept inside its branch)
+    __device__ static __forceinline__ fix to_fix(double v, double s) { return rounded(v * s); }
+    __device__ static __forceinline__ fix to_fix_neg(double d, double ps) { return rounded(d * ps); }
+    __device__ static __forceinline__ fix rounded(double v) {
+        if (((unsigned)__double2hiint(v) & 0x7fffffffu) >= (unsigned)(1023 + 62) << 20) {
+            fix r;
+            asm volatile("cvt.rni.s64.f64 %0, %1;" : "=l"(r) : "d"(v));
+            return r;
+        }
+        return to_fixed(v, 0);
+    }
+    // inv_s: a power of two
+    __device__ static __forceinline__ double from_fix(fix v, double inv_s) {
+        return from_fixed(v, 1023 - (__double2hiint(inv_s) >> 20));
+    }
     // |v| >= 2^62, half the range of a field
     __device__ static __forceinline__ bool beyond_half(fix v) {
         return (unsigned long long)v + 0x4000000000000000ull >= 0x8000000000000000ull;
@@ -258,9 +330,9 @@ struct Prec<double> {
         *rec = n;
     }
     __device__ static __forceinline__ real4 make4(double a, double b, double c, double d) { return D4{a, b, c, d}; }
-    __device__ static __forceinline__ int64_t cell_of(const real4 &p) { return (int64_t)p.w; }
+    __device__ static __forceinline__ int64_t cell_of(const real4 &p) { return to_fixed(p.w, 0); }
     __device__ static __forceinline__ real4 make_pos(double fx, double fy, double fz, int64_t cell) {
-        return D4{fx, fy, fz, (double)cell};
+        return D4{fx, fy, fz, from_fixed(cell, 0)};
     }
 };
 

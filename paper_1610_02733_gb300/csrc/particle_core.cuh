@@ -54,9 +54,17 @@ __device__ __forceinline__ void corner_rows(const CellXYZ &c, int ny, int nz, ui
 // The drift frac + dt v is one explicit fused multiply-add, so every kernel
 // that moves particles rounds it the same way whatever the compiler would
 // contract.
+// A coordinate that stays within its cell, 0 <= x < 1 (told by its bits), is done
+// at once.
+__device__ __forceinline__ bool within_cell(float x) { return (unsigned)__float_as_int(x) < 0x3f800000u; }
+__device__ __forceinline__ bool within_cell(double x) { return (unsigned)__double2hiint(x) < 0x3ff00000u; }
 template <typename T>
 __device__ __forceinline__ void advance(T &frac, int &c, T dt, T v, int n) {
     T x = fma(dt, v, frac);
+    if (within_cell(x)) {
+        frac = x;
+        return;
+    }
     T s = floor(x);
     x -= s;
     if (x >= T(1)) {  // a tiny negative offset rounded up to the next node

@@ -1027,7 +1027,7 @@ static cudaError_t md_substep_t(lbmd_ctx *ctx, int substep) {
     if (atomic && cons) {
         // spread by the bond / pair kernel above
     } else if (atomic) {
-        const unsigned sb = (unsigned)std::min<int64_t>(ctx->sm_count, (ctx->np + 255) / 256);
+        const unsigned sb = (unsigned)((ctx->np + 255) / 256);
         migrant_spread_kernel<T><<<sb, 256, 0, ctx->stream>>>(a, 1);
     } else {
         const int rows = (int)((int64_t)ctx->p.ny * ctx->p.nz);
