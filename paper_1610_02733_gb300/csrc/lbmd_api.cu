@@ -56,7 +56,8 @@ void free_all(lbmd_ctx *ctx) {
                     ctx->nb_count,     ctx->nb_invalid,    ctx->nb_ref4,       ctx->range_flag,
                     ctx->missed_total, ctx->dev_error,     ctx->arow[0],       ctx->arow[1],
                     ctx->tile_table[0], ctx->tile_table[1], ctx->edge_acc,  ctx->tile_flag,
-                    ctx->late_rows,    ctx->late_count, ctx->ccw};
+                    ctx->late_rows,    ctx->late_count, ctx->ccw,          ctx->phase_bar,
+                    ctx->nb_end};
     for (void *b : bufs)
         if (b) cudaFree(b);
     for (int b = 0; b < 2; ++b) {
@@ -230,6 +231,7 @@ lbmd_status lbmd_create(const lbmd_params *p, lbmd_ctx **out) {
         {(void **)&ctx->arow[1], arow_bytes},
         {(void **)&ctx->ccw, occ_bytes / 2},
         {(void **)&ctx->dev_error, sizeof(int32_t)},
+        {(void **)&ctx->phase_bar, 2 * sizeof(uint32_t)},
         {&ctx->tile_table[0], table_bytes},
         {&ctx->tile_table[1], table_bytes},
         {&ctx->edge_acc, table_bytes ? (size_t)ctx->cact_cap * md_tile_edge_bytes(ctx) : 0},
@@ -266,6 +268,7 @@ lbmd_status lbmd_create(const lbmd_params *p, lbmd_ctx **out) {
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->missed_total, 0, sizeof(unsigned long long), ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->range_flag, 0, sizeof(int32_t), ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->dev_error, 0, sizeof(int32_t), ctx->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->phase_bar, 0, 2 * sizeof(uint32_t), ctx->stream);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(ctx->red_partial, 0, (size_t)ctx->red_blocks * 8 * sizeof(double) + 16, ctx->stream);
     if (e == cudaSuccess && ctx->edge_acc)
@@ -327,12 +330,12 @@ static void drop_cycle_graphs(lbmd_ctx *ctx) {
 static lbmd_status ensure_nb_lists(lbmd_ctx *ctx) {
     if (ctx->nb_list) return LBMD_OK;
     const size_t maxp = (size_t)std::max<int64_t>(ctx->p.max_particles, 1);
-    void *bufs[4] = {nullptr, nullptr, nullptr, nullptr};
-    const size_t bytes[4] = {maxp * LBMD_NB_MAX * sizeof(int32_t), maxp * sizeof(int32_t), sizeof(int32_t),
-                             maxp * 4 * real_size(ctx)};
-    for (int k = 0; k < 4; ++k)
+    void *bufs[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+    const size_t bytes[5] = {maxp * LBMD_NB_MAX * sizeof(int32_t), maxp * sizeof(int32_t), sizeof(int32_t),
+                             maxp * 4 * real_size(ctx), maxp * 32};
+    for (int k = 0; k < 5; ++k)
         if (cudaMalloc(&bufs[k], bytes[k]) != cudaSuccess) {
-            for (int q = 0; q < 4; ++q)
+            for (int q = 0; q < 5; ++q)
                 if (bufs[q]) cudaFree(bufs[q]);
             cudaGetLastError();
             return fail(ctx, LBMD_ERR_OOM, "Lennard-Jones neighbour lists");
@@ -341,6 +344,7 @@ static lbmd_status ensure_nb_lists(lbmd_ctx *ctx) {
     ctx->nb_count = static_cast<int32_t *>(bufs[1]);
     ctx->nb_invalid = static_cast<int32_t *>(bufs[2]);
     ctx->nb_ref4 = bufs[3];
+    ctx->nb_end = static_cast<uint8_t *>(bufs[4]);
     return LBMD_OK;
 }
 
@@ -563,6 +567,7 @@ lbmd_status lbmd_run_cycles(lbmd_ctx *ctx, int64_t n) {
         ctx->pcur = ctx->cycle_post[key][1];
         ctx->pv = ctx->cycle_post[key][2];
         ctx->rec = 0;
+        ctx->in_buckets = true;  // the LB step re-ordered them
         ctx->lb_step += 1;
         ctx->md_step += ctx->p.n_sub;
     }
@@ -579,7 +584,7 @@ lbmd_status lbmd_observables(lbmd_ctx *ctx, lbmd_observables_t *out) {
     CK(ctx, cudaMemcpyAsync(h, ctx->red_out, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
     CK(ctx, cudaStreamSynchronize(ctx->stream));
     if (h[9] != 0.0)
-        return fail(ctx, LBMD_ERR_CUDA, "a kernel's bounded wait for its own bulk copies gave up: results are invalid");
+        return fail(ctx, LBMD_ERR_CUDA, "a kernel's bounded wait (bulk copies or grid barrier) gave up: results are invalid");
     out->mass = h[0];
     for (int d = 0; d < 3; ++d) {
         out->p_fluid[d] = h[1 + d];
@@ -745,7 +750,7 @@ lbmd_status finalise_observables(lbmd_ctx *ctx, int s) {
     out->lb_step = ctx->obs_lb[s];
     out->md_step = ctx->obs_md[s];
     if (h[9] != 0.0)
-        return fail(ctx, LBMD_ERR_CUDA, "a kernel's bounded wait for its own bulk copies gave up: results are invalid");
+        return fail(ctx, LBMD_ERR_CUDA, "a kernel's bounded wait (bulk copies or grid barrier) gave up: results are invalid");
     for (int c = 0; c < 8; ++c)
         if (!is_finite_d(h[c])) return fail(ctx, LBMD_ERR_NONFINITE, "non-finite observable");
     if (h[8] != 0.0)

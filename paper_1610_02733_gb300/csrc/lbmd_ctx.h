@@ -152,6 +152,10 @@ struct lbmd_ctx {
     unsigned long long *missed_total;  // rows left to the fallback since creation
     int fuse_spin;         // polls of a collide block's wait (0: no fused moments)
     int sm_count;
+    uint32_t *phase_bar;    // grid barrier of the MD phase (arrivals, finished blocks)
+    int64_t phase_threads;  // threads of it resident at once
+    int phase_cluster;      // largest cluster of its blocks
+    bool in_buckets;        // the particles are where the last re-ordering bucketed them
     int gather_warps;  // warps per block of the variant B row gather
     bool a_frozen_copy;  // variant A: interpolate from a frozen copy of the compact records (else the node field)
     int32_t *bond_count, *bond_partner;
@@ -160,11 +164,12 @@ struct lbmd_ctx {
     // Lennard-Jones between all particles (Kremer-Grest monomers); off while
     // lj_rc == 0
     double lj_eps, lj_sigma, lj_rc;
-    // Verlet lists of the LJ forces: per id the ids within lj_rc +
-    // LBMD_NB_SKIN, ascending, and the position at the build; a flag set once
+    // Verlet lists of the LJ forces: per id the slots of the ids within lj_rc +
+    // LBMD_NB_SKIN, ordered by (id mod 32, id), and the position at the build; a flag set once
     // any particle moved more than half the skin since (the lists are then not
     // used until the next re-ordering rebuilds them)
     int32_t *nb_list, *nb_count, *nb_invalid;
+    uint8_t *nb_end;
     void *nb_ref4;
     double *staging;   // device staging buffer for host <-> device conversions
     int64_t staging_len;

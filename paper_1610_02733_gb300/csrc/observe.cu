@@ -588,6 +588,7 @@ cudaError_t launch_particles_from_double(lbmd_ctx *ctx, int64_t first, int64_t c
                                          const double *vel, const double *mass, bool set_pos, bool set_vel,
                                          bool set_mass) {
     if (count <= 0) return cudaSuccess;
+    if (set_pos) ctx->in_buckets = false;
     const int b = ctx->pcur;
     const int assign = set_mass ? 1 : 0;  // only lbmd_add_particles sets masses
     if (ctx->p.precision == LBMD_FP64)

@@ -23,7 +23,8 @@ struct PArgs {
     T lj_eps24, lj_sig2, lj_rc2;  // Lennard-Jones: 24 eps, sigma^2, r_cut^2
     float lj_filter2;             // (r_cut + rounding margin of FP32 absolute positions)^2
     // LJ Verlet lists (null when LJ is off)
-    const int32_t *nb_list, *nb_count;
+    const int32_t *nb_list, *nb_count;  // slots by (id mod 32, id) per id, and how many (-1: too many)
+    const uint8_t *nb_end;              // per id and class: where the class ends in the list
     int32_t *nb_invalid;
     const typename P::real4 *nb_ref4;  // positions at the list build, per id
     T nb_half_skin2;                   // (skin / 2)^2: a larger move since the build voids the lists
@@ -110,13 +111,29 @@ __device__ __forceinline__ void interp_u_cached(T fx, T fy, T fz, const T rho[8]
         add_corner(wx[k & 1] * wy[(k >> 1) & 1] * wz[k >> 2], rho[k], jx[k], jy[k], jz[k], ux, uy, uz);
 }
 
+// Loads through L2 (ld.global.cg), for what other blocks of the same launch
+// write.
+__device__ __forceinline__ int4 load_l2(const int4 *p) { return __ldcg(p); }
+__device__ __forceinline__ float4 load_l2(const float4 *p) { return __ldcg(p); }
+__device__ __forceinline__ L4 load_l2(const L4 *p) {
+    const longlong2 *q = reinterpret_cast<const longlong2 *>(p);
+    const longlong2 a = __ldcg(q), b = __ldcg(q + 1);
+    return L4{a.x, a.y, b.x, b.y};
+}
+__device__ __forceinline__ D4 load_l2(const D4 *p) {
+    const double2 *q = reinterpret_cast<const double2 *>(p);
+    const double2 a = __ldcg(q), b = __ldcg(q + 1);
+    return D4{a.x, a.y, b.x, b.y};
+}
+
 // The records of the 8 corners of cell c, k = ox + 2 oy + 4 oz: the compact
 // record of an active node, the node field entry otherwise (interp_compact 0:
 // always the node field).  All active words are loaded before the first
 // record and all records before the first use, so a thread waits on two
 // round trips to memory and has 8 records in flight; fetching them row by
 // row between the divisions of the interpolation left two.
-template <typename T>
+// L2: read past L1 (the records change during the launch).
+template <bool L2 = false, typename T>
 __device__ __forceinline__ void corner_records(const PArgs<T> &a, const CellXYZ &c, typename Prec<T>::node4 n[8]) {
     using N4 = typename Prec<T>::node4;
     uint32_t rows[4];
@@ -148,11 +165,11 @@ __device__ __forceinline__ void corner_records(const PArgs<T> &a, const CellXYZ 
         }
     }
 #pragma unroll
-    for (int k = 0; k < 8; ++k) n[k] = *ptr[k];
+    for (int k = 0; k < 8; ++k) n[k] = L2 ? load_l2(ptr[k]) : *ptr[k];
 }
 
 // The same for a particle in cell c, its records read from memory.
-template <typename T>
+template <bool L2 = false, typename T>
 __device__ __forceinline__ void interp_u(const PArgs<T> &a, const CellXYZ &c, T fx, T fy, T fz, T &ux, T &uy,
                                          T &uz) {
     using P = Prec<T>;
@@ -160,7 +177,7 @@ __device__ __forceinline__ void interp_u(const PArgs<T> &a, const CellXYZ &c, T 
     corner_rows(c, a.ny, a.nz, rows);
     const int x1 = c.x + 1 == a.nx ? 0 : c.x + 1;
     typename P::node4 nn[8];
-    corner_records(a, c, nn);
+    corner_records<L2>(a, c, nn);
     interp_u_from(fx, fy, fz, a.fis, ux, uy, uz, [&](int q, typename P::node4 &n0, typename P::node4 &n1) {
         n0 = nn[2 * q];
         n1 = nn[2 * q + 1];
@@ -268,20 +285,18 @@ __device__ __forceinline__ void spread_corner_atomic(const PArgs<T> &a, int64_t 
     P::add_transfer(rec, P::to_fix_neg(delta, sx), P::to_fix_neg(delta, sy), P::to_fix_neg(delta, sz));
 }
 
-// All 8 corner transfers of the particle in slot p (position and force read
-// and the cell decoded once).
+// All 8 corner transfers of a particle at offsets (fx, fy, fz) in cell c with
+// the force F.
 template <typename T>
-__device__ __forceinline__ void spread_particle_atomic(const PArgs<T> &a, int64_t p) {
+__device__ __forceinline__ void spread_atomic(const PArgs<T> &a, const CellXYZ &c, T fx, T fy, T fz, T Fx, T Fy,
+                                              T Fz) {
     using P = Prec<T>;
-    const typename P::real4 R = a.old4[p];
-    const typename P::real4 F = a.fc4[p];
-    const CellXYZ c = cell_xyz(P::cell_of(R), a.fd_nx, a.fd_ny);
     uint32_t idx[8], rows[4];
     T delta[8];
-    corners(c, R.x, R.y, R.z, a.nx, a.ny, a.nz, idx, delta);
+    corners(c, fx, fy, fz, a.nx, a.ny, a.nz, idx, delta);
     corner_rows(c, a.ny, a.nz, rows);
     const int x1 = c.x + 1 == a.nx ? 0 : c.x + 1;
-    const T sx = F.x * a.neg_scale_dt, sy = F.y * a.neg_scale_dt, sz = F.z * a.neg_scale_dt;
+    const T sx = Fx * a.neg_scale_dt, sy = Fy * a.neg_scale_dt, sz = Fz * a.neg_scale_dt;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         const int xn = (k & 1) ? x1 : c.x;
@@ -289,6 +304,13 @@ __device__ __forceinline__ void spread_particle_atomic(const PArgs<T> &a, int64_
         typename P::node4 *rec = sl >= 0 ? &a.cact_acc[sl] : &a.inactive_acc[idx[k]];
         P::add_transfer(rec, P::to_fix_neg(delta[k], sx), P::to_fix_neg(delta[k], sy), P::to_fix_neg(delta[k], sz));
     }
+}
+
+// The same for the particle in slot p, from its kept position and force.
+template <typename T>
+__device__ __forceinline__ void spread_particle_atomic(const PArgs<T> &a, int64_t p) {
+    const typename Prec<T>::real4 R = a.old4[p], F = a.fc4[p];
+    spread_atomic(a, cell_xyz(Prec<T>::cell_of(R), a.fd_nx, a.fd_ny), R.x, R.y, R.z, F.x, F.y, F.z);
 }
 
 }  // namespace lbmd

@@ -308,44 +308,6 @@ __global__ void __launch_bounds__(256) migrant_spread_kernel(PArgs<T> a, int all
     }
 }
 
-template <typename T>
-__device__ __forceinline__ T quiet_nan();
-template <>
-__device__ __forceinline__ float quiet_nan<float>() { return __int_as_float(0x7fc00000); }
-template <>
-__device__ __forceinline__ double quiet_nan<double>() { return __longlong_as_double(0x7ff8000000000000LL); }
-
-// Bond force on a particle from a partner at minimum-image separation d
-// (partner minus particle), |d|^2 = r2: g d with
-//   harmonic U = (k/2)(r - r0)^2               g = k (r - r0) / r   (0 at r = 0)
-//   FENE     U = -(k/2) R0^2 ln(1 - (r/R0)^2)  g = k / (1 - (r/R0)^2), R0 = r0
-// (Kremer-Grest springs, Sec. 4); a FENE bond at r >= R0 gives NaN.
-template <typename T>
-__device__ __forceinline__ T bond_gain(uint8_t kind, T k, T r0, T r2) {
-    if (kind == LBMD_BOND_FENE) {
-        const T x = r2 / (r0 * r0);
-        return x < T(1) ? k / (T(1) - x) : quiet_nan<T>();
-    }
-    const T r = sqrt(r2);
-    return r > T(0) ? k * (r - r0) / r : T(0);
-}
-
-// Minimum-image separation of the partner in slot q from a particle at
-// (R, c), through the stored cell indices and offsets.
-template <typename T>
-__device__ __forceinline__ void bond_separation(const PArgs<T> &a, const typename Prec<T>::real4 &R, const CellXYZ &c,
-                                                int64_t q, T &dx, T &dy, T &dz) {
-    using P = Prec<T>;
-    const typename P::real4 S = a.pos4[q];
-    const CellXYZ d = cell_xyz(P::cell_of(S), a.fd_nx, a.fd_ny);
-    dx = T(d.x - c.x) + (S.x - R.x);
-    dy = T(d.y - c.y) + (S.y - R.y);
-    dz = T(d.z - c.z) + (S.z - R.z);
-    dx -= T(a.nx) * rint(dx / T(a.nx));
-    dy -= T(a.ny) * rint(dy / T(a.ny));
-    dz -= T(a.nz) * rint(dz / T(a.nz));
-}
-
 // Bond forces (harmonic or FENE) at the current positions (minimum image),
 // summed per particle over its partners in a fixed order; with KICK, also
 // the second velocity-Verlet half-kick with the stored coupling force.
@@ -357,17 +319,8 @@ __global__ void __launch_bounds__(256) bond_kick_kernel(PArgs<T> a) {
     const typename P::real4 R = a.pos4[p];
     const CellXYZ c = cell_xyz(P::cell_of(R), a.fd_nx, a.fd_ny);
     const int64_t id = a.pid[p];
-    T Fx = T(0), Fy = T(0), Fz = T(0);
-    const int nbond = a.bond_count[id];
-    for (int b = 0; b < nbond; ++b) {
-        const int64_t e = id * LBMD_MAX_BONDS_PER_PARTICLE + b;
-        T dx, dy, dz;
-        bond_separation(a, R, c, a.slot_of[a.bond_partner[e]], dx, dy, dz);
-        const T g = bond_gain(a.bond_kind[e], (T)a.bond_k[e], (T)a.bond_r0[e], dx * dx + dy * dy + dz * dz);
-        Fx += g * dx;
-        Fy += g * dy;
-        Fz += g * dz;
-    }
+    T Fx, Fy, Fz;
+    bond_forces(a, id, R, c, Fx, Fy, Fz);
     a.fcons4[p] = P::make4(Fx, Fy, Fz, T(0));
     if (KICK) {
         typename P::real4 V = a.vel4[p];
@@ -397,29 +350,18 @@ __global__ void __launch_bounds__(256) bond_kick_kernel(PArgs<T> a) {
 // the cut-off); lane b < n_bonds(i) adds bond b.  The lane sums are combined
 // by a fixed butterfly, so the result does not depend on the slot order.
 // With KICK, lane 0 also makes the second velocity-Verlet half-kick.
-template <typename T>
-struct PairTile {
-    static constexpr int N = sizeof(T) == 4 ? 1024 : 512;  // 40 / 26 KB of shared memory
-};
-
 constexpr int PAIR_THREADS = 256;  // eight particles per block
 
 template <typename T, bool KICK>
 __global__ void __launch_bounds__(PAIR_THREADS) pair_kick_kernel(PArgs<T> a) {
     using P = Prec<T>;
-    constexpr int TILE = PairTile<T>::N;
-    __shared__ T s_f[3][TILE];
-    __shared__ int s_c[3][TILE];
-    __shared__ float4 s_abs[TILE];  // FP32 absolute positions, for the filter
+    __shared__ PairTile<T> tile;
     const int lane = threadIdx.x & 31;
     const int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const bool live = i < a.np;
     const int64_t p = live ? a.slot_of[i] : 0;
     const typename P::real4 R = a.pos4[p];
     const CellXYZ c = cell_xyz(P::cell_of(R), a.fd_nx, a.fd_ny);
-    const float xi = (float)(T(c.x) + R.x), yi = (float)(T(c.y) + R.y), zi = (float)(T(c.z) + R.z);
-    const float fnx = (float)a.nx, fny = (float)a.ny, fnz = (float)a.nz;
-    const float inx = 1.0f / fnx, iny = 1.0f / fny, inz = 1.0f / fnz;
     T Fx = T(0), Fy = T(0), Fz = T(0);
     // Verlet lists when they hold every pair within the cut-off (no particle
     // moved more than half the skin since the build, no list overflowed in
@@ -429,95 +371,17 @@ __global__ void __launch_bounds__(PAIR_THREADS) pair_kick_kernel(PArgs<T> a) {
     int use_all = a.nb_list == nullptr || *a.nb_invalid != 0;
     if (!use_all && live && a.nb_count[i] < 0) use_all = 1;
     use_all = __syncthreads_or(use_all);
-    if (!use_all && live) {
-        // the lanes evaluate 32 listed pairs at a time; each term then goes,
-        // in list (= id) order, to the lane that owns its id (j mod 32)
-        const int cnt = a.nb_count[i];
-        const int32_t *L = a.nb_list + i * LBMD_NB_MAX;
-        for (int e0 = 0; e0 < cnt; e0 += 32) {
-            int32_t j = -1;
-            T g = T(0), dx = T(0), dy = T(0), dz = T(0);
-            if (e0 + lane < cnt) {
-                j = L[e0 + lane];
-                const typename P::real4 S = a.pos4[a.slot_of[j]];
-                const CellXYZ d = cell_xyz(P::cell_of(S), a.fd_nx, a.fd_ny);
-                dx = T(nearest_image(d.x - c.x, a.nx)) + (S.x - R.x);
-                dy = T(nearest_image(d.y - c.y, a.ny)) + (S.y - R.y);
-                dz = T(nearest_image(d.z - c.z, a.nz)) + (S.z - R.z);
-                const T r2 = dx * dx + dy * dy + dz * dz;
-                if (r2 < a.lj_rc2) {  // beyond the cut-off: g = 0 adds nothing
-                    const T s = a.lj_sig2 / r2;
-                    const T t = s * s * s;
-                    g = -a.lj_eps24 * (T(2) * t * t - t) / r2;
-                }
-            }
-            const int m = cnt - e0 < 32 ? cnt - e0 : 32;
-            for (int k = 0; k < m; ++k) {
-                const int32_t jk = __shfl_sync(0xffffffffu, j, k);
-                const T gk = __shfl_sync(0xffffffffu, g, k);
-                const T xk = __shfl_sync(0xffffffffu, dx, k);
-                const T yk = __shfl_sync(0xffffffffu, dy, k);
-                const T zk = __shfl_sync(0xffffffffu, dz, k);
-                if ((jk & 31) == lane) {
-                    Fx += gk * xk;
-                    Fy += gk * yk;
-                    Fz += gk * zk;
-                }
-            }
-        }
-    }
-    for (int64_t j0 = 0; use_all && j0 < a.np; j0 += TILE) {
-        const int cnt = a.np - j0 < TILE ? (int)(a.np - j0) : TILE;
-        __syncthreads();  // the previous tile is consumed
-        for (int k = threadIdx.x; k < cnt; k += blockDim.x) {
-            const typename P::real4 S = a.pos4[a.slot_of[j0 + k]];
-            const CellXYZ d = cell_xyz(P::cell_of(S), a.fd_nx, a.fd_ny);
-            s_f[0][k] = S.x;
-            s_f[1][k] = S.y;
-            s_f[2][k] = S.z;
-            s_c[0][k] = d.x;
-            s_c[1][k] = d.y;
-            s_c[2][k] = d.z;
-            s_abs[k] = make_float4((float)(T(d.x) + S.x), (float)(T(d.y) + S.y), (float)(T(d.z) + S.z), 0.0f);
-        }
-        __syncthreads();
-        if (!live) continue;
-        for (int k = lane; k < cnt; k += 32) {
-            // filter on FP32 absolute positions: a pair whose approximate
-            // distance is beyond the cut-off plus the rounding margin is
-            // beyond the cut-off (the exact test below would reject it too)
-            const float4 A = s_abs[k];
-            float ex = A.x - xi, ey = A.y - yi, ez = A.z - zi;
-            ex -= fnx * rintf(ex * inx);
-            ey -= fny * rintf(ey * iny);
-            ez -= fnz * rintf(ez * inz);
-            if (ex * ex + ey * ey + ez * ez >= a.lj_filter2) continue;
-            const int ix = nearest_image(s_c[0][k] - c.x, a.nx);
-            const int iy = nearest_image(s_c[1][k] - c.y, a.ny);
-            const int iz = nearest_image(s_c[2][k] - c.z, a.nz);
-            const T dx = T(ix) + (s_f[0][k] - R.x);
-            const T dy = T(iy) + (s_f[1][k] - R.y);
-            const T dz = T(iz) + (s_f[2][k] - R.z);
-            const T r2 = dx * dx + dy * dy + dz * dz;
-            if (j0 + k != i && r2 < a.lj_rc2) {
-                const T s = a.lj_sig2 / r2;
-                const T t = s * s * s;
-                const T g = -a.lj_eps24 * (T(2) * t * t - t) / r2;
-                Fx += g * dx;
-                Fy += g * dy;
-                Fz += g * dz;
-            }
-        }
-    }
+    if (!use_all && live) listed_pairs(a, i, lane, R, c, Fx, Fy, Fz);  // whole warps
+    if (use_all) all_pairs<false>(a, tile, i, live, lane, R, c, Fx, Fy, Fz);
     if (!live) return;  // whole warps, after the block's last barrier
     if (lane < a.bond_count[i]) {
         const int64_t e = i * LBMD_MAX_BONDS_PER_PARTICLE + lane;
         T dx, dy, dz;
         bond_separation(a, R, c, a.slot_of[a.bond_partner[e]], dx, dy, dz);
         const T g = bond_gain(a.bond_kind[e], (T)a.bond_k[e], (T)a.bond_r0[e], dx * dx + dy * dy + dz * dz);
-        Fx += g * dx;
-        Fy += g * dy;
-        Fz += g * dz;
+        Fx = fma(g, dx, Fx);
+        Fy = fma(g, dy, Fy);
+        Fz = fma(g, dz, Fz);
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
@@ -547,8 +411,10 @@ __global__ void __launch_bounds__(PAIR_THREADS) pair_kick_kernel(PArgs<T> a) {
 // list: the lanes run over the particles of the row buckets
 // within ceil(r_list) rows in y and z (each distinct row once; the buckets'
 // slot ranges are concatenated and shared out 32 at a time), keep the ids
-// j != i closer than r_list = r_cut + skin, and write them in ascending order
-// (each lane ranks its entries by counting the smaller ids).  A particle with
+// j != i closer than r_list = r_cut + skin, and write their slots (fixed until
+// the next re-ordering) ordered by (id mod 32, id), so that a lane of the pair
+// loop reads its own share and nothing else (each lane ranks its entries by
+// counting the smaller ones).  A particle with
 // more than LBMD_NB_MAX candidates gets count -1 (its block then uses all
 // pairs).  The positions at the build are kept per id.
 constexpr int NB_WARPS = 8;
@@ -556,7 +422,7 @@ constexpr int NB_WARPS = 8;
 template <typename T>
 __global__ void __launch_bounds__(32 * NB_WARPS) nb_build_kernel(PArgs<T> a, T rlist2, int reach) {
     using P = Prec<T>;
-    __shared__ int32_t s_ids[NB_WARPS][LBMD_NB_MAX];
+    __shared__ int32_t s_ids[NB_WARPS][LBMD_NB_MAX], s_slots[NB_WARPS][LBMD_NB_MAX];
     __shared__ int s_cnt[NB_WARPS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t q = (int64_t)blockIdx.x * NB_WARPS + warp;
@@ -613,7 +479,10 @@ __global__ void __launch_bounds__(32 * NB_WARPS) nb_build_kernel(PArgs<T> a, T r
             const T dz = T(nearest_image(d.z - c.z, a.nz)) + (S.z - R.z);
             if (dx * dx + dy * dy + dz * dz < rlist2) {
                 const int k = atomicAdd(&s_cnt[warp], 1);
-                if (k < LBMD_NB_MAX) s_ids[warp][k] = j;
+                if (k < LBMD_NB_MAX) {
+                    s_ids[warp][k] = j;
+                    s_slots[warp][k] = sl;
+                }
             }
         }
     }
@@ -623,13 +492,20 @@ __global__ void __launch_bounds__(32 * NB_WARPS) nb_build_kernel(PArgs<T> a, T r
         if (lane == 0) const_cast<int32_t *>(a.nb_count)[i] = -1;
         return;
     }
+    // slots by (id mod 32, id); the end of each class
     int32_t *L = const_cast<int32_t *>(a.nb_list) + (int64_t)i * LBMD_NB_MAX;
     for (int k = lane; k < cnt; k += 32) {
         const int32_t j = s_ids[warp][k];
         int rank = 0;
-        for (int m = 0; m < cnt; ++m) rank += s_ids[warp][m] < j ? 1 : 0;
-        L[rank] = j;
+        for (int m = 0; m < cnt; ++m) {
+            const int32_t o = s_ids[warp][m];
+            rank += (o & 31) < (j & 31) || ((o & 31) == (j & 31) && o < j) ? 1 : 0;
+        }
+        L[rank] = s_slots[warp][k];
     }
+    int end = 0;
+    for (int m = 0; m < cnt; ++m) end += (s_ids[warp][m] & 31) <= lane ? 1 : 0;
+    const_cast<uint8_t *>(a.nb_end)[(int64_t)i * 32 + lane] = (uint8_t)end;
     if (lane == 0) const_cast<int32_t *>(a.nb_count)[i] = cnt;
 }
 
@@ -862,6 +738,17 @@ static size_t gather_smem_bytes(const lbmd_ctx *ctx, int warps) {
     return gather_occ_bytes(warps, active_words(ctx->p.nx)) + (size_t)warps * acc_words<fix>(ctx->p.nx) * sizeof(fix);
 }
 
+template <typename T, bool CLUSTER>
+static const void *phase_kernel(bool half, int cons) {
+    if (half)
+        return cons == 2   ? (const void *)team_phase_kernel<T, true, 2, CLUSTER>
+               : cons == 1 ? (const void *)team_phase_kernel<T, true, 1, CLUSTER>
+                           : (const void *)team_phase_kernel<T, true, 0, CLUSTER>;
+    return cons == 2   ? (const void *)team_phase_kernel<T, false, 2, CLUSTER>
+           : cons == 1 ? (const void *)team_phase_kernel<T, false, 1, CLUSTER>
+                       : (const void *)team_phase_kernel<T, false, 0, CLUSTER>;
+}
+
 // The row gather's shared memory grows with nx: as many warps per block (at
 // most GATHER_WARPS) as fit in 200 KB, and the opt-in above the default
 // 48 KB per block.
@@ -874,6 +761,36 @@ static cudaError_t setup_t(lbmd_ctx *ctx) {
     ctx->gather_warps = warps;
     cudaError_t e = cudaFuncSetAttribute(spread_rows_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
+    // threads of the team phase that are resident at once
+    int per_sm = 1 << 30;
+    for (int k = 0; k < 6; ++k) {
+        int n = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, phase_kernel<T, false>(k >= 3, k % 3), 2 * PHASE_THREADS, 0);
+        if (e != cudaSuccess) return e;
+        per_sm = std::min(per_sm, n);
+        e = cudaFuncSetAttribute(phase_kernel<T, true>(k >= 3, k % 3), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+    }
+    ctx->phase_threads = (int64_t)per_sm * ctx->sm_count * 2 * PHASE_THREADS;
+    // the largest cluster every form can run as
+    for (ctx->phase_cluster = PHASE_CLUSTER; ctx->phase_cluster > 1; ctx->phase_cluster /= 2) {
+        int least = 1;
+        for (int k = 0; k < 6; ++k) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)ctx->phase_cluster);
+            cfg.blockDim = dim3(PHASE_THREADS);
+            cudaLaunchAttribute at = {};
+            at.id = cudaLaunchAttributeClusterDimension;
+            at.val.clusterDim.x = (unsigned)ctx->phase_cluster;
+            at.val.clusterDim.y = at.val.clusterDim.z = 1;
+            cfg.attrs = &at;
+            cfg.numAttrs = 1;
+            int n = 0;
+            if ((e = cudaOccupancyMaxActiveClusters(&n, phase_kernel<T, true>(k >= 3, k % 3), &cfg)) != cudaSuccess) return e;
+            least = std::min(least, n);
+        }
+        if (least > 0) break;
+    }
     return md_tile_setup_kernels(ctx);
 }
 
@@ -910,6 +827,7 @@ static PArgs<T> make_pargs(lbmd_ctx *ctx, int substep) {
     const bool lists = ctx->lj_rc > 0.0 && ctx->nb_list;
     a.nb_list = lists ? ctx->nb_list : nullptr;
     a.nb_count = lists ? ctx->nb_count : nullptr;
+    a.nb_end = lists ? ctx->nb_end : nullptr;
     a.nb_invalid = lists ? ctx->nb_invalid : nullptr;
     a.nb_ref4 = lists ? static_cast<const typename P::real4 *>(ctx->nb_ref4) : nullptr;
     a.nb_half_skin2 = (T)(0.25 * LBMD_NB_SKIN * LBMD_NB_SKIN);
@@ -976,6 +894,41 @@ static cudaError_t md_phase_t(lbmd_ctx *ctx, int substep, int count, bool *done)
         else
             frozen_phase_kernel<T, false><<<blocks, 128, 0, ctx->stream>>>(a, count);
         return cudaGetLastError();
+    }
+    // Variants B and C, and conservative forces in any variant, while a team
+    // of lanes per particle fits the GPU at once.
+    if (ctx->p.spread == LBMD_SPREAD_AUTO || ctx->p.spread == LBMD_SPREAD_ATOMIC) {
+        const bool half = ctx->p.integrator == LBMD_INTEGRATOR_HALF_STEP;
+        const int cons = ctx->lj_rc > 0.0 ? 2 : has_cons(ctx) ? 1 : 0;
+        const int64_t threads = ctx->np * (cons == 2 ? 32 : 8);
+        if (threads <= ctx->phase_threads) {
+            PArgs<T> a = make_pargs<T>(ctx, substep);
+            GridBarrier words{ctx->phase_bar, ctx->dev_error};
+            void *args[] = {&a, &count, &words};
+            // one block per SM if that takes at most twice the threads each
+            const int per = threads > (int64_t)PHASE_THREADS * ctx->sm_count ? 2 * PHASE_THREADS : PHASE_THREADS;
+            unsigned blocks = (unsigned)((threads + per - 1) / per);
+            const bool cluster = blocks <= (unsigned)ctx->phase_cluster;
+            if (cluster)  // a power of two; teams beyond the particles idle
+                while (blocks & (blocks - 1)) ++blocks;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(blocks);
+            cfg.blockDim = dim3(per);
+            cfg.stream = ctx->stream;
+            cudaLaunchAttribute at = {};
+            if (cluster) {
+                at.id = cudaLaunchAttributeClusterDimension;
+                at.val.clusterDim.x = blocks;
+                at.val.clusterDim.y = at.val.clusterDim.z = 1;
+            } else {
+                at.id = cudaLaunchAttributeCooperative;
+                at.val.cooperative = 1;
+            }
+            cfg.attrs = &at;
+            cfg.numAttrs = 1;
+            return cudaLaunchKernelExC(&cfg, cluster ? phase_kernel<T, true>(half, cons) : phase_kernel<T, false>(half, cons),
+                                       args);
+        }
     }
     *done = false;
     return cudaSuccess;
@@ -1154,6 +1107,7 @@ cudaError_t launch_active_sync(lbmd_ctx *ctx) {
 }
 
 cudaError_t launch_md_steps(lbmd_ctx *ctx, int substep, int count) {
+    ctx->in_buckets = false;
     const bool dbl = ctx->p.precision == LBMD_FP64;
     bool done = false;
     cudaError_t e = dbl ? lbmd::md_phase_t<double>(ctx, substep, count, &done)
@@ -1163,7 +1117,14 @@ cudaError_t launch_md_steps(lbmd_ctx *ctx, int substep, int count) {
     return e;
 }
 
+// The conservative forces at the current positions; right after a re-ordering
+// the Lennard-Jones lists are built first (they are otherwise void until the
+// next LB step, and the pairs all pairs).
 cudaError_t launch_bond_forces_only(lbmd_ctx *ctx) {
+    if (ctx->in_buckets) {
+        const cudaError_t e = launch_nb_build(ctx);
+        if (e != cudaSuccess) return e;
+    }
     return ctx->p.precision == LBMD_FP64 ? lbmd::bond_forces_t<double>(ctx) : lbmd::bond_forces_t<float>(ctx);
 }
 
@@ -1176,5 +1137,6 @@ cudaError_t launch_nb_build(lbmd_ctx *ctx) {
 }
 
 cudaError_t launch_sort_particles(lbmd_ctx *ctx) {
+    ctx->in_buckets = true;
     return ctx->p.precision == LBMD_FP64 ? lbmd::sort_t<double>(ctx) : lbmd::sort_t<float>(ctx);
 }

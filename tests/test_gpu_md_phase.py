@@ -37,3 +37,41 @@ def test_variant_a_phase(precision, integrator, shape, n, m):
         want = _run(shape, n, kT_init, "eeee", spread="rows", **kw)
         for steps, spread in (("gggg", "auto"), ("gege", "auto"), ("egge", "atomic")):
             _same(_run(shape, n, kT_init, steps, spread=spread, **kw), want)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("integrator", ["start", "half_step"])
+@pytest.mark.parametrize("variant", ["B", "C"])
+@pytest.mark.parametrize("shape,n,m", [((7, 5, 6), 1, 3), ((40, 6, 5), 33, 4), ((20, 19, 18), 330, 3), ((33, 32, 31), 19000, 2)])
+def test_coupled_phase(precision, integrator, variant, shape, n, m):
+    # one block, a cluster of blocks (33 particles: one team in the second
+    # block), and more than one block of the larger size per SM
+    for kT_init in (1e-4, 0.2):
+        kw = dict(variant=variant, precision=precision, integrator=integrator, n_sub=m)
+        want = _run(shape, n, kT_init, "eee", spread="rows", **kw)
+        for steps, spread in (("ggg", "auto"), ("geg", "atomic")):
+            _same(_run(shape, n, kT_init, steps, spread=spread, **kw), want)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("integrator", ["start", "half_step"])
+@pytest.mark.parametrize("variant", ["A", "B", "C"])
+def test_coupled_phase_with_bonds(precision, integrator, variant):
+    # chains longer than a block, a particle with the largest number of
+    # bonds, and unbonded ones
+    shape, m = (16, 15, 14), 5
+    out = []
+    for spread, steps in (("rows", "eee"), ("auto", "ggg"), ("atomic", "egg")):
+        pos, bonds = inputs.bead_spring_chains(3, 150, shape, 5)
+        g = lbmd.LBMD(*shape, kT=1e-3, zeta=1.0, seed=11, max_particles=460, max_bonds=1000, variant=variant,
+                      precision=precision, integrator=integrator, n_sub=m, spread=spread)
+        g.add_particles(pos, inputs.maxwell_velocities(450, 1e-3, 5))
+        g.add_particles(inputs.uniform_positions(10, shape, 1), inputs.maxwell_velocities(10, 1e-3, 1))
+        g.add_bonds(bonds, 1.0, 1.0)
+        g.add_fene_bonds([(451, 452 + k) for k in range(8)], 0.5, 60.0)
+        for s in steps:
+            g.run_cycles(1) if s == "g" else g.cycle(1)
+        out.append((g.populations(), g.node_field(), *g.particles()))
+        g.close()
+    _same(out[1], out[0])
+    _same(out[2], out[0])
