@@ -500,8 +500,7 @@ static cudaError_t lb_step_t(lbmd_ctx *ctx) {
     a.fx = fixed_constants(ctx->fix.e, ctx->co.noise_amp, ctx->co.body_force);
     a.variant = ctx->p.variant;
     const dim3 block = node_block(ctx), grid = node_grid(ctx, block);
-    cudaError_t e = cudaMemsetAsync(ctx->lb_missed, 0, sizeof(int32_t), ctx->stream);
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     const bool full = ctx->co.gamma_bulk == 0.0 && ctx->co.gamma_ghost == 0.0;
     if (full)
         launch_collide<T, S, true>(ctx, a, grid, block);
@@ -555,10 +554,8 @@ static cudaError_t init_equilibrium_t(lbmd_ctx *ctx) {
 // step), then collide and stream with the post-stream moments fused in
 // (node field and the new active nodes' compact records).
 cudaError_t launch_lb_step(lbmd_ctx *ctx) {
-    cudaError_t e = launch_sort_particles(ctx);
+    cudaError_t e = launch_reorder(ctx);
     if (e != cudaSuccess) return e;
-    if ((e = launch_nb_build(ctx)) != cudaSuccess) return e;
-    if ((e = launch_active_set(ctx)) != cudaSuccess) return e;
     if ((e = md_tile_build_table(ctx, (int)((ctx->lb_step + 1) & 1))) != cudaSuccess) return e;
     if ((e = LBMD_DISPATCH_POPS(ctx, lbmd::lb_step_t, ctx)) != cudaSuccess) return e;
     ctx->cur ^= 1;

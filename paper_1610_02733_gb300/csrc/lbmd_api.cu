@@ -57,7 +57,7 @@ void free_all(lbmd_ctx *ctx) {
                     ctx->missed_total, ctx->dev_error,     ctx->arow[0],       ctx->arow[1],
                     ctx->tile_table[0], ctx->tile_table[1], ctx->edge_acc,  ctx->tile_flag,
                     ctx->late_rows,    ctx->late_count, ctx->ccw,          ctx->phase_bar,
-                    ctx->nb_end};
+                    ctx->nb_end,      ctx->active_count};
     for (void *b : bufs)
         if (b) cudaFree(b);
     for (int b = 0; b < 2; ++b) {
@@ -215,6 +215,7 @@ lbmd_status lbmd_create(const lbmd_params *p, lbmd_ctx **out) {
         {(void **)&ctx->slot_of, (size_t)maxp * sizeof(int32_t)},
         {(void **)&ctx->row_count, (size_t)p->ny * p->nz * sizeof(int32_t)},
         {(void **)&ctx->sort_rank, (size_t)maxp * sizeof(int32_t)},
+        {(void **)&ctx->active_count, (size_t)p->ny * p->nz * sizeof(int32_t)},
         {(void **)&ctx->chunk_total, (size_t)1024 * sizeof(int32_t)},
         {(void **)&ctx->row_start, ((size_t)p->ny * p->nz + 1) * sizeof(int32_t)},
         {(void **)&ctx->slot_row, (size_t)maxp * sizeof(int32_t)},
@@ -395,7 +396,7 @@ lbmd_status lbmd_add_particles(lbmd_ctx *ctx, int64_t n, const double *pos, cons
     // re-order now, so that every particle sits in the row bucket of its cell
     // (the MD kernels of variant B walk the buckets; the active nodes stay
     // those of the last LB step until the next one)
-    CK(ctx, launch_sort_particles(ctx));
+    CK(ctx, launch_bucket_particles(ctx));
     CK(ctx, md_tile_build_table(ctx, (int)(ctx->lb_step & 1)));
     if (has_cons(ctx)) CK(ctx, launch_bond_forces_only(ctx));
     CK(ctx, cudaStreamSynchronize(ctx->stream));
@@ -1055,7 +1056,7 @@ lbmd_status lbmd_load_state(lbmd_ctx *ctx, const void *buf, int64_t bytes) {
     CK(ctx, launch_node_moments(ctx, false));
     CK(ctx, launch_clear_transfer(ctx));
     // every particle into the row bucket of its cell (see lbmd_add_particles)
-    if (ctx->np > 0) CK(ctx, launch_sort_particles(ctx));
+    if (ctx->np > 0) CK(ctx, launch_bucket_particles(ctx));
     CK(ctx, md_tile_build_table(ctx, (int)(ctx->lb_step & 1)));
     if (ctx->np > 0 && has_cons(ctx)) CK(ctx, launch_bond_forces_only(ctx));
     CK(ctx, cudaStreamSynchronize(ctx->stream));

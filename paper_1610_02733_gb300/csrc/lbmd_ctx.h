@@ -124,6 +124,7 @@ struct lbmd_ctx {
     int32_t *slot_of;
     void *fc4[2], *old4;  // fc4 indexed by pcur: it carries the last F_c over steps (HALF_STEP)
     int32_t *row_count, *sort_rank, *chunk_total;
+    int32_t *active_count;  // active nodes per lattice row (re-ordering in one launch)
     int32_t *row_start;     // first slot of every cell row (ny*nz + 1 entries)
     int32_t *slot_row;      // per slot: the row bucket it belongs to, -1 if none
     int32_t *migrant_slot;  // variant B: slots that left their row bucket
@@ -281,8 +282,8 @@ cudaError_t launch_particles_from_double(lbmd_ctx *ctx, int64_t first, int64_t c
                                          bool set_mass);
 cudaError_t launch_particles_to_double(lbmd_ctx *ctx, double *pos, double *vel);
 cudaError_t launch_clear_transfer(lbmd_ctx *ctx);
-cudaError_t launch_sort_particles(lbmd_ctx *ctx);
-cudaError_t launch_active_set(lbmd_ctx *ctx);
+cudaError_t launch_bucket_particles(lbmd_ctx *ctx);
+cudaError_t launch_reorder(lbmd_ctx *ctx);
 cudaError_t launch_active_sync(lbmd_ctx *ctx);
 cudaError_t setup_particle_kernels(lbmd_ctx *ctx);
 // the tiled variant-B MD step (md_tile.cu)

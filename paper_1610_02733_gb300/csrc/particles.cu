@@ -515,18 +515,18 @@ __global__ void nb_validate_kernel(int32_t *invalid) { *invalid = 0; }
 // ---------------------------------------------------------------------------
 // Re-ordering by lattice row.
 // ---------------------------------------------------------------------------
-// Every particle's rank within its cell row and, with ccw, its cell marked in
-// the row's occupancy words.  The particles come mostly in row order (the
+// Every particle's rank within its cell row, and its cell marked in the row's
+// occupancy words.  The particles come mostly in row order (the
 // order of the last re-ordering), so the valid lanes of a warp form runs of
 // equal rows (and of equal occupancy words): each run takes its ranks with one
 // atomic on the row's count, and ORs its cells into a word with one atomic.
 // The order within a row is free: every later sum is order-independent.
+// (All lanes of a warp come here; those with p < np are a prefix of it.)
 template <typename T>
-__global__ void __launch_bounds__(256)
-    sort_count_kernel(const typename Prec<T>::real4 *pos4, int64_t np, FastDiv fnx, int32_t *row_count, int32_t *rank,
-                      uint32_t *ccw, int W) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const unsigned act = __ballot_sync(0xffffffffu, p < np);  // a prefix of the warp's lanes
+__device__ __forceinline__ void count_particle(const typename Prec<T>::real4 *pos4, int64_t p, int64_t np,
+                                               const FastDiv &fnx, int32_t *row_count, int32_t *rank, uint32_t *ccw,
+                                               int W) {
+    const unsigned act = __ballot_sync(0xffffffffu, p < np);
     if (p >= np) return;
     const int lane = (int)(threadIdx.x & 31), nvalid = __popc(act);
     const unsigned upto = 0xffffffffu >> (31 - lane);  // lanes 0..lane
@@ -542,27 +542,34 @@ __global__ void __launch_bounds__(256)
     if (lane == head) base = atomicAdd(&row_count[row], next - head);
     base = __shfl_sync(act, base, head);
     rank[p] = base + (lane - head);
-    if (ccw) {
-        const uint32_t cx = cell - row * fnx.d;
-        const unsigned long long key = (unsigned long long)row * (unsigned)W + (cx >> 5);
-        const unsigned long long key_prev = __shfl_up_sync(act, key, 1);
-        const unsigned kheads = __ballot_sync(act, lane == 0 || key_prev != key);
-        const unsigned kafter = kheads & ~upto;
-        const int knext = kafter ? __ffs((int)kafter) - 1 : nvalid;
-        // the run's cells ORed towards its first lane (segmented, log steps)
-        uint32_t bits = 1u << (cx & 31);
+    const uint32_t cx = cell - row * fnx.d;
+    const unsigned long long key = (unsigned long long)row * (unsigned)W + (cx >> 5);
+    const unsigned long long key_prev = __shfl_up_sync(act, key, 1);
+    const unsigned kheads = __ballot_sync(act, lane == 0 || key_prev != key);
+    const unsigned kafter = kheads & ~upto;
+    const int knext = kafter ? __ffs((int)kafter) - 1 : nvalid;
+    // the run's cells ORed towards its first lane (segmented, log steps)
+    uint32_t bits = 1u << (cx & 31);
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const uint32_t o = __shfl_down_sync(act, bits, off);
-            if (lane + off < knext) bits |= o;
-        }
-        if (kheads & (1u << lane)) atomicOr(&ccw[key], bits);
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t o = __shfl_down_sync(act, bits, off);
+        if (lane + off < knext) bits |= o;
     }
+    if (kheads & (1u << lane)) atomicOr(&ccw[key], bits);
 }
 
-// Block-wide exclusive scan of one value per thread (1024 threads).
+template <typename T>
+__global__ void __launch_bounds__(256)
+    sort_count_kernel(const typename Prec<T>::real4 *pos4, int64_t np, FastDiv fnx, int32_t *row_count, int32_t *rank,
+                      uint32_t *ccw, int W) {
+    count_particle<T>(pos4, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, np, fnx, row_count, rank, ccw, W);
+}
+
+// Block-wide exclusive scan of one value per thread (whole warps, up to 1024
+// threads).
 __device__ __forceinline__ int32_t block_exclusive_scan(int32_t v, int32_t *total) {
     __shared__ int32_t warp_sum[32];
+    const int warps = (int)(blockDim.x >> 5);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int32_t x = v;
 #pragma unroll
@@ -573,13 +580,13 @@ __device__ __forceinline__ int32_t block_exclusive_scan(int32_t v, int32_t *tota
     if (lane == 31) warp_sum[w] = x;
     __syncthreads();
     if (w == 0) {
-        int32_t s = warp_sum[lane];
+        int32_t s = lane < warps ? warp_sum[lane] : 0;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
             const int32_t y = __shfl_up_sync(0xffffffffu, s, off);
             if (lane >= off) s += y;
         }
-        warp_sum[lane] = s;  // inclusive prefix of warp sums
+        warp_sum[lane] = s;  // inclusive prefix of warp sums (the total beyond the last)
     }
     __syncthreads();
     const int32_t before = w > 0 ? warp_sum[w - 1] : 0;
@@ -615,26 +622,36 @@ __global__ void __launch_bounds__(1024) sort_finalize_kernel(const int32_t *row_
 // conservative force (if any) and its last coupling force (integrator
 // HALF_STEP, where it carries over to the next MD step).
 template <typename T>
-__global__ void __launch_bounds__(256)
-    sort_scatter_kernel(const typename Prec<T>::real4 *pos_in, const typename Prec<T>::real4 *vel_in,
-                        const typename Prec<T>::real4 *fcons_in, const typename Prec<T>::real4 *fc_in,
-                        const int32_t *pid_in, typename Prec<T>::real4 *pos_out, typename Prec<T>::real4 *vel_out,
-                        typename Prec<T>::real4 *fcons_out, typename Prec<T>::real4 *fc_out, int32_t *pid_out,
-                        int32_t *slot_of, int32_t *slot_row, const int32_t *row_start, const int32_t *rank, int64_t np,
-                        FastDiv fnx, int bonds, int carry_fc) {
+struct ScatterArgs {
+    using R4 = typename Prec<T>::real4;
+    const R4 *pos_in, *vel_in, *fcons_in, *fc_in;
+    const int32_t *pid_in;
+    R4 *pos_out, *vel_out, *fcons_out, *fc_out;
+    int32_t *pid_out, *slot_of, *slot_row;
+    int32_t *rank;
+    int64_t np;
+    FastDiv fnx;
+    int bonds, carry_fc;
+};
+template <typename T>
+__device__ __forceinline__ void scatter_particle(const ScatterArgs<T> &a, int64_t p, uint32_t row, int32_t dst) {
+    a.slot_row[dst] = (int32_t)row;
+    a.vel_out[dst] = a.vel_in[p];
+    if (a.bonds) a.fcons_out[dst] = a.fcons_in[p];
+    if (a.carry_fc) a.fc_out[dst] = a.fc_in[p];
+    const int32_t id = a.pid_in[p];
+    a.pid_out[dst] = id;
+    a.slot_of[id] = dst;
+}
+template <typename T>
+__global__ void __launch_bounds__(256) sort_scatter_kernel(ScatterArgs<T> a, const int32_t *row_start) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= np) return;
-    const typename Prec<T>::real4 R = pos_in[p];
-    const uint32_t row = fdiv((uint32_t)Prec<T>::cell_of(R), fnx);
-    const int32_t dst = row_start[row] + rank[p];
-    slot_row[dst] = (int32_t)row;
-    pos_out[dst] = R;
-    vel_out[dst] = vel_in[p];
-    if (bonds) fcons_out[dst] = fcons_in[p];
-    if (carry_fc) fc_out[dst] = fc_in[p];
-    const int32_t id = pid_in[p];
-    pid_out[dst] = id;
-    slot_of[id] = dst;
+    if (p >= a.np) return;
+    const typename Prec<T>::real4 R = a.pos_in[p];
+    const uint32_t row = fdiv((uint32_t)Prec<T>::cell_of(R), a.fnx);
+    const int32_t dst = row_start[row] + a.rank[p];
+    a.pos_out[dst] = R;
+    scatter_particle(a, p, row, dst);
 }
 
 // ---------------------------------------------------------------------------
@@ -646,13 +663,11 @@ __global__ void __launch_bounds__(256)
 // (L = min(32, W rounded up to a power of two)) builds one row's words from
 // the cell-occupancy words ccw, with the in-row slot of each word's first
 // active node (a scan over the group), and the row's count.
-__global__ void __launch_bounds__(256)
-    active_rows_kernel(const uint32_t *ccw, int nx, FastDiv fny, int nz, int W, int L, uint2 *occw, int32_t *row_count,
-                       int n_rows) {
-    const int lane = (int)(threadIdx.x & 31);
-    const int gwarp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const int nrow = gwarp * (32 / L) + lane / L, sub = lane % L;
-    const bool valid = nrow < n_rows;
+// (All lanes of a warp come here; valid: nrow is a row.)  Returns the row's
+// count, in every lane of the group.
+template <bool L2 = false>
+__device__ __forceinline__ int active_row(const uint32_t *ccw, int nx, const FastDiv &fny, int nz, int W, int L,
+                                          uint2 *occw, int nrow, int sub, bool valid) {
     const int ny = (int)fny.d;
     int cr[4] = {0, 0, 0, 0};
     if (valid) {
@@ -665,6 +680,7 @@ __global__ void __launch_bounds__(256)
     }
     const int last = nx - 1;
     const uint32_t tail_mask = (nx & 31) ? ((1u << (nx & 31)) - 1u) : 0xffffffffu;
+    auto word = [&](const uint32_t *p) { return L2 ? __ldcg(p) : *p; };
     int carry = 0;
     for (int w0 = 0; w0 < W; w0 += L) {  // uniform over the warp
         const int w = w0 + sub;
@@ -673,10 +689,10 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const uint32_t *cw = ccw + (size_t)cr[c] * W;
-                const uint32_t b = cw[w];
+                const uint32_t b = word(cw + w);
                 // cell x - 1 of bit x: the previous word's top bit, or (w = 0)
                 // the periodic neighbour x = nx - 1
-                const uint32_t in = w > 0 ? (cw[w - 1] >> 31) : ((cw[last >> 5] >> (last & 31)) & 1u);
+                const uint32_t in = w > 0 ? (word(cw + w - 1) >> 31) : ((word(cw + (last >> 5)) >> (last & 31)) & 1u);
                 a |= b | (b << 1) | in;
             }
             if (w == W - 1) a &= tail_mask;
@@ -691,7 +707,17 @@ __global__ void __launch_bounds__(256)
         if (valid && w < W) occw[(size_t)nrow * W + w] = make_uint2(a, (uint32_t)(carry + incl - cnt));
         carry += __shfl_sync(0xffffffffu, incl, L - 1, L);
     }
-    if (valid && sub == 0) row_count[nrow] = carry;
+    return carry;
+}
+__global__ void __launch_bounds__(256)
+    active_rows_kernel(const uint32_t *ccw, int nx, FastDiv fny, int nz, int W, int L, uint2 *occw, int32_t *row_count,
+                       int n_rows) {
+    const int lane = (int)(threadIdx.x & 31);
+    const int gwarp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int nrow = gwarp * (32 / L) + lane / L, sub = lane % L;
+    const bool valid = nrow < n_rows;
+    const int cnt = active_row(ccw, nx, fny, nz, W, L, occw, nrow, sub, valid);
+    if (valid && sub == 0) row_count[nrow] = cnt;
 }
 
 // Level 2 (after sort_chunk_scan_kernel turned the row counts into offsets
@@ -715,6 +741,76 @@ __global__ void __launch_bounds__(1024) active_finalize_kernel(const int32_t *ro
         if (i == row * W) arow[row] = (int32_t)b;  // the row's first compact slot
         if (row == n_rows - 1 && i == w_end - 1) arow[n_rows] = (int32_t)(wd.y + __popc(wd.x));  // closes the table
     }
+}
+
+// The re-ordering and the active set in one launch, for lattices of at most one
+// row per thread of the grid: the counting of the particles, the scan of the
+// rows with the marking of the active nodes, and the move of the particles with
+// the numbering of the nodes, between two grid barriers.  Block b takes the
+// rows [b per, (b + 1) per); for the scans it adds up the counts of all rows
+// before its own (at most 38,912 values out of L2).  row_count and ccw are zero
+// before and after.  As seven launches and two memsets the same took 23 us at
+// 64^3 nodes, where each of them is a launch's latency; this takes 9.
+constexpr int REORDER_THREADS = 256;
+
+// sum of v[0..n) over the block, read past L1
+__device__ __forceinline__ int32_t block_sum_before(const int32_t *v, int n) {
+    int32_t s = 0;
+    for (int i = (int)threadIdx.x; i < n; i += REORDER_THREADS) s += __ldcg(v + i);
+    int32_t total;
+    block_exclusive_scan(s, &total);
+    return total;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(REORDER_THREADS)
+    reorder_kernel(ScatterArgs<T> a, int32_t *row_count, int32_t *active_count, int32_t *row_start, uint32_t *ccw,
+                   uint2 *occw, int32_t *arow, int32_t *lb_missed, FastDiv fny, int nz, int W, int L, int per,
+                   GridBarrier words) {
+    PhaseBarrier<false> bar{words};
+    const int n_rows = (int)fny.d * nz, nx = (int)a.fnx.d;
+    const int64_t stride = (int64_t)gridDim.x * REORDER_THREADS, start = (int64_t)blockIdx.x * REORDER_THREADS;
+    const int tid = (int)threadIdx.x, lane = tid & 31;
+    for (int64_t b = start; b < a.np; b += stride)
+        count_particle<T>(a.pos_in, b + tid, a.np, a.fnx, row_count, a.rank, ccw, W);
+    if (blockIdx.x == 0 && tid == 0) *lb_missed = 0;
+    if (!bar.wait()) return;
+    const int r0 = min(n_rows, (int)blockIdx.x * per), r1 = min(n_rows, r0 + per), r = r0 + tid;
+    int32_t before = block_sum_before(row_count, r0);
+    const int32_t first = before + block_exclusive_scan(r < r1 ? __ldcg(row_count + r) : 0, nullptr);
+    if (r < r1) row_start[r] = first;
+    if (blockIdx.x == 0 && tid == 0) row_start[n_rows] = (int32_t)a.np;
+    const int rows_per_warp = 32 / L;
+    for (int q = r0 + (tid >> 5) * rows_per_warp; q < r1; q += (REORDER_THREADS / 32) * rows_per_warp) {
+        const int nrow = q + lane / L;
+        const bool valid = nrow < r1;
+        const int cnt = active_row<true>(ccw, nx, fny, nz, W, L, occw, nrow, lane % L, valid);
+        if (valid && lane % L == 0) active_count[nrow] = cnt;
+    }
+    if (!bar.wait()) return;
+    before = block_sum_before(active_count, r0);
+    const int32_t mine = r < r1 ? __ldcg(active_count + r) : 0;
+    __shared__ int32_t s_base[REORDER_THREADS];
+    s_base[tid] = before + block_exclusive_scan(mine, nullptr);
+    if (r < r1) {
+        arow[r] = s_base[tid];
+        if (r == n_rows - 1) arow[n_rows] = s_base[tid] + mine;
+        row_count[r] = 0;
+    }
+    __syncthreads();
+    for (int i = tid; i < (r1 - r0) * W; i += REORDER_THREADS) {
+        const size_t w = (size_t)r0 * W + i;
+        occw[w].y += (uint32_t)s_base[i / W];
+        ccw[w] = 0u;
+    }
+    for (int64_t p = start + tid; p < a.np; p += stride) {
+        const typename Prec<T>::real4 R = a.pos_in[p];
+        const uint32_t row = fdiv((uint32_t)Prec<T>::cell_of(R), a.fnx);
+        const int32_t dst = __ldcg(row_start + row) + a.rank[p];
+        a.pos_out[dst] = R;
+        scatter_particle(a, p, row, dst);
+    }
+    bar.finish();
 }
 
 // Node field entries of the active nodes brought up to date from their
@@ -761,21 +857,23 @@ static cudaError_t setup_t(lbmd_ctx *ctx) {
     ctx->gather_warps = warps;
     cudaError_t e = cudaFuncSetAttribute(spread_rows_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    // threads of the team phase that are resident at once
+    // threads of the team phase that are resident at once: the Lennard-Jones
+    // forms take the most registers and shared memory
     int per_sm = 1 << 30;
     for (int k = 0; k < 6; ++k) {
-        int n = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, phase_kernel<T, false>(k >= 3, k % 3), 2 * PHASE_THREADS, 0);
-        if (e != cudaSuccess) return e;
-        per_sm = std::min(per_sm, n);
         e = cudaFuncSetAttribute(phase_kernel<T, true>(k >= 3, k % 3), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
+        if (k % 3 != 2) continue;
+        int n = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, phase_kernel<T, false>(k >= 3, 2), 2 * PHASE_THREADS, 0);
+        if (e != cudaSuccess) return e;
+        per_sm = std::min(per_sm, n);
     }
     ctx->phase_threads = (int64_t)per_sm * ctx->sm_count * 2 * PHASE_THREADS;
     // the largest cluster every form can run as
     for (ctx->phase_cluster = PHASE_CLUSTER; ctx->phase_cluster > 1; ctx->phase_cluster /= 2) {
         int least = 1;
-        for (int k = 0; k < 6; ++k) {
+        for (int half = 0; half < 2; ++half) {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3((unsigned)ctx->phase_cluster);
             cfg.blockDim = dim3(PHASE_THREADS);
@@ -786,7 +884,8 @@ static cudaError_t setup_t(lbmd_ctx *ctx) {
             cfg.attrs = &at;
             cfg.numAttrs = 1;
             int n = 0;
-            if ((e = cudaOccupancyMaxActiveClusters(&n, phase_kernel<T, true>(k >= 3, k % 3), &cfg)) != cudaSuccess) return e;
+            if ((e = cudaOccupancyMaxActiveClusters(&n, phase_kernel<T, true>(half != 0, 2), &cfg)) != cudaSuccess)
+                return e;
             least = std::min(least, n);
         }
         if (least > 0) break;
@@ -1006,10 +1105,33 @@ static cudaError_t bond_forces_t(lbmd_ctx *ctx) {
 }
 
 template <typename T>
-static cudaError_t sort_t(lbmd_ctx *ctx) {
+static ScatterArgs<T> scatter_args(lbmd_ctx *ctx) {
     using R4 = typename Prec<T>::real4;
     const int b = ctx->pcur, o = b ^ 1;
     const int v = ctx->pv, vo = v ^ 1;  // position / velocity buffers
+    ScatterArgs<T> a;
+    a.pos_in = static_cast<const R4 *>(ctx->pos4[v]);
+    a.vel_in = static_cast<const R4 *>(ctx->vel4[v]);
+    a.fcons_in = static_cast<const R4 *>(ctx->fcons4[b]);
+    a.fc_in = static_cast<const R4 *>(ctx->fc4[b]);
+    a.pid_in = ctx->pid[b];
+    a.pos_out = static_cast<R4 *>(ctx->pos4[vo]);
+    a.vel_out = static_cast<R4 *>(ctx->vel4[vo]);
+    a.fcons_out = static_cast<R4 *>(ctx->fcons4[o]);
+    a.fc_out = static_cast<R4 *>(ctx->fc4[o]);
+    a.pid_out = ctx->pid[o];
+    a.slot_of = ctx->slot_of;
+    a.slot_row = ctx->slot_row;
+    a.rank = ctx->sort_rank;
+    a.np = ctx->np;
+    a.fnx = make_fastdiv((uint32_t)ctx->p.nx);
+    a.bonds = has_cons(ctx) ? 1 : 0;
+    a.carry_fc = ctx->p.integrator == LBMD_INTEGRATOR_HALF_STEP ? 1 : 0;
+    return a;
+}
+
+template <typename T>
+static cudaError_t sort_t(lbmd_ctx *ctx) {
     const int64_t rows = (int64_t)ctx->p.ny * ctx->p.nz;
     const int W = active_words(ctx->p.nx);
     cudaError_t e = cudaMemsetAsync(ctx->row_count, 0, (size_t)rows * sizeof(int32_t), ctx->stream);
@@ -1018,10 +1140,10 @@ static cudaError_t sort_t(lbmd_ctx *ctx) {
         (e = cudaMemsetAsync(ctx->ccw, 0, (size_t)rows * W * sizeof(uint32_t), ctx->stream)) != cudaSuccess)
         return e;
     if (ctx->np > 0) {
+        const ScatterArgs<T> a = scatter_args<T>(ctx);
         const unsigned blocks = (unsigned)((ctx->np + 255) / 256);
-        sort_count_kernel<T><<<blocks, 256, 0, ctx->stream>>>(static_cast<const R4 *>(ctx->pos4[v]), ctx->np,
-                                                                make_fastdiv((uint32_t)ctx->p.nx), ctx->row_count,
-                                                                ctx->sort_rank, ctx->ccw, W);
+        sort_count_kernel<T><<<blocks, 256, 0, ctx->stream>>>(a.pos_in, ctx->np, a.fnx, ctx->row_count, ctx->sort_rank,
+                                                                ctx->ccw, W);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         const int n_chunks = (int)((rows + 1023) / 1024);
         sort_chunk_scan_kernel<<<n_chunks, 1024, 0, ctx->stream>>>(ctx->row_count, rows, ctx->chunk_total);
@@ -1029,17 +1151,11 @@ static cudaError_t sort_t(lbmd_ctx *ctx) {
         sort_finalize_kernel<<<n_chunks, 1024, 0, ctx->stream>>>(ctx->row_count, ctx->chunk_total, rows,
                                                                  ctx->row_start, (int32_t)ctx->np);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        sort_scatter_kernel<T><<<blocks, 256, 0, ctx->stream>>>(
-            static_cast<const R4 *>(ctx->pos4[v]), static_cast<const R4 *>(ctx->vel4[v]),
-            static_cast<const R4 *>(ctx->fcons4[b]), static_cast<const R4 *>(ctx->fc4[b]), ctx->pid[b],
-            static_cast<R4 *>(ctx->pos4[vo]), static_cast<R4 *>(ctx->vel4[vo]), static_cast<R4 *>(ctx->fcons4[o]),
-            static_cast<R4 *>(ctx->fc4[o]), ctx->pid[o], ctx->slot_of, ctx->slot_row, ctx->row_start,
-            ctx->sort_rank, ctx->np, make_fastdiv((uint32_t)ctx->p.nx), has_cons(ctx) ? 1 : 0,
-            ctx->p.integrator == LBMD_INTEGRATOR_HALF_STEP ? 1 : 0);
+        sort_scatter_kernel<T><<<blocks, 256, 0, ctx->stream>>>(a, ctx->row_start);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    ctx->pcur = o;
-    ctx->pv = vo;
+    ctx->pcur ^= 1;
+    ctx->pv ^= 1;
     return cudaSuccess;
 }
 
@@ -1071,6 +1187,37 @@ static cudaError_t active_set_t(lbmd_ctx *ctx) {
     return cudaGetLastError();
 }
 
+// Re-ordering and active set of the coming cycle in one launch (reorder_kernel),
+// while a thread of the grid takes at most one row and 8 particles; larger
+// systems take the separate kernels, which fill the GPU.
+static bool reorder_fits(const lbmd_ctx *ctx) {
+    const int64_t threads = (int64_t)ctx->sm_count * REORDER_THREADS;
+    return ctx->np > 0 && (int64_t)ctx->p.ny * ctx->p.nz <= threads && ctx->np <= 8 * threads;
+}
+template <typename T>
+static cudaError_t reorder_t(lbmd_ctx *ctx) {
+    ScatterArgs<T> a = scatter_args<T>(ctx);
+    const int rows = ctx->p.ny * ctx->p.nz;
+    int W = active_words(ctx->p.nx), L = 1, nz = ctx->p.nz;
+    while (L < W && L < 32) L <<= 1;
+    const int64_t most = std::max<int64_t>(ctx->np, rows);
+    const unsigned blocks =
+        (unsigned)std::min<int64_t>(ctx->sm_count, (most + REORDER_THREADS - 1) / REORDER_THREADS);
+    int per = (rows + (int)blocks - 1) / (int)blocks;
+    uint2 *occw = active_words_next(ctx);
+    int32_t *arow = ctx->arow[(ctx->lb_step + 1) & 1];
+    FastDiv fny = make_fastdiv((uint32_t)ctx->p.ny);
+    GridBarrier words{ctx->phase_bar, ctx->dev_error};
+    void *args[] = {&a,    &ctx->row_count, &ctx->active_count, &ctx->row_start, &ctx->ccw, &occw, &arow,
+                    &ctx->lb_missed, &fny, &nz, &W, &L, &per, &words};
+    const cudaError_t e = cudaLaunchCooperativeKernel((const void *)reorder_kernel<T>, dim3(blocks),
+                                                      dim3(REORDER_THREADS), args, 0, ctx->stream);
+    if (e != cudaSuccess) return e;
+    ctx->pcur ^= 1;
+    ctx->pv ^= 1;
+    return cudaSuccess;
+}
+
 template <typename T>
 static cudaError_t active_sync_t(lbmd_ctx *ctx) {
     using N4 = typename Prec<T>::node4;
@@ -1097,8 +1244,22 @@ static cudaError_t nb_build_t(lbmd_ctx *ctx) {
 
 }  // namespace lbmd
 
-cudaError_t launch_active_set(lbmd_ctx *ctx) {
-    return ctx->p.precision == LBMD_FP64 ? lbmd::active_set_t<double>(ctx) : lbmd::active_set_t<float>(ctx);
+static cudaError_t launch_sort_particles(lbmd_ctx *ctx);
+
+// The particles in row order and the active nodes of the coming cycle; the list
+// of rows the collide leaves to its follow-up emptied.
+cudaError_t launch_reorder(lbmd_ctx *ctx) {
+    const bool dbl = ctx->p.precision == LBMD_FP64;
+    cudaError_t e;
+    if (lbmd::reorder_fits(ctx)) {
+        ctx->in_buckets = true;
+        if ((e = dbl ? lbmd::reorder_t<double>(ctx) : lbmd::reorder_t<float>(ctx)) != cudaSuccess) return e;
+        return launch_nb_build(ctx);
+    }
+    if ((e = launch_sort_particles(ctx)) != cudaSuccess) return e;
+    if ((e = launch_nb_build(ctx)) != cudaSuccess) return e;
+    if ((e = dbl ? lbmd::active_set_t<double>(ctx) : lbmd::active_set_t<float>(ctx)) != cudaSuccess) return e;
+    return cudaMemsetAsync(ctx->lb_missed, 0, sizeof(int32_t), ctx->stream);
 }
 
 cudaError_t launch_active_sync(lbmd_ctx *ctx) {
@@ -1136,7 +1297,18 @@ cudaError_t launch_nb_build(lbmd_ctx *ctx) {
     return ctx->p.precision == LBMD_FP64 ? lbmd::nb_build_t<double>(ctx) : lbmd::nb_build_t<float>(ctx);
 }
 
-cudaError_t launch_sort_particles(lbmd_ctx *ctx) {
+// The re-ordering alone; leaves the counting arrays dirty.
+static cudaError_t launch_sort_particles(lbmd_ctx *ctx) {
     ctx->in_buckets = true;
     return ctx->p.precision == LBMD_FP64 ? lbmd::sort_t<double>(ctx) : lbmd::sort_t<float>(ctx);
+}
+
+// Outside the cycles (particles added, a state loaded): every particle into the
+// row bucket of its cell, the counting arrays cleared for reorder_kernel.
+cudaError_t launch_bucket_particles(lbmd_ctx *ctx) {
+    cudaError_t e = launch_sort_particles(ctx);
+    if (e != cudaSuccess) return e;
+    const size_t rows = (size_t)ctx->p.ny * ctx->p.nz;
+    if ((e = cudaMemsetAsync(ctx->row_count, 0, rows * sizeof(int32_t), ctx->stream)) != cudaSuccess) return e;
+    return cudaMemsetAsync(ctx->ccw, 0, rows * lbmd::active_words(ctx->p.nx) * sizeof(uint32_t), ctx->stream);
 }
