@@ -43,6 +43,7 @@
 #include "lbmd_ctx.h"
 #include "lbmd_device.cuh"
 #include "particle_core.cuh"
+#include "phase_barrier.cuh"
 
 namespace lbmd {
 
@@ -410,6 +411,179 @@ __global__ void __launch_bounds__(128) ad_scatter_adj(AdArgs<T> a, AdRec<T> rec,
     atomic_addT(n + 3, s.w);
 }
 
+// The MD steps of a cycle, and their adjoints, in one launch each while 8 lanes
+// per particle fit the GPU at once: a handful of particles made every step two
+// launches of a few threads (8 + 3 us forward, 5 + 3 us adjoint).  Lane k of a
+// particle's team takes corner k; the blocks meet at a barrier after the nodes
+// are read and after they are updated.
+constexpr int AD_THREADS = 128;
+
+__device__ __forceinline__ int4 ad_load(const int4 *p) { return __ldcg(p); }
+__device__ __forceinline__ float4 ad_load(const float4 *p) { return __ldcg(p); }
+__device__ __forceinline__ L4 ad_load(const L4 *p) {
+    const longlong2 *q = reinterpret_cast<const longlong2 *>(p);
+    const longlong2 a = __ldcg(q), b = __ldcg(q + 1);
+    return L4{a.x, a.y, b.x, b.y};
+}
+__device__ __forceinline__ D4 ad_load(const D4 *p) {
+    const double2 *q = reinterpret_cast<const double2 *>(p);
+    const double2 a = __ldcg(q), b = __ldcg(q + 1);
+    return D4{a.x, a.y, b.x, b.y};
+}
+template <typename T>
+__device__ __forceinline__ T team_sum(T v) {
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off, 8);
+    return v;
+}
+
+template <typename T>
+struct AdCorner {
+    uint32_t node;
+    T w0, w1, w2;  // the corner's weight factors
+    __device__ __forceinline__ AdCorner(const AdArgs<T> &a, const CellXYZ &c, T fx, T fy, T fz, int k) {
+        const int ox = k & 1, oy = (k >> 1) & 1, oz = k >> 2;
+        const int x = ox ? (c.x + 1 == a.nx ? 0 : c.x + 1) : c.x;
+        const int y = oy ? (c.y + 1 == a.ny ? 0 : c.y + 1) : c.y;
+        const int z = oz ? (c.z + 1 == a.nz ? 0 : c.z + 1) : c.z;
+        node = (uint32_t)x + (uint32_t)a.nx * ((uint32_t)y + (uint32_t)a.ny * (uint32_t)z);
+        w0 = ox ? fx : T(1) - fx;
+        w1 = oy ? fy : T(1) - fy;
+        w2 = oz ? fz : T(1) - fz;
+    }
+};
+
+// The n_sub MD steps from pos_in, vel_in (as ad_couple and ad_transfer, sums
+// over the corners in the same order); drag: F_x per step and particle; rec:
+// with a record, its place for step 0 (the next ones follow).
+template <typename T, bool CLUSTER>
+__global__ void __launch_bounds__(AD_THREADS)
+    ad_md_phase(AdArgs<T> a, const typename Prec<T>::real4 *pos_in, const typename Prec<T>::real4 *vel_in,
+                typename Prec<T>::real4 *pos_out, typename Prec<T>::real4 *vel_out, typename Prec<T>::node4 *node,
+                T *drag, typename Prec<T>::real4 *rec, uint32_t step0, GridBarrier words) {
+    using P = Prec<T>;
+    PhaseBarrier<CLUSTER> bar{words};
+    const int t = blockIdx.x * AD_THREADS + threadIdx.x, k = (int)threadIdx.x & 7;
+    const bool live = (t >> 3) < a.np;
+    const int p = live ? t >> 3 : 0;
+    typename P::real4 R = pos_in[p], V = vel_in[p];
+    CellXYZ c = cell_xyz(P::cell_of(R), a.fd_nx, a.fd_ny);
+    T fx = R.x, fy = R.y, fz = R.z;
+    const T hm = a.half_dt * V.w;
+    for (int s = 0; s < a.n_sub; ++s) {
+        const AdCorner<T> q(a, c, fx, fy, fz, k);
+        const typename P::node4 n = ad_load(&node[q.node]);
+        const T rho = P::rho_of(n), jx = P::from_fix(P::jx_of(n), a.fis), jy = P::from_fix(P::jy_of(n), a.fis),
+                jz = P::from_fix(P::jz_of(n), a.fis);
+        const T delta = q.w0 * q.w1 * q.w2, w = delta / rho;
+        T ux = T(0), uy = T(0), uz = T(0);
+#pragma unroll
+        for (int h = 0; h < 8; ++h) {
+            const T wh = __shfl_sync(0xffffffffu, w, h, 8);
+            ux = fma(wh, __shfl_sync(0xffffffffu, jx, h, 8), ux);
+            uy = fma(wh, __shfl_sync(0xffffffffu, jy, h, 8), uy);
+            uz = fma(wh, __shfl_sync(0xffffffffu, jz, h, 8), uz);
+        }
+        T Fx = -a.zeta * (V.x - ux), Fy = -a.zeta * (V.y - uy), Fz = -a.zeta * (V.z - uz);
+        if (a.amp != T(0)) {
+            const U4 rnd = philox4x32_10(U4{(uint32_t)p, step0 + (uint32_t)s, 1u, 0u}, a.key0, a.key1);
+            Fx = fma(a.amp, unit_uniform<T>(rnd.x), Fx);
+            Fy = fma(a.amp, unit_uniform<T>(rnd.y), Fy);
+            Fz = fma(a.amp, unit_uniform<T>(rnd.z), Fz);
+        }
+        if (live) {
+            if (k == 0) drag[(size_t)s * a.np + p] = Fx;
+            if (rec) {
+                typename P::real4 *r = rec + (size_t)s * a.np * 12;
+                if (k == 0) r[p] = P::make_pos(fx, fy, fz, c.x + (int64_t)a.nx * (c.y + (int64_t)a.ny * c.z));
+                if (k == 1) r[a.np + p] = V;
+                if (k == 2) r[2 * a.np + p] = P::make4(Fx, Fy, Fz, T(0));
+                if (k == 3) r[3 * a.np + p] = P::make4(ux, uy, uz, T(0));
+                r[4 * a.np + 8 * (size_t)p + k] = P::make4(rho, jx, jy, jz);
+            }
+        }
+        V.x = fma(hm, Fx, V.x);
+        V.y = fma(hm, Fy, V.y);
+        V.z = fma(hm, Fz, V.z);
+        advance(fx, c.x, a.dt, V.x, a.nx);
+        advance(fy, c.y, a.dt, V.y, a.ny);
+        advance(fz, c.z, a.dt, V.z, a.nz);
+        V.x = fma(hm, Fx, V.x);
+        V.y = fma(hm, Fy, V.y);
+        V.z = fma(hm, Fz, V.z);
+        if (!bar.wait()) return;  // every particle has read the nodes
+        if (live)
+            P::add_transfer(&node[q.node], P::to_fix_neg(delta, Fx * a.neg_scale_dt),
+                            P::to_fix_neg(delta, Fy * a.neg_scale_dt), P::to_fix_neg(delta, Fz * a.neg_scale_dt));
+        if (s + 1 < a.n_sub && !bar.wait()) return;  // all transfers are in
+    }
+    bar.finish();
+    if (!live || k != 0) return;
+    pos_out[p] = P::make_pos(fx, fy, fz, c.x + (int64_t)a.nx * (c.y + (int64_t)a.ny * c.z));
+    vel_out[p] = V;
+}
+
+// The adjoints of the n_sub MD steps, last first (as ad_particle_adj and
+// ad_scatter_adj; sums over the corners by a butterfly).
+template <typename T, bool CLUSTER>
+__global__ void __launch_bounds__(AD_THREADS)
+    ad_adjoint_phase(AdArgs<T> a, const typename Prec<T>::real4 *rec, typename Prec<T>::real4 *nbar,
+                     typename Prec<T>::real4 *Rbar, typename Prec<T>::real4 *vbar, T *zbar, GridBarrier words) {
+    using P = Prec<T>;
+    PhaseBarrier<CLUSTER> bar{words};
+    const int t = blockIdx.x * AD_THREADS + threadIdx.x, k = (int)threadIdx.x & 7;
+    const bool live = (t >> 3) < a.np;
+    const int p = live ? t >> 3 : 0;
+    typename P::real4 xb = Rbar[p], vb = vbar[p];
+    const T dt = a.dt;
+    for (int s = a.n_sub - 1; s >= 0; --s) {
+        const typename P::real4 *r = rec + (size_t)s * a.np * 12;
+        const typename P::real4 R = r[p], V = r[a.np + p], F = r[2 * a.np + p], U = r[3 * a.np + p];
+        const typename P::real4 ck = r[4 * a.np + 8 * (size_t)p + k];
+        const CellXYZ c = cell_xyz(P::cell_of(R), a.fd_nx, a.fd_ny);
+        const AdCorner<T> q(a, c, R.x, R.y, R.z, k);
+        const typename P::real4 nb = ad_load(&nbar[q.node]);
+        const T delta = q.w0 * q.w1 * q.w2, im = V.w, dd = dt * delta;
+        // F-bar: through v' = v + (dt/m) F, x' = x + dt v + dt^2/(2m) F, the
+        // transfers -dt delta_k F and the drag term of the loss
+        const T Fb[3] = {im * dt * vb.x + a.half_dt * im * dt * xb.x + a.norm - team_sum(dd * nb.y),
+                         im * dt * vb.y + a.half_dt * im * dt * xb.y - team_sum(dd * nb.z),
+                         im * dt * vb.z + a.half_dt * im * dt * xb.z - team_sum(dd * nb.w)};
+        // positions: gradient of the weights delta_k(d) within the cell
+        const T s0 = (k & 1) ? T(1) : T(-1), s1 = (k & 2) ? T(1) : T(-1), s2 = (k & 4) ? T(1) : T(-1);
+        const T irk = T(1) / ck.x;
+        const T uF = (ck.y * Fb[0] + ck.z * Fb[1] + ck.w * Fb[2]) * irk;  // u_k . F-bar
+        const T coef = a.zeta * uF - dt * (F.x * nb.y + F.y * nb.z + F.z * nb.w);
+        const T gx = xb.x + team_sum(coef * s0 * q.w1 * q.w2), gy = xb.y + team_sum(coef * q.w0 * s1 * q.w2),
+                gz = xb.z + team_sum(coef * q.w0 * q.w1 * s2);
+        if (live && k == 0) {
+            // zeta: F = -zeta (v - u) + sqrt(zeta) (...) xi
+            const T Fr[3] = {F.x + a.zeta * (V.x - U.x), F.y + a.zeta * (V.y - U.y), F.z + a.zeta * (V.z - U.z)};
+            T zb = -(Fb[0] * (V.x - U.x) + Fb[1] * (V.y - U.y) + Fb[2] * (V.z - U.z));
+            if (a.zeta > T(0)) zb += (Fb[0] * Fr[0] + Fb[1] * Fr[1] + Fb[2] * Fr[2]) / (T(2) * a.zeta);
+            zbar[(size_t)s * a.np + p] = zb;
+        }
+        vb = P::make4(vb.x + dt * xb.x - a.zeta * Fb[0], vb.y + dt * xb.y - a.zeta * Fb[1],
+                      vb.z + dt * xb.z - a.zeta * Fb[2], T(0));
+        xb = P::make4(gx, gy, gz, T(0));
+        if (!bar.wait()) return;  // every particle has read the node adjoints
+        if (live) {
+            // j_k gets zeta delta_k / rho_k F-bar, rho_k -zeta delta_k (u_k . F-bar) / rho_k
+            const T sk = a.zeta * delta * irk;
+            T *n = reinterpret_cast<T *>(&nbar[q.node]);
+            atomic_addT(n + 0, -sk * uF);
+            atomic_addT(n + 1, sk * Fb[0]);
+            atomic_addT(n + 2, sk * Fb[1]);
+            atomic_addT(n + 3, sk * Fb[2]);
+        }
+        if (s > 0 && !bar.wait()) return;  // all of this step's are in
+    }
+    bar.finish();
+    if (!live || k != 0) return;
+    Rbar[p] = xb;
+    vbar[p] = vb;
+}
+
 template <typename T>
 __global__ void ad_particles_from_double(typename Prec<T>::real4 *pos4, typename Prec<T>::real4 *vel4,
                                          const double *pos, const double *vel, int np, int nx, int ny, int nz) {
@@ -462,6 +636,9 @@ struct lbmd_adjoint {
     void *zbar = nullptr;                    // K m np
     double *staging = nullptr;               // host-conversion scratch, 8 K m np doubles or more
     int64_t staging_len = 0;
+    uint32_t *phase_words = nullptr;         // grid barrier of the phases (2 words), then its error flag
+    int64_t phase_threads = 0;               // threads of a phase resident at once
+    int phase_cluster = 1;                   // largest cluster of its blocks
     std::string err;
 };
 
@@ -491,7 +668,7 @@ lbmd_status afail(lbmd_adjoint *a, lbmd_status s, const std::string &msg) {
 void free_ad(lbmd_adjoint *a) {
     void *bufs[] = {a->fchk, a->pchk, a->pos,  a->vel,  a->old,  a->fc,  a->node,    a->drag,    a->rec,
                     a->fbar[0], a->fbar[1], a->nbar[0], a->nbar[1], a->Rbar, a->vbar, a->scat, a->zbar,
-                    a->staging};
+                    a->staging, a->phase_words};
     for (void *b : bufs)
         if (b) cudaFree(b);
     if (a->own_stream && a->stream) cudaStreamDestroy(a->stream);
@@ -558,8 +735,35 @@ typename Prec<T>::real4 *pchk_at(const lbmd_adjoint *ad, int c) {
 
 unsigned nb(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
+bool in_phases(const lbmd_adjoint *ad) {
+    return ad->p.n_particles > 0 && 8ll * ad->p.n_particles <= ad->phase_threads;
+}
+
+template <typename T>
+cudaError_t launch_ad(const lbmd_adjoint *ad, const void *cluster_kernel, const void *grid_kernel, void **args) {
+    return launch_phase(cluster_kernel, grid_kernel, nb(8ll * ad->p.n_particles, AD_THREADS), AD_THREADS,
+                        ad->phase_cluster, args, ad->stream);
+}
+
+// how many threads, and blocks as a cluster, of a phase run at once
+template <typename T>
+cudaError_t setup_phases(lbmd_adjoint *ad) {
+    int dev = 0, sms = 1, md = 0, adj = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&md, ad_md_phase<T, false>, AD_THREADS, 0);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&adj, ad_adjoint_phase<T, false>, AD_THREADS, 0);
+    ad->phase_threads = (int64_t)std::min(md, adj) * sms * AD_THREADS;
+    ad->phase_cluster = 16;
+    if (e == cudaSuccess) e = limit_cluster((const void *)ad_md_phase<T, true>, AD_THREADS, ad->phase_cluster);
+    if (e == cudaSuccess) e = limit_cluster((const void *)ad_adjoint_phase<T, true>, AD_THREADS, ad->phase_cluster);
+    return e;
+}
+
 // one cycle's MD steps from the checkpoint of cycle c (node field from the
-// checkpointed populations), optionally recording every MD step
+// checkpointed populations), optionally recording every MD step; the particles
+// end in the checkpoint of cycle c + 1, where its recomputation leaves the same
 template <typename T>
 cudaError_t run_md(lbmd_adjoint *ad, int c, bool record) {
     using R4 = typename Prec<T>::real4;
@@ -571,7 +775,18 @@ cudaError_t run_md(lbmd_adjoint *ad, int c, bool record) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (np == 0) return cudaSuccess;
-    R4 *ck = pchk_at<T>(ad, c);
+    R4 *ck = pchk_at<T>(ad, c), *next = pchk_at<T>(ad, c + 1);
+    if (in_phases(ad)) {
+        AdArgs<T> args_a = a;
+        const R4 *pos_in = ck, *vel_in = ck + np;
+        R4 *pos_out = next, *vel_out = next + np, *rec = record ? static_cast<R4 *>(ad->rec) : nullptr;
+        N4 *node = static_cast<N4 *>(ad->node);
+        T *drag = static_cast<T *>(ad->drag) + (size_t)c * m * np;
+        uint32_t step0 = (uint32_t)(c * m);
+        GridBarrier words{ad->phase_words, reinterpret_cast<int32_t *>(ad->phase_words + 2)};
+        void *args[] = {&args_a, &pos_in, &vel_in, &pos_out, &vel_out, &node, &drag, &rec, &step0, &words};
+        return launch_ad<T>(ad, (const void *)ad_md_phase<T, true>, (const void *)ad_md_phase<T, false>, args);
+    }
     if ((e = cudaMemcpyAsync(ad->pos, ck, np * sizeof(R4), cudaMemcpyDeviceToDevice, ad->stream)) != cudaSuccess)
         return e;
     if ((e = cudaMemcpyAsync(ad->vel, ck + np, np * sizeof(R4), cudaMemcpyDeviceToDevice, ad->stream)) != cudaSuccess)
@@ -588,7 +803,19 @@ cudaError_t run_md(lbmd_adjoint *ad, int c, bool record) {
                                                             static_cast<N4 *>(ad->node));
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    return cudaSuccess;
+    if ((e = cudaMemcpyAsync(next, ad->pos, np * sizeof(R4), cudaMemcpyDeviceToDevice, ad->stream)) != cudaSuccess)
+        return e;
+    return cudaMemcpyAsync(next + np, ad->vel, np * sizeof(R4), cudaMemcpyDeviceToDevice, ad->stream);
+}
+
+// A wait of a phase that gave up (see PhaseBarrier) since the last check;
+// synchronises.
+cudaError_t check_phases(lbmd_adjoint *ad) {
+    int32_t gave_up = 0;
+    cudaError_t e = cudaMemcpyAsync(&gave_up, ad->phase_words + 2, sizeof(gave_up), cudaMemcpyDeviceToHost, ad->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ad->stream);
+    if (e == cudaSuccess && gave_up) e = cudaErrorLaunchTimeout;
+    return e;
 }
 
 template <typename T>
@@ -614,15 +841,6 @@ cudaError_t forward_t(lbmd_adjoint *ad, const double *pos0, const double *vel0, 
     const bool full = ad->co.gamma_bulk == 0.0 && ad->co.gamma_ghost == 0.0;
     for (int c = 0; c < K; ++c) {
         if ((e = run_md<T>(ad, c, false)) != cudaSuccess) return e;
-        if (np > 0) {
-            R4 *nx = pchk_at<T>(ad, c + 1);
-            if ((e = cudaMemcpyAsync(nx, ad->pos, np * sizeof(R4), cudaMemcpyDeviceToDevice, ad->stream)) !=
-                cudaSuccess)
-                return e;
-            if ((e = cudaMemcpyAsync(nx + np, ad->vel, np * sizeof(R4), cudaMemcpyDeviceToDevice, ad->stream)) !=
-                cudaSuccess)
-                return e;
-        }
         if (full)
             ad_collide_push<T, true><<<nb(ad->N, 256), 256, 0, ad->stream>>>(
                 fchk_at<T>(ad, c), fchk_at<T>(ad, c + 1), static_cast<N4 *>(ad->node), a, (uint32_t)c);
@@ -641,7 +859,7 @@ cudaError_t forward_t(lbmd_adjoint *ad, const double *pos0, const double *vel0, 
         if ((e = cudaMemcpyAsync(h.data(), ad->staging, nd * sizeof(double), cudaMemcpyDeviceToHost, ad->stream)) !=
             cudaSuccess)
             return e;
-        if ((e = cudaStreamSynchronize(ad->stream)) != cudaSuccess) return e;
+        if ((e = check_phases(ad)) != cudaSuccess) return e;
         for (int64_t i = 0; i < nd; ++i) L += h[i];
         L /= (double)nd;
     } else if ((e = cudaStreamSynchronize(ad->stream)) != cudaSuccess) {
@@ -674,7 +892,18 @@ cudaError_t backward_t(lbmd_adjoint *ad, double *dzeta, double *dpos) {
             static_cast<R4 *>(ad->nbar[cur]), static_cast<T *>(ad->fbar[o]), static_cast<R4 *>(ad->nbar[o]), a,
             (uint32_t)c);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        for (int s = m - 1; s >= 0 && np > 0; --s) {
+        if (in_phases(ad)) {
+            AdArgs<T> args_a = a;
+            const R4 *rec = static_cast<const R4 *>(ad->rec);
+            R4 *nbar = static_cast<R4 *>(ad->nbar[o]), *Rbar = static_cast<R4 *>(ad->Rbar),
+               *vbar = static_cast<R4 *>(ad->vbar);
+            T *zb = static_cast<T *>(ad->zbar) + (size_t)c * m * np;
+            GridBarrier words{ad->phase_words, reinterpret_cast<int32_t *>(ad->phase_words + 2)};
+            void *args[] = {&args_a, &rec, &nbar, &Rbar, &vbar, &zb, &words};
+            e = launch_ad<T>(ad, (const void *)ad_adjoint_phase<T, true>, (const void *)ad_adjoint_phase<T, false>, args);
+            if (e != cudaSuccess) return e;
+        }
+        for (int s = m - 1; s >= 0 && np > 0 && !in_phases(ad); --s) {
             AdRec<T> r = rec_at<T>(ad, s);
             T *zb = static_cast<T *>(ad->zbar) + ((size_t)c * m + s) * np;
             ad_particle_adj<T><<<nb(np, 128), 128, 0, ad->stream>>>(a, r, static_cast<R4 *>(ad->nbar[o]),
@@ -705,7 +934,7 @@ cudaError_t backward_t(lbmd_adjoint *ad, double *dzeta, double *dpos) {
             cudaSuccess)
             return e;
     }
-    if ((e = cudaStreamSynchronize(ad->stream)) != cudaSuccess) return e;
+    if ((e = check_phases(ad)) != cudaSuccess) return e;
     double z = 0.0;
     for (int64_t i = 0; i < nz; ++i) z += hz[i];
     *dzeta = z;
@@ -770,6 +999,7 @@ lbmd_status lbmd_adjoint_create(const lbmd_adjoint_params *p, lbmd_adjoint **out
         {&a->fbar[1], 19 * N * rs}, {&a->nbar[0], N * r4}, {&a->nbar[1], N * r4}, {&a->Rbar, np * r4},
         {&a->vbar, np * r4}, {&a->scat, 8 * np * r4}, {&a->zbar, K * m * np * rs},
         {(void **)&a->staging, (size_t)a->staging_len * sizeof(double)},
+        {(void **)&a->phase_words, 3 * sizeof(uint32_t)},
     };
     for (auto &x : allocs) {
         cudaError_t e = cudaMalloc(x.ptr, x.bytes);
@@ -779,6 +1009,13 @@ lbmd_status lbmd_adjoint_create(const lbmd_adjoint_params *p, lbmd_adjoint **out
             return afail(nullptr, e == cudaErrorMemoryAllocation ? LBMD_ERR_OOM : LBMD_ERR_CUDA,
                          std::string("cudaMalloc: ") + cudaGetErrorString(e));
         }
+    }
+    cudaError_t e = cudaMemsetAsync(a->phase_words, 0, 3 * sizeof(uint32_t), a->stream);
+    if (e == cudaSuccess) e = p->precision == LBMD_FP64 ? setup_phases<double>(a) : setup_phases<float>(a);
+    if (e != cudaSuccess) {
+        free_ad(a);
+        delete a;
+        return afail(nullptr, LBMD_ERR_CUDA, std::string("adjoint phases: ") + cudaGetErrorString(e));
     }
     *out = a;
     return LBMD_OK;

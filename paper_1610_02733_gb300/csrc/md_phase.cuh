@@ -23,6 +23,7 @@
 #include "lbmd_device.cuh"
 #include "particle_core.cuh"
 #include "particle_step.cuh"
+#include "phase_barrier.cuh"
 
 namespace lbmd {
 
@@ -195,62 +196,6 @@ __device__ __forceinline__ void bond_forces(const PArgs<T> &a, int64_t id, const
         Fz = fma(g, dz, Fz);
     }
 }
-
-// Barrier of all blocks of a launch whose blocks are resident together.  Up to
-// 16 blocks form one thread-block cluster and use its hardware barrier (0.25 us;
-// 1.1 us with a load and an atomic of each thread in flight).  More blocks are a
-// cooperative launch and count their arrivals in one word, which only grows
-// during the launch (1.2 us / 1.8 us at 128 blocks of 256 threads; a count that
-// the last block clears beside a generation word took 2.2 / 2.9 us).  The last
-// block to finish clears the word for the next launch.  The wait is bounded
-// (the blocks arrive within microseconds; 2^22 polls are seconds): a block that
-// gives up sets the context's device error flag, and the kernel ends.
-struct GridBarrier {
-    uint32_t *word;  // arrivals, finished blocks
-    int32_t *error;
-};
-template <bool CLUSTER>
-struct PhaseBarrier {
-    GridBarrier g;
-    uint32_t target = 0;
-    __device__ __forceinline__ bool wait() {
-        if (gridDim.x == 1) {
-            __syncthreads();
-            return true;
-        }
-        if (CLUSTER) {
-            asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-            return true;
-        }
-        target += gridDim.x;
-        bool ok = true;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            uint32_t v;
-            asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(v) : "l"(g.word) : "memory");
-            ++v;
-            int polls = 0;
-            while ((int32_t)(v - target) < 0) {
-                if (++polls > (1 << 22)) {
-                    atomicExch(g.error, 1);
-                    ok = false;
-                    break;
-                }
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(g.word) : "memory");
-            }
-        }
-        return __syncthreads_and(ok) != 0;
-    }
-    // the block's last act
-    __device__ __forceinline__ void finish() {
-        if (CLUSTER || gridDim.x == 1) return;
-        __syncthreads();
-        if (threadIdx.x == 0 && atomicAdd(g.word + 1, 1u) == gridDim.x - 1) {
-            g.word[0] = 0u;
-            g.word[1] = 0u;
-        }
-    }
-};
 
 // Lennard-Jones force on the particle at (R, c) from the one at S, if within the
 // cut-off; explicit FMAs, so that every path rounds alike.

@@ -871,25 +871,10 @@ static cudaError_t setup_t(lbmd_ctx *ctx) {
     }
     ctx->phase_threads = (int64_t)per_sm * ctx->sm_count * 2 * PHASE_THREADS;
     // the largest cluster every form can run as
-    for (ctx->phase_cluster = PHASE_CLUSTER; ctx->phase_cluster > 1; ctx->phase_cluster /= 2) {
-        int least = 1;
-        for (int half = 0; half < 2; ++half) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3((unsigned)ctx->phase_cluster);
-            cfg.blockDim = dim3(PHASE_THREADS);
-            cudaLaunchAttribute at = {};
-            at.id = cudaLaunchAttributeClusterDimension;
-            at.val.clusterDim.x = (unsigned)ctx->phase_cluster;
-            at.val.clusterDim.y = at.val.clusterDim.z = 1;
-            cfg.attrs = &at;
-            cfg.numAttrs = 1;
-            int n = 0;
-            if ((e = cudaOccupancyMaxActiveClusters(&n, phase_kernel<T, true>(half != 0, 2), &cfg)) != cudaSuccess)
-                return e;
-            least = std::min(least, n);
-        }
-        if (least > 0) break;
-    }
+    ctx->phase_cluster = PHASE_CLUSTER;
+    for (int half = 0; half < 2; ++half)
+        if ((e = limit_cluster(phase_kernel<T, true>(half != 0, 2), PHASE_THREADS, ctx->phase_cluster)) != cudaSuccess)
+            return e;
     return md_tile_setup_kernels(ctx);
 }
 
@@ -1006,27 +991,8 @@ static cudaError_t md_phase_t(lbmd_ctx *ctx, int substep, int count, bool *done)
             void *args[] = {&a, &count, &words};
             // one block per SM if that takes at most twice the threads each
             const int per = threads > (int64_t)PHASE_THREADS * ctx->sm_count ? 2 * PHASE_THREADS : PHASE_THREADS;
-            unsigned blocks = (unsigned)((threads + per - 1) / per);
-            const bool cluster = blocks <= (unsigned)ctx->phase_cluster;
-            if (cluster)  // a power of two; teams beyond the particles idle
-                while (blocks & (blocks - 1)) ++blocks;
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(blocks);
-            cfg.blockDim = dim3(per);
-            cfg.stream = ctx->stream;
-            cudaLaunchAttribute at = {};
-            if (cluster) {
-                at.id = cudaLaunchAttributeClusterDimension;
-                at.val.clusterDim.x = blocks;
-                at.val.clusterDim.y = at.val.clusterDim.z = 1;
-            } else {
-                at.id = cudaLaunchAttributeCooperative;
-                at.val.cooperative = 1;
-            }
-            cfg.attrs = &at;
-            cfg.numAttrs = 1;
-            return cudaLaunchKernelExC(&cfg, cluster ? phase_kernel<T, true>(half, cons) : phase_kernel<T, false>(half, cons),
-                                       args);
+            return launch_phase(phase_kernel<T, true>(half, cons), phase_kernel<T, false>(half, cons),
+                                (unsigned)((threads + per - 1) / per), per, ctx->phase_cluster, args, ctx->stream);
         }
     }
     *done = false;

@@ -97,3 +97,23 @@ def test_torch_autograd_function():
     assert float(loss.detach()) == L
     assert float(zeta.grad) == pytest.approx(2.0 * dz, rel=1e-14)
     assert np.allclose(R0.grad.numpy(), 2.0 * dpos, rtol=1e-14, atol=0)
+
+
+@pytest.mark.parametrize("n,zeta", [(1, 1.5), (16, 1.5), (17, 1.5), (300, 0.5), (60000, 0.002)])
+def test_adjoint_by_number_of_particles(n, zeta):
+    # one block, a cluster of blocks, a grid of them, and more particles than
+    # the steps of a cycle in one launch take
+    shape, n_sub, cycles = (12, 10, 8), 3, 2
+    pos, vel = _particles(n, shape, 4, 2e-3)
+    ad = lbmd.Adjoint(*shape, n_particles=n, n_cycles=cycles, n_sub=n_sub, precision="fp64", kT=1e-4,
+                      body_force=BODY, seed=5)
+    for _ in range(2):  # the barrier's words are left as they were found
+        L = ad.forward(zeta, pos, vel)
+        dz, dpos = ad.backward()
+    Lo, dzo = _tangent(shape, n_sub, cycles, zeta, 1e-4, pos, vel, dzeta=1.0)
+    scale = float(np.abs(vel).mean()) * zeta  # of the drags the mean is taken of
+    assert abs(L - Lo) <= 1e-12 * max(abs(Lo), scale)
+    assert abs(dz - dzo) <= 1e-9 * max(abs(dzo), scale / zeta)
+    e = inputs.uniform(pos.shape, -1.0, 1.0, 21)
+    _, de = _tangent(shape, n_sub, cycles, zeta, 1e-4, pos, vel, dpos=e)
+    assert abs(float((dpos * e).sum()) - de) <= 1e-9 * float(np.abs(dpos * e).sum())
