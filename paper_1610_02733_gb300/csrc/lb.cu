@@ -312,15 +312,18 @@ __device__ __forceinline__ void collide_push_node(const LbArgs<T, S> &a, int x, 
     }
 }
 
-// Resident blocks per SM the compiler plans registers for: 7 (32 registers)
-// for the forms with full relaxation, uniform noise and FP32 or
-// rounded-to-nearest 16-bit storage, measured faster than 6 (40 registers)
-// despite their spills: FP32 cycle -0.8 %, FP16 / BF16 LB step -6.5 % /
-// -4.3 %; the stochastic-rounding form measured slower at 7, and it and the
-// Gaussian-noise and partial-relaxation forms keep 6 (3 in FP64).
+// Resident blocks per SM the compiler plans registers for.  FP32 storage: 6 (40
+// registers; two cycles at 256^3 with 10^6 particles 3396 us, 5 blocks 3461,
+// 7 blocks, with spills, 3482).  Rounded-to-nearest 16-bit storage with full
+// relaxation and uniform noise: 7 (3183 us, 6 blocks 3287); the stochastic
+// rounding form measured slower at 7.  Variant C 5.  FP64: 2 with the
+// collision in integers (128 registers), 3 in its FP64 form.
 template <typename T, typename S, bool RELAX_FULL, bool GAUSS, bool C>
 constexpr int collide_min_blocks() {
-    return sizeof(T) == 8 ? (RELAX_FULL ? 2 : 3) : C ? 5 : (RELAX_FULL && !GAUSS && !PopStore<S, T>::stochastic ? 7 : 6);
+    return sizeof(T) == 8                                                              ? (RELAX_FULL ? 2 : 3)
+           : C                                                                         ? 5
+           : RELAX_FULL && PopStore<S, T>::deviation && !PopStore<S, T>::stochastic ? 7
+                                                                                       : 6;
 }
 
 template <typename T, typename S, bool RELAX_FULL, bool GAUSS, bool C>

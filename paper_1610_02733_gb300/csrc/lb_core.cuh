@@ -24,12 +24,22 @@ constexpr bool inv_bnorm_matches() {
 static_assert(inv_bnorm_matches(), "INV_BNORM(k) must be 1 / BNORM(k)");
 
 // The D3Q19 order pairs every moving velocity with its opposite:
-// c_{2p+2} = -c_{2p+1}, p = 0..8.  Even modes (0, 4-9, 16-18) see only the
-// pair sums s_p = f_{2p+1} + f_{2p+2}, odd modes (1-3, 10-15) only the
-// differences d_p = f_{2p+1} - f_{2p+2}; the back-transform likewise returns
-// an even part E_p and an odd part O_p with f_{2p+1} = w (E_p + O_p) and
-// f_{2p+2} = w (E_p - O_p).  This halves the arithmetic of both transforms.
-__host__ __device__ constexpr bool EVEN_MODE(int k) { return k == 0 || (k >= 4 && k <= 9) || k >= 16; }
+// c_{2p+2} = -c_{2p+1}, p = 0..8 (x, y, z, then the diagonals of the xy, xz and
+// yz planes, two each).  Even modes (0, 4-9, 16-18) see only the pair sums s_p,
+// odd modes (1-3, 10-15) only the differences d_p; the back-transform likewise
+// returns an even part E and an odd part O with f_{2p+1} = E + O and f_{2p+2} =
+// E - O.  Within each, the three axes and the three planes share their sums.
+template <typename T>
+struct PairSums {
+    T s[9], d[9];
+    __device__ __forceinline__ explicit PairSums(const T f[Q]) {
+#pragma unroll
+        for (int p = 0; p < 9; ++p) {
+            s[p] = f[2 * p + 1] + f[2 * p + 2];
+            d[p] = f[2 * p + 1] - f[2 * p + 2];
+        }
+    }
+};
 
 // MRT collision with forcing and noise at one node; f holds f* on entry and
 // f' on exit -- or, for a deviation storage form, f* - b and f' - b with b the
@@ -96,76 +106,92 @@ __device__ __forceinline__ void apply_transfer(T f[Q], T rho, T jx, T jy, T jz, 
     }
 }
 
+// (2h + 1) - 65536 for a 16-bit h, the low (high = 0) or the high half of a
+// word, exactly: twice h - 32767.5.  FP32 builds 2^23 + 2h + 1 from its bit
+// pattern (no int-to-float conversion) and subtracts once; FP64 goes through
+// its fields.
+__device__ __forceinline__ float centred16x2(uint32_t word, int high, float) {
+    const uint32_t t = high ? word >> 15 : word << 1;
+    return __uint_as_float((t & 0x1fffeu) | 0x4B000001u) - 8454144.0f;
+}
+__device__ __forceinline__ double centred16x2(uint32_t word, int high, double) {
+    const uint32_t h = high ? word >> 16 : word & 0xffffu;
+    return from_fixed((long long)(2u * h) - 65535ll, 0);
+}
+
 // RELAX_FULL: gamma_bulk = gamma_ghost = 0 (the default reading), so the
 // bulk and ghost modes relax fully, m'_k = m^eq_k exactly, and their moments
-// m_k need not be computed (gamma (m - m^eq) is +-0 for finite m).
+// m_k are not needed.
 // A: any struct with the members gamma_bulk, gamma_shear, gamma_ghost,
 // amp16[Q] and noisy (the single-box, batched and adjoint kernels), and for
 // GAUSS (normal variates) ampg[Q]; the Philox key (key0, key1) and counters
 // (node, step) come as arguments.
+//
+// The kernels that call this issue instructions about as fast as they move
+// bytes, so the operations are counted: ~250 besides the noise bits, against
+// ~430 when every mode and every population was summed on its own.  The
+// stress terms (1 - gamma) rho u u + (1 + gamma) (u F + F u)/2 are u q + q u with
+// q = (1 - gamma) rho u/2 + (1 + gamma) F/2; the 1/b_k and weights are constants of the
+// back-transform.  The rest weight is taken as 1 - 24/36 of what the moving
+// populations got, so that the weights add up to one whatever their rounding.
+// Explicit multiply-adds: every kernel rounds alike.
 template <typename T, bool RELAX_FULL, typename A, bool GAUSS = false>
 __device__ __forceinline__ void collide(T f[Q], T rho, T rho_m, T jx, T jy, T jz, T Fx, T Fy, T Fz, const A &a,
                                         uint32_t key0, uint32_t key1, uint32_t node, uint32_t step) {
     T inv_rho, sr;
     rho_factors(rho, inv_rho, sr);
-    const T ux = (jx + T(0.5) * Fx) * inv_rho;
-    const T uy = (jy + T(0.5) * Fy) * inv_rho;
-    const T uz = (jz + T(0.5) * Fz) * inv_rho;
-    const T uu = ux * ux + uy * uy + uz * uz;
-    const T uF = ux * Fx + uy * Fy + uz * Fz;
+    const T ux = fma(T(0.5), Fx, jx) * inv_rho;
+    const T uy = fma(T(0.5), Fy, jy) * inv_rho;
+    const T uz = fma(T(0.5), Fz, jz) * inv_rho;
+    const T cu = (T(0.5) - T(0.5) * a.gamma_shear) * rho, cf = T(0.5) + T(0.5) * a.gamma_shear;
+    const T qx = fma(cu, ux, cf * Fx), qy = fma(cu, uy, cf * Fy), qz = fma(cu, uz, cf * Fz);
+    const T bu = RELAX_FULL ? rho : rho - a.gamma_bulk * rho, bf = RELAX_FULL ? T(1) : T(1) + a.gamma_bulk;
+    const T bx = fma(bu, ux, RELAX_FULL ? Fx : bf * Fx), by = fma(bu, uy, RELAX_FULL ? Fy : bf * Fy),
+            bz = fma(bu, uz, RELAX_FULL ? Fz : bf * Fz);
 
-    T s[9], d[9];
-#pragma unroll
-    for (int p = 0; p < 9; ++p) {
-        s[p] = f[2 * p + 1] + f[2 * p + 2];
-        d[p] = f[2 * p + 1] - f[2 * p + 2];
-    }
-    // non-conserved moments m_k = sum_i e_k(c_i) f_i, k = 4..18
+    // post-collision modes 4..18: equilibrium and forcing, what is left of the
+    // moments m_k = sum_i e_k(c_i) f_i, noise
     T m[Q];
-#pragma unroll
-    for (int k = 4; k < Q; ++k) {
-        T acc = T(0);
-        if (EVEN_MODE(k) && EMODE(k, 0) != 0) acc = T(EMODE(k, 0)) * f[0];
-#pragma unroll
-        for (int p = 0; p < 9; ++p) {
-            const int e = EMODE(k, 2 * p + 1);
-            if (e != 0) acc += T(e) * (EVEN_MODE(k) ? s[p] : d[p]);
-        }
-        m[k] = acc;
+    m[4] = fma(uz, bz, fma(uy, by, ux * bx));
+    {
+        const T txx = T(2) * (ux * qx), tyy = T(2) * (uy * qy), tzz = T(2) * (uz * qz);
+        m[5] = fma(T(2), txx, -(tyy + tzz));
+        m[6] = tyy - tzz;
+        m[7] = fma(ux, qy, uy * qx);
+        m[8] = fma(ux, qz, uz * qx);
+        m[9] = fma(uy, qz, uz * qy);
     }
-    // equilibria of the stress modes (ghost equilibria vanish)
-    T meq[Q];
+    {
+        const PairSums<T> v(f);
+        const T *s = v.s, *d = v.d;
+        const T sxy = s[3] + s[4], sxz = s[5] + s[6], syz = s[7] + s[8];
+        const T a5 = fma(T(2), s[0], -(s[1] + s[2])), g5 = fma(T(-2), syz, sxy + sxz);
+        const T a6 = s[1] - s[2], g6 = sxy - sxz;
+        const T gs = a.gamma_shear;
+        m[5] = fma(gs, a5 + g5, m[5]);
+        m[6] = fma(gs, a6 + g6, m[6]);
+        m[7] = fma(gs, s[3] - s[4], m[7]);
+        m[8] = fma(gs, s[5] - s[6], m[8]);
+        m[9] = fma(gs, s[7] - s[8], m[9]);
+        if constexpr (RELAX_FULL) {
 #pragma unroll
-    for (int k = 0; k < Q; ++k) meq[k] = T(0);
-    meq[4] = rho * uu;
-    meq[5] = rho * (T(3) * ux * ux - uu);
-    meq[6] = rho * (uy * uy - uz * uz);
-    meq[7] = rho * ux * uy;
-    meq[8] = rho * ux * uz;
-    meq[9] = rho * uy * uz;
-
-    T mp[Q];
-    mp[0] = rho_m;
-    mp[1] = jx + Fx;
-    mp[2] = jy + Fy;
-    mp[3] = jz + Fz;
-#pragma unroll
-    for (int k = 4; k < Q; ++k) {
-        if (RELAX_FULL && (k == 4 || k >= 10)) {
-            mp[k] = meq[k];
-            continue;
+            for (int k = 10; k < Q; ++k) m[k] = T(0);
+        } else {
+            const T gg = a.gamma_ghost, A3 = (s[0] + s[1]) + s[2], G = (sxy + sxz) + syz;
+            m[4] = fma(a.gamma_bulk, G - f[0], m[4]);
+            const T xy_x = d[3] + d[4], xy_y = d[3] - d[4], xz_x = d[5] + d[6], xz_z = d[5] - d[6],
+                    yz_y = d[7] + d[8], yz_z = d[7] - d[8];
+            m[10] = gg * fma(T(-2), d[0], xy_x + xz_x);
+            m[11] = gg * fma(T(-2), d[1], xy_y + yz_y);
+            m[12] = gg * fma(T(-2), d[2], xz_z + yz_z);
+            m[13] = gg * (xy_x - xz_x);
+            m[14] = gg * (yz_y - xy_y);
+            m[15] = gg * (xz_z - yz_z);
+            m[16] = gg * (fma(T(-2), A3, f[0]) + G);
+            m[17] = gg * (g5 - a5);
+            m[18] = gg * (g6 - a6);
         }
-        const T gk = k == 4 ? a.gamma_bulk : (k <= 9 ? a.gamma_shear : a.gamma_ghost);
-        mp[k] = meq[k] + gk * (m[k] - meq[k]);
     }
-    const T fb = T(1) + a.gamma_bulk, fs = T(1) + a.gamma_shear;
-    mp[4] += fb * uF;
-    mp[5] += fs * (T(3) * ux * Fx - uF);
-    mp[6] += fs * (uy * Fy - uz * Fz);
-    mp[7] += fs * T(0.5) * (ux * Fy + uy * Fx);
-    mp[8] += fs * T(0.5) * (ux * Fz + uz * Fx);
-    mp[9] += fs * T(0.5) * (uy * Fz + uz * Fy);
-
     if constexpr (GAUSS) {
         if (a.noisy) {
             // 15 normal variates from four Philox calls, a Box-Muller pair
@@ -179,7 +205,7 @@ __device__ __forceinline__ void collide(T f[Q], T rho, T rho_m, T jx, T jy, T jz
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
                     const int k = 4 + 4 * (int)q + t;
-                    if (k < Q) mp[k] += (a.ampg[k] * sr) * g[t];
+                    if (k < Q) m[k] = fma(a.ampg[k] * sr, g[t], m[k]);
                 }
             }
         }
@@ -187,7 +213,15 @@ __device__ __forceinline__ void collide(T f[Q], T rho, T rho_m, T jx, T jy, T jz
         // 15 variates from two Philox calls: two 16-bit halves per 32-bit
         // word, low half first, in mode order k = 4..18.  The variate
         // sqrt(12) ((h + 1/2) 2^-16 - 1/2) is (h - 32767.5) times
-        // sqrt(12) 2^-16, folded into amp16[k] = amp[k] sqrt(12) 2^-16.
+        // sqrt(12) 2^-16, folded into amp16[k] = amp[k] sqrt(12) 2^-16, the
+        // same for the modes of a class (7-9, 10-12, 13-15).
+        const T half = T(0.5) * sr;
+        T amp[Q];
+#pragma unroll
+        for (int k = 4; k < Q; ++k) {
+            const bool same = k == 8 || k == 9 || k == 11 || k == 12 || k == 14 || k == 15;
+            amp[k] = same ? amp[k - 1] : a.amp16[k] * half;
+        }
 #pragma unroll
         for (uint32_t q = 0; q < 2; ++q) {
             const U4 r = philox4x32_10(U4{node, step, 0u, q}, key0, key1);
@@ -195,35 +229,46 @@ __device__ __forceinline__ void collide(T f[Q], T rho, T rho_m, T jx, T jy, T jz
 #pragma unroll
             for (int t = 0; t < 8; ++t) {
                 const int k = 4 + 8 * (int)q + t;
-                const uint32_t h = (t & 1) ? (bits[t >> 1] >> 16) : (bits[t >> 1] & 0xffffu);
-                if (k < Q) mp[k] += (a.amp16[k] * sr) * centred16(h, T(0));
+                if (k < Q) m[k] = fma(amp[k], centred16x2(bits[t >> 1], t & 1, T(0)), m[k]);
             }
         }
     }
-#pragma unroll
-    for (int k = 0; k < Q; ++k) mp[k] *= T(INV_BNORM(k));
+    m[1] = jx + Fx;
+    m[2] = jy + Fy;
+    m[3] = jz + Fz;
+    // back-transform f_i = w_i sum_k e_k(c_i) m_k / b_k
+    const T r36 = rho_m * T(1.0 / 36.0), r18 = r36 + r36, r0 = fma(T(-24), r36, rho_m);
+    f[0] = fma(m[16], T(1.0 / 6.0), fma(m[4], T(-0.5), r0));
     {
-        T acc = T(0);
+        const T base = fma(m[16], T(-1.0 / 18.0), r18), e5 = m[5] - m[17], e6 = m[6] - m[18];
+        const T side = fma(e5, T(-0.75 / 18.0), base);
+        const T E[3] = {fma(e5, T(1.5 / 18.0), base), fma(e6, T(2.25 / 18.0), side), fma(e6, T(-2.25 / 18.0), side)};
 #pragma unroll
-        for (int k = 0; k < Q; ++k)
-            if (EVEN_MODE(k) && EMODE(k, 0) != 0) acc += T(EMODE(k, 0)) * mp[k];
-        f[0] = T(WEIGHT(0)) * acc;
-    }
-#pragma unroll
-    for (int p = 0; p < 9; ++p) {
-        T ev = T(0), od = T(0);
-#pragma unroll
-        for (int k = 0; k < Q; ++k) {
-            const int e = EMODE(k, 2 * p + 1);
-            if (e == 0) continue;
-            if (EVEN_MODE(k))
-                ev += T(e) * mp[k];
-            else
-                od += T(e) * mp[k];
+        for (int c = 0; c < 3; ++c) {
+            const T o = m[1 + c] - m[10 + c];
+            f[2 * c + 1] = fma(o, T(3.0 / 18.0), E[c]);
+            f[2 * c + 2] = fma(o, T(-3.0 / 18.0), E[c]);
         }
-        const T w = T(WEIGHT(2 * p + 1));
-        f[2 * p + 1] = w * (ev + od);
-        f[2 * p + 2] = w * (ev - od);
+    }
+    {
+        const T base = fma(m[16], T(0.5 / 36.0), fma(m[4], T(1.5 / 36.0), r36)), e5 = m[5] + m[17], e6 = m[6] + m[18];
+        const T side = fma(e5, T(0.75 / 36.0), base);
+        const T E[3] = {fma(e6, T(2.25 / 36.0), side), fma(e6, T(-2.25 / 36.0), side), fma(e5, T(-1.5 / 36.0), base)};
+        T X[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) X[c] = fma(m[10 + c], T(1.5 / 36.0), m[1 + c] * T(3.0 / 36.0));
+        const T k = T(4.5 / 36.0);
+        const T first[3] = {fma(m[13], k, X[0]), fma(m[13], -k, X[0]), fma(m[14], k, X[1])};
+        const T second[3] = {fma(m[14], -k, X[1]), fma(m[15], k, X[2]), fma(m[15], -k, X[2])};
+#pragma unroll
+        for (int p = 0; p < 3; ++p) {  // xy, xz, yz
+            const T ep = fma(m[7 + p], T(9.0 / 36.0), E[p]), em = fma(m[7 + p], T(-9.0 / 36.0), E[p]);
+            const T op = first[p] + second[p], om = first[p] - second[p];
+            f[7 + 4 * p] = ep + op;
+            f[8 + 4 * p] = ep - op;
+            f[9 + 4 * p] = em + om;
+            f[10 + 4 * p] = em - om;
+        }
     }
 }
 

@@ -492,12 +492,16 @@ struct PopStore<bf16_sr, float> {
 // values are bitwise identical wherever they are recomputed.
 template <typename T>
 __device__ __forceinline__ void node_moments(const T f[Q], T &rho, T &jx, T &jy, T &jz) {
-    rho = f[0];
+    T s[9], d[9];  // sums and differences of opposite velocities
 #pragma unroll
-    for (int i = 1; i < Q; ++i) rho += f[i];
-    jx = (f[1] - f[2]) + (f[7] - f[8]) + (f[9] - f[10]) + (f[11] - f[12]) + (f[13] - f[14]);
-    jy = (f[3] - f[4]) + (f[7] - f[8]) + (f[10] - f[9]) + (f[15] - f[16]) + (f[17] - f[18]);
-    jz = (f[5] - f[6]) + (f[11] - f[12]) + (f[14] - f[13]) + (f[15] - f[16]) + (f[18] - f[17]);
+    for (int p = 0; p < 9; ++p) {
+        s[p] = f[2 * p + 1] + f[2 * p + 2];
+        d[p] = f[2 * p + 1] - f[2 * p + 2];
+    }
+    rho = f[0] + (((s[0] + s[1]) + s[2]) + (((s[3] + s[4]) + (s[5] + s[6])) + (s[7] + s[8])));
+    jx = d[0] + ((d[3] + d[4]) + (d[5] + d[6]));
+    jy = d[1] + ((d[3] - d[4]) + (d[7] + d[8]));
+    jz = d[2] + ((d[5] - d[6]) + (d[7] - d[8]));
 }
 
 // The same from the values the arithmetic works on (PopStore::arith): rho_m

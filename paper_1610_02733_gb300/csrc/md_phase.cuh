@@ -147,36 +147,70 @@ __device__ __forceinline__ float quiet_nan<float>() { return __int_as_float(0x7f
 template <>
 __device__ __forceinline__ double quiet_nan<double>() { return __longlong_as_double(0x7ff8000000000000LL); }
 
-// Bond force on a particle from a partner at minimum-image separation d
-// (partner minus particle), |d|^2 = r2: g d with
-//   harmonic U = (k/2)(r - r0)^2               g = k (r - r0) / r   (0 at r = 0)
-//   FENE     U = -(k/2) R0^2 ln(1 - (r/R0)^2)  g = k / (1 - (r/R0)^2), R0 = r0
-// (Kremer-Grest springs, Sec. 4); a FENE bond at r >= R0 gives NaN.
+// Separation of a bond partner (partner minus particle, minimum image): the
+// rounded components and what the rounding left out.
 template <typename T>
-__device__ __forceinline__ T bond_gain(uint8_t kind, T k, T r0, T r2) {
-    if (kind == LBMD_BOND_FENE) {
-        const T x = r2 / (r0 * r0);
-        return x < T(1) ? k / (T(1) - x) : quiet_nan<T>();
-    }
-    const T r = sqrt(r2);
-    return r > T(0) ? k * (r - r0) / r : T(0);
+struct Separation {
+    T x, y, z, lx, ly, lz;
+};
+
+// a - b and a + b with their rounding errors (Knuth's two-sum)
+template <typename T>
+__device__ __forceinline__ T two_sum(T a, T b, T &err) {
+    const T s = a + b, t = s - a;
+    err = (a - (s - t)) + (b - t);
+    return s;
 }
 
-// Minimum-image separation of the partner in slot q from a particle at
-// (R, c), through the stored cell indices and offsets.
-// L2: the partner's position was written during the launch.
+// One component: d whole cells plus the difference of the offsets.  The image is
+// taken off the whole cells: off the rounded sum it would cost a bond across
+// the periodic boundary the last bits of the box length.
+template <typename T>
+__device__ __forceinline__ T separation_component(int d, T there, T here, int n, T &lo) {
+    T l1, l2;
+    const T f = two_sum(there, -here, l1);
+    d -= n * (int)rint((T(d) + f) / T(n));
+    const T x = two_sum(T(d), f, l2);
+    lo = l1 + l2;
+    return x;
+}
+
+// Through the stored cell indices and offsets, for the partner in slot q of a
+// particle at (R, c).  L2: the partner's position was written during the launch.
 template <bool L2 = false, typename T>
-__device__ __forceinline__ void bond_separation(const PArgs<T> &a, const typename Prec<T>::real4 &R, const CellXYZ &c,
-                                                int64_t q, T &dx, T &dy, T &dz) {
+__device__ __forceinline__ Separation<T> bond_separation(const PArgs<T> &a, const typename Prec<T>::real4 &R,
+                                                         const CellXYZ &c, int64_t q) {
     using P = Prec<T>;
     const typename P::real4 S = L2 ? load_l2(&a.pos4[q]) : a.pos4[q];
     const CellXYZ d = cell_xyz(P::cell_of(S), a.fd_nx, a.fd_ny);
-    dx = T(d.x - c.x) + (S.x - R.x);
-    dy = T(d.y - c.y) + (S.y - R.y);
-    dz = T(d.z - c.z) + (S.z - R.z);
-    dx -= T(a.nx) * rint(dx / T(a.nx));
-    dy -= T(a.ny) * rint(dy / T(a.ny));
-    dz -= T(a.nz) * rint(dz / T(a.nz));
+    Separation<T> v;
+    v.x = separation_component(d.x - c.x, S.x, R.x, a.nx, v.lx);
+    v.y = separation_component(d.y - c.y, S.y, R.y, a.ny, v.ly);
+    v.z = separation_component(d.z - c.z, S.z, R.z, a.nz, v.lz);
+    return v;
+}
+
+// Bond force g d on a particle from a partner at separation d, |d| = r, with
+//   harmonic U = (k/2)(r - r0)^2               g = k (r - r0) / r   (0 at r = 0)
+//   FENE     U = -(k/2) R0^2 ln(1 - (r/R0)^2)  g = k / (1 - (r/R0)^2), R0 = r0
+// (Kremer-Grest springs, Sec. 4); a FENE bond at r >= R0 gives NaN.  The
+// harmonic one, stiff and near r0, takes r - r0 = (r^2 - r0^2) / (r + r0) with the
+// squares' and sums' rounding errors carried along.
+template <typename T>
+__device__ __forceinline__ T bond_gain(uint8_t kind, T k, T r0, const Separation<T> &d) {
+    const T px = d.x * d.x, py = d.y * d.y, pz = d.z * d.z;
+    if (kind == LBMD_BOND_FENE) {
+        const T x = fma(d.z, d.z, fma(d.y, d.y, px)) / (r0 * r0);
+        return x < T(1) ? k / (T(1) - x) : quiet_nan<T>();
+    }
+    const T p0 = r0 * r0;
+    T e1, e2, e3;
+    const T s = two_sum(two_sum(two_sum(px, -p0, e1), py, e2), pz, e3);
+    const T small = fma(T(2) * d.x, d.lx, fma(T(2) * d.y, d.ly, (T(2) * d.z) * d.lz));
+    const T squares = (fma(d.x, d.x, -px) + fma(d.y, d.y, -py)) + (fma(d.z, d.z, -pz) - fma(r0, r0, -p0));
+    const T e = s + ((((e1 + e2) + e3) + squares) + small);  // r^2 - r0^2
+    const T r = sqrt(fma(d.z, d.z, fma(d.y, d.y, px)));
+    return r > T(0) ? k * e / (r * (r + r0)) : T(0);
 }
 
 // Bond forces on particle `id` at (R, c), summed over its partners in a fixed
@@ -188,12 +222,11 @@ __device__ __forceinline__ void bond_forces(const PArgs<T> &a, int64_t id, const
     const int nbond = a.bond_count[id];
     for (int b = 0; b < nbond; ++b) {
         const int64_t e = id * LBMD_MAX_BONDS_PER_PARTICLE + b;
-        T dx, dy, dz;
-        bond_separation<L2>(a, R, c, a.slot_of[a.bond_partner[e]], dx, dy, dz);
-        const T g = bond_gain(a.bond_kind[e], (T)a.bond_k[e], (T)a.bond_r0[e], dx * dx + dy * dy + dz * dz);
-        Fx = fma(g, dx, Fx);
-        Fy = fma(g, dy, Fy);
-        Fz = fma(g, dz, Fz);
+        const Separation<T> d = bond_separation<L2>(a, R, c, a.slot_of[a.bond_partner[e]]);
+        const T g = bond_gain(a.bond_kind[e], (T)a.bond_k[e], (T)a.bond_r0[e], d);
+        Fx = fma(g, d.x, Fx);
+        Fy = fma(g, d.y, Fy);
+        Fz = fma(g, d.z, Fz);
     }
 }
 
@@ -409,8 +442,11 @@ __global__ void __launch_bounds__(2 * PHASE_THREADS, sizeof(T) == 4 ? 2 : 1)
             const typename P::real4 R = P::make_pos(fx, fy, fz, 0);
             T g = T(0), dx = T(0), dy = T(0), dz = T(0);
             if (lane < nbond) {
-                bond_separation<true>(a, R, c, partner, dx, dy, dz);
-                g = bond_gain(kind, bond_k, bond_r0, dx * dx + dy * dy + dz * dz);
+                const Separation<T> d = bond_separation<true>(a, R, c, partner);
+                dx = d.x;
+                dy = d.y;
+                dz = d.z;
+                g = bond_gain(kind, bond_k, bond_r0, d);
             }
             Bx = By = Bz = T(0);
             if (CONS == 1) {

@@ -376,12 +376,11 @@ __global__ void __launch_bounds__(PAIR_THREADS) pair_kick_kernel(PArgs<T> a) {
     if (!live) return;  // whole warps, after the block's last barrier
     if (lane < a.bond_count[i]) {
         const int64_t e = i * LBMD_MAX_BONDS_PER_PARTICLE + lane;
-        T dx, dy, dz;
-        bond_separation(a, R, c, a.slot_of[a.bond_partner[e]], dx, dy, dz);
-        const T g = bond_gain(a.bond_kind[e], (T)a.bond_k[e], (T)a.bond_r0[e], dx * dx + dy * dy + dz * dz);
-        Fx = fma(g, dx, Fx);
-        Fy = fma(g, dy, Fy);
-        Fz = fma(g, dz, Fz);
+        const Separation<T> d = bond_separation(a, R, c, a.slot_of[a.bond_partner[e]]);
+        const T g = bond_gain(a.bond_kind[e], (T)a.bond_k[e], (T)a.bond_r0[e], d);
+        Fx = fma(g, d.x, Fx);
+        Fy = fma(g, d.y, Fy);
+        Fz = fma(g, d.z, Fz);
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
