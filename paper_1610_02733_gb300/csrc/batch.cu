@@ -90,6 +90,7 @@ struct BLbArgs {
     const int *unstable;
     unsigned *items_done;  // per replica: items of the moments kernel taken so far
     int advance;           // the moments kernel advances the LB step counters
+    int reverse;           // take the items from the last to the first
     int nodes_per_block;
     T fs, fis;             // fixed-point scale of the momentum density and its inverse
     // members read by collide()
@@ -116,10 +117,11 @@ __device__ __forceinline__ L4 load_cg(const L4 *p) {
 // it): interpolation (Eq. (5)), friction and random force (Eq. (4)) with the
 // Philox counter of the replica's MD step lb_step m_r + cyc (cyc: the MD step
 // within the replica's LB cycle), velocity Verlet with the force held over
-// the step; variant A hands the transfer straight to the accumulator,
-// variant B keeps the start position and the force for the transfer.  Shared
-// by both schedules of lbmd_batch_run, so that they do the same arithmetic.
-template <typename T, bool CG = false>
+// the step; variant A hands the transfer straight to the accumulator (unless
+// DEFER), variant B keeps the start position and the force for the transfer.
+// Shared by both schedules of lbmd_batch_run, so that they do the same
+// arithmetic.
+template <typename T, bool CG = false, bool DEFER = false>
 __device__ __forceinline__ void batch_couple_particle(const BArgs<T> &a, int64_t p, int r, const BRep<T> &rp,
                                                       int64_t local, unsigned long long lb_step, int cyc) {
     using P = Prec<T>;
@@ -165,7 +167,7 @@ __device__ __forceinline__ void batch_couple_particle(const BArgs<T> &a, int64_t
     }
     a.pos4[p] = P::make_pos(fx, fy, fz, cx + (int64_t)rp.nx * (cy + (int64_t)rp.ny * cz));
     a.vel4[p] = V;
-    if (rp.variant == LBMD_VARIANT_A) {
+    if (!DEFER && rp.variant == LBMD_VARIANT_A) {
         spread_to<T>(a.jacc + rp.node_off, idx, delta, Fx * rp.neg_scale_dt, Fy * rp.neg_scale_dt,
                      Fz * rp.neg_scale_dt);
     } else {
@@ -189,6 +191,12 @@ __device__ __forceinline__ void batch_transfer_particle(const BArgs<T> &a, int64
                  F.z * rp.neg_scale_dt);
 }
 
+// whether the per-tick schedule spreads the transfers with a thread per corner
+template <typename T>
+__host__ __device__ constexpr bool transfers_by_corner() {
+    return sizeof(T) == 4;
+}
+
 // One MD step of every particle (per-tick schedule).
 template <typename T>
 __global__ void __launch_bounds__(256) batch_couple_kernel(BArgs<T> a) {
@@ -200,19 +208,37 @@ __global__ void __launch_bounds__(256) batch_couple_kernel(BArgs<T> a) {
     const BRep<T> &rp = a.rep[r];
     const int64_t local = p - rp.part_off;
     if (local >= rp.np || a.unstable[r]) return;
-    batch_couple_particle(a, p, r, rp, local, a.lb_step[r], a.tick % rp.n_sub);
+    batch_couple_particle<T, false, transfers_by_corner<T>()>(a, p, r, rp, local, a.lb_step[r], a.tick % rp.n_sub);
 }
 
-// Variant B: the transfers of the MD step (per-tick schedule), once every
-// particle has read the node field.
+// The transfers of the MD step (per-tick schedule), once every particle has
+// read the node field.  FP32: of both variants, one thread per corner, so
+// that no thread queues 16 atomics; FP64: of variant B, one thread per
+// particle (its arithmetic would be repeated per corner on the slow FP64 pipe).
 template <typename T>
 __global__ void __launch_bounds__(256) batch_transfer_kernel(BArgs<T> a) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    using P = Prec<T>;
+    constexpr int per = transfers_by_corner<T>() ? 8 : 1;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, p = t / per;
     if (p >= a.n_slots) return;
     const int r = a.prep[p];
     const BRep<T> &rp = a.rep[r];
-    if (rp.variant != LBMD_VARIANT_B || p - rp.part_off >= rp.np || a.unstable[r]) return;
-    batch_transfer_particle(a, p, rp);
+    if (p - rp.part_off >= rp.np || a.unstable[r]) return;
+    if constexpr (per == 1) {
+        if (rp.variant == LBMD_VARIANT_B) batch_transfer_particle(a, p, rp);
+    } else {
+        const typename P::real4 R = a.old4[p], F = a.fc4[p];
+        const CellXYZ c = cell_xyz(P::cell_of(R), rp.fd_nx, rp.fd_ny);
+        const int k = (int)t & 7, ox = k & 1, oy = (k >> 1) & 1, oz = k >> 2;
+        const int x = ox ? (c.x + 1 == rp.nx ? 0 : c.x + 1) : c.x;
+        const int y = oy ? (c.y + 1 == rp.ny ? 0 : c.y + 1) : c.y;
+        const int z = oz ? (c.z + 1 == rp.nz ? 0 : c.z + 1) : c.z;
+        const T d = (ox ? R.x : T(1) - R.x) * (oy ? R.y : T(1) - R.y) * (oz ? R.z : T(1) - R.z);
+        typename P::node4 *field = (rp.variant == LBMD_VARIANT_A ? a.jacc : a.node) + rp.node_off;
+        P::add_transfer(field + ((uint32_t)x + (uint32_t)rp.nx * ((uint32_t)y + (uint32_t)rp.ny * (uint32_t)z)),
+                        P::to_fix_neg(d, F.x * rp.neg_scale_dt), P::to_fix_neg(d, F.y * rp.neg_scale_dt),
+                        P::to_fix_neg(d, F.z * rp.neg_scale_dt));
+    }
 }
 
 // The LB kernels walk their work table with persistent blocks: block b takes
@@ -254,7 +280,7 @@ __device__ __forceinline__ void fetch_item(const BLbArgs<T> &a, ItemWindow &win,
         win.w = make_int2(-1, 0);
         int live = 0;
         if (it < a.n_items) {
-            win.w = a.work[it];
+            win.w = a.work[a.reverse ? a.n_items - 1 - it : it];
             live = !a.unstable[win.w.x];
         }
         win.live = __ballot_sync(0xffffffffu, live);
@@ -388,11 +414,18 @@ __device__ __forceinline__ void batch_collide_node(const BLbArgs<T> &a, const BR
     const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
     const int ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
     const int zm = z == 0 ? nz - 1 : z - 1, zp = z == nz - 1 ? 0 : z + 1;
-    const int X[3] = {xm, x, xp}, Y[3] = {ym, y, yp}, Z[3] = {zm, z, zp};
+    // 32-bit node offsets (a replica has at most 2^27 nodes) and one running
+    // pointer over the 19 arrays: the replica's sizes are not compile-time or
+    // kernel constants here, so 64-bit products per store cost more
+    const uint32_t X[3] = {(uint32_t)xm, (uint32_t)x, (uint32_t)xp};
+    const uint32_t Y[3] = {(uint32_t)(ym * nx), (uint32_t)(y * nx), (uint32_t)(yp * nx)};
+    const uint32_t plane = (uint32_t)(nx * ny);
+    const uint32_t Z[3] = {(uint32_t)zm * plane, (uint32_t)z * plane, (uint32_t)zp * plane};
+    T *fo = fout;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-        const int64_t d = (int64_t)X[CX(i) + 1] + (int64_t)nx * (Y[CY(i) + 1] + (int64_t)ny * Z[CZ(i) + 1]);
-        fout[(int64_t)i * N + d] = f[i];
+        fo[X[CX(i) + 1] + Y[CY(i) + 1] + Z[CZ(i) + 1]] = f[i];
+        fo += N;
     }
 }
 
@@ -426,7 +459,11 @@ __global__ void __launch_bounds__(BATCH_LB_MAX_THREADS, sizeof(T) == 4 ? 4 : 2) 
         const T *fin = ((it.step & 1ull) ? a.f1 : a.f0) + 19 * rp.node_off + loc;
         T *dst = s_pop + (size_t)buf * Q * nb + t;
 #pragma unroll
-        for (int i = 0; i < Q; ++i) cp_async<sizeof(T)>(dst + i * nb, fin + i * N);
+        for (int i = 0; i < Q; ++i) {
+            cp_async<sizeof(T)>(dst, fin);
+            dst += nb;
+            fin += N;
+        }
         const N4 *rec = (rp.variant == LBMD_VARIANT_B ? a.node : a.jacc) + rp.node_off + loc;
         unsigned char *dn = s_node + ((size_t)buf * nb + t) * sizeof(N4);
 #pragma unroll
@@ -464,7 +501,11 @@ __global__ void __launch_bounds__(BATCH_LB_MAX_THREADS) batch_moments_kernel(BLb
         const T *f = (((it.step + 1ull) & 1ull) ? a.f1 : a.f0) + 19 * rp.node_off + loc;
         T *dst = s_pop + (size_t)buf * Q * nb + t;
 #pragma unroll
-        for (int i = 0; i < Q; ++i) cp_async<sizeof(T)>(dst + i * nb, f + i * N);
+        for (int i = 0; i < Q; ++i) {
+            cp_async<sizeof(T)>(dst, f);
+            dst += nb;
+            f += N;
+        }
     };
     auto body = [&](const BItem<T> &it, int64_t loc, int buf) {
         const BRep<T> &rp = it.rep;
@@ -899,6 +940,7 @@ BLbArgs<T> make_lbargs(lbmd_batch *b, int64_t table) {
     a.unstable = b->unstable;
     a.items_done = b->items_done;
     a.advance = 0;
+    a.reverse = 0;
     a.nodes_per_block = b->nodes_per_block;
     a.fs = (T)b->fix.scale;
     a.fis = (T)b->fix.inv_scale;
@@ -928,9 +970,13 @@ unsigned lb_grid(const lbmd_batch *b, K kernel, int64_t n_items, size_t smem) {
     return (unsigned)g;
 }
 
+// The moments walk the table backwards: the populations the collide wrote
+// last are still in L2 (a tick writes more than it holds), and the next
+// collide, forwards again, starts with what the moments read last.
 template <typename T>
-cudaError_t launch_moments(lbmd_batch *b, const BLbArgs<T> &a) {
+cudaError_t launch_moments(lbmd_batch *b, BLbArgs<T> a) {
     if (a.n_items == 0) return cudaSuccess;
+    a.reverse = 1;
     const size_t smem = lb_smem_bytes<T>(b->nodes_per_block, false);
     batch_moments_kernel<T><<<lb_grid(b, batch_moments_kernel<T>, a.n_items, smem), lb_threads(b->nodes_per_block),
                               smem, b->stream>>>(a);
@@ -963,8 +1009,9 @@ cudaError_t launch_particles(lbmd_batch *b, const BArgs<T> &a, bool any_b) {
     const unsigned blocks = (unsigned)((b->n_slots + b->particle_block - 1) / b->particle_block);
     batch_couple_kernel<T><<<blocks, b->particle_block, 0, b->stream>>>(a);
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || !any_b) return e;
-    batch_transfer_kernel<T><<<blocks, b->particle_block, 0, b->stream>>>(a);
+    if (e != cudaSuccess || !(any_b || transfers_by_corner<T>())) return e;
+    const unsigned per = transfers_by_corner<T>() ? 8u : 1u;
+    batch_transfer_kernel<T><<<blocks * per, b->particle_block, 0, b->stream>>>(a);
     return cudaGetLastError();
 }
 
