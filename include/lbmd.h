@@ -111,7 +111,10 @@ enum { LBMD_INTEGRATOR_START = 0, LBMD_INTEGRATOR_HALF_STEP = 1 };
  * bonds or Lennard-Jones forces, nx <= 512, ny and nz >= 6; otherwise ROWS is
  * used; measured slower than ROWS at 0.06 particles per node).  AUTO: ATOMIC
  * while there are fewer than LBMD_SPREAD_ATOMIC_PER_ROW particles per lattice
- * row (y, z) on average, ROWS above (measured crossover).  The transfers are
+ * row (y, z) on average (10 in FP64), ROWS above (measured crossover: 256^3
+ * nodes, m = 10, us per cycle ATOMIC / ROWS: 6.1 per row 1065 / 1211, 9.9 per
+ * row 1384 / 1432, 15.3 per row 1780 / 1672; 128^3: 15.3 per row 360 / 381,
+ * 30.5 per row 548 / 491).  The transfers are
  * fixed-point integers, so all of them give bitwise the same results. */
 enum { LBMD_SPREAD_AUTO = 0, LBMD_SPREAD_ROWS = 1, LBMD_SPREAD_ATOMIC = 2, LBMD_SPREAD_TILES = 3 };
 /* Distribution of the random numbers of the thermal noise (fluid modes,
@@ -128,7 +131,7 @@ enum { LBMD_SPREAD_AUTO = 0, LBMD_SPREAD_ROWS = 1, LBMD_SPREAD_ATOMIC = 2, LBMD_
  * 0), words (x, y) and (z, w) for its three components.  GAUSS needs FP32 or
  * FP64 storage (LBMD_ERR_ARG otherwise). */
 enum { LBMD_NOISE_UNIFORM = 0, LBMD_NOISE_GAUSS = 1 };
-#define LBMD_SPREAD_ATOMIC_PER_ROW 10
+#define LBMD_SPREAD_ATOMIC_PER_ROW 12
 
 typedef struct lbmd_params {
     int32_t nx, ny, nz;    /* lattice nodes per axis (periodic), each >= 2 */

@@ -294,6 +294,17 @@ __global__ void __launch_bounds__(32 * GATHER_WARPS) spread_rows_kernel(PArgs<T>
 // gather is done (spread_particle_atomic, particle_step.cuh).  With `all`,
 // every particle is spread this way and the row gather does not run
 // (LBMD_SPREAD_ATOMIC).
+// Every particle's transfers with atomics (LBMD_SPREAD_ATOMIC), FP32: one thread
+// per corner -- 8 times the threads for a kernel whose threads each wait on
+// their loads and then queue 16 atomics (7 -> 4.5 us at 53,000 particles).  FP64,
+// whose arithmetic would be repeated per corner on its slow pipe, keeps a
+// thread per particle (128^3 nodes, 131,072 particles: 1032 us a cycle, 1121 with this).
+template <typename T>
+__global__ void __launch_bounds__(256) spread_all_kernel(PArgs<T> a) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < 2) a.migrant_count[t] = 0;  // the row gather's lists are not in use
+    if ((t >> 3) < a.np) spread_corner_atomic(a, t >> 3, (int)t & 7);
+}
 template <typename T>
 __global__ void __launch_bounds__(256) migrant_spread_kernel(PArgs<T> a, int all) {
     using P = Prec<T>;
@@ -752,10 +763,19 @@ __global__ void __launch_bounds__(1024) active_finalize_kernel(const int32_t *ro
 // 64^3 nodes, where each of them is a launch's latency; this takes 9.
 constexpr int REORDER_THREADS = 256;
 
-// sum of v[0..n) over the block, read past L1
+// sum of v[0..n) over the block, read past L1, 16 values of a thread in flight
 __device__ __forceinline__ int32_t block_sum_before(const int32_t *v, int n) {
+    const int4 *v4 = reinterpret_cast<const int4 *>(v);
     int32_t s = 0;
-    for (int i = (int)threadIdx.x; i < n; i += REORDER_THREADS) s += __ldcg(v + i);
+    for (int i = (int)threadIdx.x; i < n / 4; i += 4 * REORDER_THREADS) {
+        int4 q[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            q[u] = i + u * REORDER_THREADS < n / 4 ? __ldcg(v4 + i + u * REORDER_THREADS) : make_int4(0, 0, 0, 0);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) s += (q[u].x + q[u].y) + (q[u].z + q[u].w);
+    }
+    if ((int)threadIdx.x < n % 4) s += __ldcg(v + n / 4 * 4 + threadIdx.x);
     int32_t total;
     block_exclusive_scan(s, &total);
     return total;
@@ -955,7 +975,8 @@ static PArgs<T> make_pargs(lbmd_ctx *ctx, int substep) {
 static bool spreads_atomic(const lbmd_ctx *ctx) {
     return ctx->p.spread == LBMD_SPREAD_ATOMIC ||
            (ctx->p.spread == LBMD_SPREAD_AUTO &&
-            ctx->np < (int64_t)LBMD_SPREAD_ATOMIC_PER_ROW * ctx->p.ny * ctx->p.nz);
+            // (the FP64 atomics, a thread per particle, cross over earlier)
+            ctx->np < (int64_t)(ctx->p.precision == LBMD_FP64 ? 10 : LBMD_SPREAD_ATOMIC_PER_ROW) * ctx->p.ny * ctx->p.nz);
 }
 
 // `count` MD steps from `substep` on in one launch, where the system allows it.
@@ -965,11 +986,11 @@ static cudaError_t md_phase_t(lbmd_ctx *ctx, int substep, int count, bool *done)
     *done = true;
     if (ctx->np == 0) return cudaSuccess;
     const bool atomic = spreads_atomic(ctx);
-    // Variant A without conservative forces.  A single step of a dense system
-    // keeps the row gather, whose plain stores cost less than one atomic
-    // hand-over per particle; from two steps on the phase has fewer of both.
-    if (ctx->p.variant == LBMD_VARIANT_A && !has_cons(ctx) &&
-        (atomic || (ctx->p.spread == LBMD_SPREAD_AUTO && count > 1))) {
+    // Variant A without conservative forces, from two steps on; a single step
+    // has nothing to keep in registers (139x146x135 nodes, 32,748 particles, m =
+    // 1: 192 us a cycle against 189 with the separate kernels).
+    if (ctx->p.variant == LBMD_VARIANT_A && !has_cons(ctx) && count > 1 &&
+        (atomic || ctx->p.spread == LBMD_SPREAD_AUTO)) {
         const PArgs<T> a = make_pargs<T>(ctx, substep);
         const unsigned blocks = (unsigned)((ctx->np + 127) / 128);
         if (ctx->p.integrator == LBMD_INTEGRATOR_HALF_STEP)
@@ -1044,8 +1065,10 @@ static cudaError_t md_substep_t(lbmd_ctx *ctx, int substep) {
     if (atomic && cons) {
         // spread by the bond / pair kernel above
     } else if (atomic) {
-        const unsigned sb = (unsigned)((ctx->np + 255) / 256);
-        migrant_spread_kernel<T><<<sb, 256, 0, ctx->stream>>>(a, 1);
+        if (sizeof(T) == 4)
+            spread_all_kernel<T><<<(unsigned)((8 * ctx->np + 255) / 256), 256, 0, ctx->stream>>>(a);
+        else
+            migrant_spread_kernel<T><<<blocks, 256, 0, ctx->stream>>>(a, 1);
     } else {
         const int rows = (int)((int64_t)ctx->p.ny * ctx->p.nz);
         const int gw = ctx->gather_warps;
