@@ -52,6 +52,7 @@ constexpr int64_t BATCH_MAX_PERIOD = 256;
 constexpr int BATCH_VMAX2 = 1;  // |v|^2 beyond which a replica counts as unstable
 constexpr int BATCH_LB_MAX_NODES = 256;  // nodes per work item of the LB kernels, at most
 constexpr int BATCH_LB_MAX_THREADS = BATCH_LB_MAX_NODES + 32;
+constexpr int BATCH_ITEM_WORDS = 8;  // words of a bit per node of an item (at most 256 nodes)
 
 // Per-replica constants, one entry per replica in device memory.
 template <typename T>
@@ -60,6 +61,7 @@ struct BRep {
     int variant, np;
     int64_t node_off;  // first node of the replica in the node arrays (populations: 19 x that)
     int64_t part_off;  // first particle slot of the replica
+    uint32_t word_off, words;  // the replica's words of the touched-node bits
     FastDiv fd_nx, fd_ny;
     uint32_t key0, key1;
     T zeta, dt, half_dt, amp, neg_scale_dt;
@@ -75,6 +77,7 @@ struct BArgs {
     typename P::node4 *node, *jacc;
     const unsigned long long *lb_step;
     int *unstable;
+    uint32_t *touched;  // per replica, a bit per node that took a transfer since its LB step (or null)
     int tick;  // MD step within the period
     T fis;     // 1 / fixed-point scale of the momentum density (shared rho0)
 };
@@ -90,6 +93,8 @@ struct BLbArgs {
     const int *unstable;
     unsigned *items_done;  // per replica: items of the moments kernel taken so far
     int advance;           // the moments kernel advances the LB step counters
+    uint32_t *touched;     // collide: read the transfer of these nodes only, and clear them (null: of all)
+    int newest;            // moments: of the current populations, not those the collide just wrote
     int reverse;           // take the items from the last to the first
     int nodes_per_block;
     T fs, fis;             // fixed-point scale of the momentum density and its inverse
@@ -235,9 +240,10 @@ __global__ void __launch_bounds__(256) batch_transfer_kernel(BArgs<T> a) {
         const int z = oz ? (c.z + 1 == rp.nz ? 0 : c.z + 1) : c.z;
         const T d = (ox ? R.x : T(1) - R.x) * (oy ? R.y : T(1) - R.y) * (oz ? R.z : T(1) - R.z);
         typename P::node4 *field = (rp.variant == LBMD_VARIANT_A ? a.jacc : a.node) + rp.node_off;
-        P::add_transfer(field + ((uint32_t)x + (uint32_t)rp.nx * ((uint32_t)y + (uint32_t)rp.ny * (uint32_t)z)),
-                        P::to_fix_neg(d, F.x * rp.neg_scale_dt), P::to_fix_neg(d, F.y * rp.neg_scale_dt),
+        const uint32_t n = (uint32_t)x + (uint32_t)rp.nx * ((uint32_t)y + (uint32_t)rp.ny * (uint32_t)z);
+        P::add_transfer(field + n, P::to_fix_neg(d, F.x * rp.neg_scale_dt), P::to_fix_neg(d, F.y * rp.neg_scale_dt),
                         P::to_fix_neg(d, F.z * rp.neg_scale_dt));
+        if (a.touched) atomicOr(&a.touched[rp.word_off + (n >> 5)], 1u << (n & 31));
     }
 }
 
@@ -254,6 +260,7 @@ struct BItem {
     BRep<T> rep;
     unsigned long long step;  // the replica's LB step counter
     int r, first;             // replica (< 0: the block has no further item), first node
+    uint32_t touched[BATCH_ITEM_WORDS];  // collide: the touched bits of the item's nodes
 };
 static_assert(sizeof(BRep<float>) % 4 == 0 && sizeof(BRep<double>) % 4 == 0, "BRep is copied by words");
 
@@ -293,6 +300,10 @@ __device__ __forceinline__ void fetch_item(const BLbArgs<T> &a, ItemWindow &win,
     const uint32_t *rw = reinterpret_cast<const uint32_t *>(a.rep + r);
     uint32_t *ow = reinterpret_cast<uint32_t *>(&out->rep);
     for (int k = lane; k < (int)(sizeof(BRep<T>) / 4); k += 32) ow[k] = rw[k];
+    if (a.touched && lane < a.nodes_per_block / 32) {
+        const uint32_t w = (uint32_t)(first >> 5) + (uint32_t)lane;
+        out->touched[lane] = w < a.rep[r].words ? a.touched[a.rep[r].word_off + w] : 0u;
+    }
     if (lane == 0) {
         out->step = a.lb_step[r];
         out->r = r;
@@ -382,9 +393,11 @@ __device__ __forceinline__ typename Prec<T>::node4 staged_node(const unsigned ch
 // (A), MRT collision with noise) from its populations f and record n, and
 // push the result to the neighbours in the other buffer.  Shared by both
 // schedules of lbmd_batch_run.
+// have: the node took a transfer (n holds it), else it has none.
 template <typename T, bool RELAX_FULL>
 __device__ __forceinline__ void batch_collide_node(const BLbArgs<T> &a, const BRep<T> &rp, unsigned long long step,
-                                                   int64_t loc, T (&f)[Q], const typename Prec<T>::node4 &n) {
+                                                   int64_t loc, T (&f)[Q], const typename Prec<T>::node4 &n,
+                                                   bool have = true) {
     using P = Prec<T>;
     using N4 = typename P::node4;
     const int64_t N = (int64_t)rp.nx * rp.ny * rp.nz;
@@ -396,8 +409,9 @@ __device__ __forceinline__ void batch_collide_node(const BLbArgs<T> &a, const BR
     const int y = (int)(row - (uint32_t)z * rp.fd_ny.d);
     T rho, jx, jy, jz;
     node_moments(f, rho, jx, jy, jz);
-    T Fx, Fy, Fz;
-    if (rp.variant == LBMD_VARIANT_B) {
+    T Fx = T(0), Fy = T(0), Fz = T(0);
+    if (!have) {
+    } else if (rp.variant == LBMD_VARIANT_B) {
         Fx = P::from_fix(P::jx_of(n) - P::to_fix(jx, a.fs), a.fis);
         Fy = P::from_fix(P::jy_of(n) - P::to_fix(jy, a.fs), a.fis);
         Fz = P::from_fix(P::jz_of(n) - P::to_fix(jz, a.fs), a.fis);
@@ -442,8 +456,10 @@ __device__ __forceinline__ void batch_moments_node(const BLbArgs<T> &a, const BR
 
 // LB collide and push of the due replicas (Eq. (3)) on the nodes
 // [first, first + nodes_per_block) of each item.  Staged per node: the 19
-// populations and the node record (variant B) or the transfer accumulator
-// (variant A).
+// populations and, of a node that took a transfer, the node record (variant B)
+// or the transfer accumulator (variant A): about an eighth of the nodes at a
+// few hundred particles per replica, whose bits the prefetch warp fetches with
+// the item's header.
 template <typename T, bool RELAX_FULL>
 __global__ void __launch_bounds__(BATCH_LB_MAX_THREADS, sizeof(T) == 4 ? 4 : 2) batch_collide_kernel(BLbArgs<T> a) {
     using P = Prec<T>;
@@ -464,6 +480,7 @@ __global__ void __launch_bounds__(BATCH_LB_MAX_THREADS, sizeof(T) == 4 ? 4 : 2) 
             dst += nb;
             fin += N;
         }
+        if (a.touched && !(it.touched[t >> 5] >> (t & 31) & 1u)) return;
         const N4 *rec = (rp.variant == LBMD_VARIANT_B ? a.node : a.jacc) + rp.node_off + loc;
         unsigned char *dn = s_node + ((size_t)buf * nb + t) * sizeof(N4);
 #pragma unroll
@@ -478,8 +495,12 @@ __global__ void __launch_bounds__(BATCH_LB_MAX_THREADS, sizeof(T) == 4 ? 4 : 2) 
         T f[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i) f[i] = src[i * nb];
-        const N4 n = staged_node<T>(s_node + ((size_t)buf * nb + t) * sizeof(N4));
-        batch_collide_node<T, RELAX_FULL>(a, rp, it.step, loc, f, n);
+        const uint32_t word = a.touched ? it.touched[t >> 5] : 0xffffffffu;
+        const bool have = word >> (t & 31) & 1u;
+        N4 n = {};
+        if (have) n = staged_node<T>(s_node + ((size_t)buf * nb + t) * sizeof(N4));
+        if (a.touched && (t & 31) == 0 && word) a.touched[rp.word_off + ((uint32_t)loc >> 5)] = 0u;
+        batch_collide_node<T, RELAX_FULL>(a, rp, it.step, loc, f, n, have);
     };
     for_items(a, issue, body, [](const BItem<T> &) {});
 }
@@ -498,7 +519,7 @@ __global__ void __launch_bounds__(BATCH_LB_MAX_THREADS) batch_moments_kernel(BLb
         const BRep<T> &rp = it.rep;
         const int64_t N = (int64_t)rp.nx * rp.ny * rp.nz;
         if (loc >= N) return;
-        const T *f = (((it.step + 1ull) & 1ull) ? a.f1 : a.f0) + 19 * rp.node_off + loc;
+        const T *f = (((it.step + (a.newest ? 0ull : 1ull)) & 1ull) ? a.f1 : a.f0) + 19 * rp.node_off + loc;
         T *dst = s_pop + (size_t)buf * Q * nb + t;
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
@@ -527,6 +548,56 @@ __global__ void __launch_bounds__(BATCH_LB_MAX_THREADS) batch_moments_kernel(BLb
         }
     };
     for_items(a, issue, body, advance);
+}
+
+// Replicas with an LB step after every MD step (m = 1), per-tick schedule, FP32:
+// their particles read the node records once, at the positions they have now,
+// so only the records of those corners are made (about an eighth of the nodes;
+// the moments of all of them read and wrote 92 bytes per node).  One thread
+// per corner; corners shared by particles write the same record.  The last
+// block to finish advances the LB step counters of these replicas (each read
+// above).
+template <typename T>
+__global__ void __launch_bounds__(256)
+    batch_corner_moments_kernel(BLbArgs<T> a, const typename Prec<T>::real4 *pos4, const int32_t *prep,
+                                const int32_t *slots, int64_t n_slots, const int32_t *reps, int n_reps,
+                                unsigned *arrived) {
+    using P = Prec<T>;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if ((t >> 3) < n_slots) {
+        const int64_t p = slots[t >> 3];
+        const int r = prep[p];
+        const BRep<T> &rp = a.rep[r];
+        if (p - rp.part_off < rp.np && !a.unstable[r]) {
+            const typename P::real4 R = pos4[p];
+            const CellXYZ c = cell_xyz(P::cell_of(R), rp.fd_nx, rp.fd_ny);
+            const int k = (int)t & 7, ox = k & 1, oy = (k >> 1) & 1, oz = k >> 2;
+            const int x = ox ? (c.x + 1 == rp.nx ? 0 : c.x + 1) : c.x;
+            const int y = oy ? (c.y + 1 == rp.ny ? 0 : c.y + 1) : c.y;
+            const int z = oz ? (c.z + 1 == rp.nz ? 0 : c.z + 1) : c.z;
+            const int64_t N = (int64_t)rp.nx * rp.ny * rp.nz;
+            const int64_t loc = x + (int64_t)rp.nx * (y + (int64_t)rp.ny * z);
+            const T *f = (((a.lb_step[r] + 1ull) & 1ull) ? a.f1 : a.f0) + 19 * rp.node_off + loc;
+            T fl[Q];
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                fl[i] = *f;
+                f += N;
+            }
+            batch_moments_node(a, rp, loc, fl);
+        }
+    }
+    __shared__ int last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(arrived, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    for (int i = (int)threadIdx.x; i < n_reps; i += (int)blockDim.x)
+        if (!a.unstable[reps[i]]) a.lb_step[reps[i]] += 1ull;
+    if (threadIdx.x == 0) *arrived = 0u;
 }
 
 // Persistent schedule (LBMD_BATCH_PERSISTENT).  One launch runs the `ticks`
@@ -786,6 +857,16 @@ struct lbmd_batch {
     bool particles_tuned = false;
     int2 *work = nullptr;
     std::vector<int64_t> work_off, work_len;
+    // FP32: touched-node bits; the replicas with m = 1 come first in every work
+    // table (m1_len items), with their slots, and whether their node records
+    // hold every node (dense) or the particles' corners only
+    uint32_t *touched = nullptr;
+    int64_t n_words = 0, m1_len = 0;
+    std::vector<int32_t> m1_reps, m1_slots;
+    int32_t *d_m1 = nullptr;        // m1_reps, then m1_slots
+    unsigned *m1_arrived = nullptr;
+    bool m1_dense = true;
+    bool all_touched = false;       // transfers were made without setting the bits
     int64_t ticks = 0;  // MD steps done by every replica
     cudaGraphExec_t graph = nullptr;
     double tune_ms_lb[3] = {0, 0, 0}, tune_ms_part[3] = {0, 0, 0};
@@ -839,7 +920,7 @@ size_t real_bytes(const lbmd_batch *b) { return b->precision == LBMD_FP64 ? 8 : 
 void free_batch(lbmd_batch *b) {
     void *bufs[] = {b->f[0], b->f[1],  b->node,  b->jacc,  b->pos4,  b->vel4,  b->fc4,  b->old4,
                     b->prep, b->rep,   b->lb_step, b->unstable, b->items_done, b->kin, b->staging, b->work,
-                    b->order, b->queue, b->taken, b->dtick};
+                    b->order, b->queue, b->taken, b->dtick, b->touched, b->d_m1, b->m1_arrived};
     for (void *p : bufs)
         if (p) cudaFree(p);
     if (b->graph) cudaGraphExecDestroy(b->graph);
@@ -850,6 +931,7 @@ void free_batch(lbmd_batch *b) {
 template <typename T>
 void fill_reps(const lbmd_batch *b, std::vector<BRep<T>> &out) {
     out.resize(b->R);
+    uint32_t words = 0;
     for (int r = 0; r < b->R; ++r) {
         BRep<T> &q = out[r];
         q.nx = b->nx[r];
@@ -860,6 +942,9 @@ void fill_reps(const lbmd_batch *b, std::vector<BRep<T>> &out) {
         q.np = b->np[r];
         q.node_off = b->node_off[r];
         q.part_off = b->part_off[r];
+        q.word_off = words;
+        q.words = (uint32_t)(((int64_t)b->nx[r] * b->ny[r] * b->nz[r] + 31) / 32);
+        words += q.words;
         q.fd_nx = make_fastdiv((uint32_t)b->nx[r]);
         q.fd_ny = make_fastdiv((uint32_t)b->ny[r]);
         q.key0 = (uint32_t)(b->seed[r] & 0xffffffffu);
@@ -890,11 +975,14 @@ cudaError_t build_tables(lbmd_batch *b) {
     const int nb = b->nodes_per_block;
     for (int64_t k = 0; k <= b->period; ++k) {
         b->work_off[k] = (int64_t)work.size();
-        for (int r = 0; r < b->R; ++r) {
-            const bool is_due = k == b->period || (k + 1) % b->n_sub[r] == 0;
-            if (!is_due) continue;
-            const int64_t N = (int64_t)b->nx[r] * b->ny[r] * b->nz[r];
-            for (int64_t s = 0; s < N; s += nb) work.push_back(make_int2(r, (int)s));
+        for (int first : {1, 0}) {  // m = 1 first: due in every tick
+            for (int r = 0; r < b->R; ++r) {
+                const bool is_due = k == b->period || (k + 1) % b->n_sub[r] == 0;
+                if (!is_due || (b->n_sub[r] == 1) != (first == 1)) continue;
+                const int64_t N = (int64_t)b->nx[r] * b->ny[r] * b->nz[r];
+                for (int64_t s = 0; s < N; s += nb) work.push_back(make_int2(r, (int)s));
+            }
+            if (first == 1) b->m1_len = (int64_t)work.size() - b->work_off[k];
         }
         b->work_len[k] = (int64_t)work.size() - b->work_off[k];
     }
@@ -921,6 +1009,7 @@ BArgs<T> make_bargs(lbmd_batch *b, int tick) {
     a.jacc = static_cast<typename P::node4 *>(b->jacc);
     a.lb_step = b->lb_step;
     a.unstable = b->unstable;
+    a.touched = b->touched;
     a.tick = tick;
     a.fis = (T)b->fix.inv_scale;
     return a;
@@ -940,6 +1029,8 @@ BLbArgs<T> make_lbargs(lbmd_batch *b, int64_t table) {
     a.unstable = b->unstable;
     a.items_done = b->items_done;
     a.advance = 0;
+    a.touched = nullptr;
+    a.newest = 0;
     a.reverse = 0;
     a.nodes_per_block = b->nodes_per_block;
     a.fs = (T)b->fix.scale;
@@ -983,14 +1074,27 @@ cudaError_t launch_moments(lbmd_batch *b, BLbArgs<T> a) {
     return cudaGetLastError();
 }
 
-// collide and moments of the work table; with step, the moments kernel
-// advances the LB step counters of the replicas it covered
+// the node records of every node of the replicas with m = 1, where only those
+// of the particles' corners are current
+cudaError_t fill_m1_records(lbmd_batch *b) {
+    if (b->m1_dense) return cudaSuccess;
+    b->m1_dense = true;
+    BLbArgs<float> a = make_lbargs<float>(b, 0);
+    a.n_items = b->m1_len;
+    a.newest = 1;
+    return launch_moments<float>(b, a);
+}
+
+// collide and moments of the work table; with step, the moments kernels
+// advance the LB step counters of the replicas they covered
 template <typename T>
 cudaError_t launch_lb_tables(lbmd_batch *b, int64_t table, bool step) {
     BLbArgs<T> a = make_lbargs<T>(b, table);
     if (a.n_items == 0) return cudaSuccess;
     const int th = lb_threads(b->nodes_per_block);
     const size_t smem = lb_smem_bytes<T>(b->nodes_per_block, true);
+    const bool sparse = step && transfers_by_corner<T>();  // (tuning steps everything alike)
+    if (sparse) a.touched = b->touched;
     if (b->co.gamma_bulk == 0.0 && b->co.gamma_ghost == 0.0)
         batch_collide_kernel<T, true>
             <<<lb_grid(b, batch_collide_kernel<T, true>, a.n_items, smem), th, smem, b->stream>>>(a);
@@ -1000,6 +1104,16 @@ cudaError_t launch_lb_tables(lbmd_batch *b, int64_t table, bool step) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     a.advance = step ? 1 : 0;
+    a.touched = nullptr;
+    if (!sparse || b->m1_reps.empty()) return launch_moments<T>(b, a);
+    const int64_t n = (int64_t)b->m1_slots.size();
+    const int32_t *reps = b->d_m1, *slots = b->d_m1 + b->m1_reps.size();
+    batch_corner_moments_kernel<T><<<(unsigned)std::max<int64_t>(1, (8 * n + 255) / 256), 256, 0, b->stream>>>(
+        a, static_cast<const typename Prec<T>::real4 *>(b->pos4), b->prep, slots, n, reps, (int)b->m1_reps.size(),
+        b->m1_arrived);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    a.work += b->m1_len;
+    a.n_items -= b->m1_len;
     return launch_moments<T>(b, a);
 }
 
@@ -1122,6 +1236,12 @@ cudaError_t init_state(lbmd_batch *b) {
     b->dtick_valid = b->ticks == 0;
     if ((e = cudaMemsetAsync(b->unstable, 0, b->R * sizeof(int), b->stream)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(b->jacc, 0, b->n_nodes * 4 * real_bytes(b), b->stream)) != cudaSuccess) return e;
+    if (b->touched) {
+        if ((e = cudaMemsetAsync(b->touched, 0, b->n_words * sizeof(uint32_t), b->stream)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(b->m1_arrived, 0, sizeof(unsigned), b->stream)) != cudaSuccess) return e;
+    }
+    b->m1_dense = true;
+    b->all_touched = false;
     // node field of the rest state: the moments kernel reads buffer
     // (lb_step + 1) & 1, so run it on the "all" table with lb_step = 0 after
     // copying f[0] into f[1]
@@ -1204,6 +1324,7 @@ cudaError_t tune_particles(lbmd_batch *b) {
         a.node = static_cast<typename Prec<T>::node4 *>(node);
         a.jacc = static_cast<typename Prec<T>::node4 *>(jacc);
         a.unstable = unst;
+        a.touched = nullptr;
         const bool anyb = any_variant_b(b);
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
@@ -1278,6 +1399,11 @@ lbmd_status run_persistent(lbmd_batch *b, int64_t md_steps) {
     const int C = b->cluster_req ? b->cluster_req : b->cluster_tuned;
     const int nc = persistent_clusters<T>(b, C);
     if (nc < 1) return bfail(b, LBMD_ERR_CUDA, "no cluster of the persistent schedule fits on the device");
+    // it makes every node record and does not keep the touched bits
+    if (md_steps > 0) {
+        BCK(b, fill_m1_records(b));
+        b->all_touched = true;
+    }
     if (!b->dtick_valid) {
         const long long t = b->ticks;
         BCK(b, cudaStreamSynchronize(b->stream));
@@ -1455,6 +1581,27 @@ lbmd_status lbmd_batch_create(const lbmd_batch_params *p, lbmd_batch **out) {
             return s;
         }
     }
+    if (b->precision == LBMD_FP32) {
+        for (int r = 0; r < R; ++r) {
+            b->n_words += ((int64_t)b->nx[r] * b->ny[r] * b->nz[r] + 31) / 32;
+            if (b->n_sub[r] != 1) continue;
+            b->m1_reps.push_back(r);
+            for (int64_t i = 0; i < b->cap[r]; ++i) b->m1_slots.push_back((int32_t)(b->part_off[r] + i));
+        }
+        std::vector<int32_t> m1(b->m1_reps);
+        m1.insert(m1.end(), b->m1_slots.begin(), b->m1_slots.end());
+        cudaError_t e = cudaMalloc(&b->touched, (size_t)b->n_words * sizeof(uint32_t));
+        if (e == cudaSuccess) e = cudaMalloc(&b->m1_arrived, sizeof(unsigned));
+        if (e == cudaSuccess) e = cudaMalloc(&b->d_m1, std::max<size_t>(1, m1.size()) * sizeof(int32_t));
+        if (e == cudaSuccess && !m1.empty())
+            e = cudaMemcpy(b->d_m1, m1.data(), m1.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) {
+            lbmd_status s = bcuda(nullptr, e, "cudaMalloc");
+            free_batch(b);
+            delete b;
+            return s;
+        }
+    }
     std::vector<int32_t> prep((size_t)sl, 0);
     for (int r = 0; r < R; ++r)
         for (int64_t i = 0; i < b->cap[r]; ++i) prep[(size_t)(b->part_off[r] + i)] = r;
@@ -1512,6 +1659,7 @@ lbmd_status lbmd_batch_add_particles(lbmd_batch *b, int32_t r, int64_t n, const 
             static_cast<float4 *>(b->vel4), dpos, dvel, mass ? dm : nullptr);
     BCK(b, cudaGetLastError());
     b->np[r] += (int)n;
+    if (b->n_sub[r] == 1) BCK(b, fill_m1_records(b));  // the new particles' corners too
     BCK(b, LBMD_BATCH_DISPATCH(b, upload_reps, b));
     BCK(b, upload_order(b));
     BCK(b, cudaStreamSynchronize(b->stream));
@@ -1528,7 +1676,13 @@ lbmd_status lbmd_batch_run(lbmd_batch *b, int64_t md_steps) {
     if (!b || md_steps < 0) return LBMD_ERR_ARG;
     if (b->schedule == LBMD_BATCH_PERSISTENT) return LBMD_BATCH_DISPATCH(b, run_persistent, b, md_steps);
     if (!b->particles_tuned && b->n_slots > 0) BCK(b, LBMD_BATCH_DISPATCH(b, tune_particles, b));
-    if (md_steps > 0) b->dtick_valid = false;  // the device tick copy serves the persistent schedule only
+    if (md_steps > 0) {
+        b->dtick_valid = false;  // the device tick copy serves the persistent schedule only
+        if (b->touched && b->all_touched)  // after the persistent schedule: any node may hold a transfer
+            BCK(b, cudaMemsetAsync(b->touched, 0xff, b->n_words * sizeof(uint32_t), b->stream));
+        b->all_touched = false;
+        if (b->touched && !b->m1_reps.empty()) b->m1_dense = false;
+    }
     int64_t left = md_steps;
     // eager ticks up to the next period boundary, whole periods from the
     // captured graph, eager ticks for the rest
