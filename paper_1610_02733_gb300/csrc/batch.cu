@@ -52,6 +52,12 @@ constexpr int64_t BATCH_MAX_PERIOD = 256;
 constexpr int BATCH_VMAX2 = 1;  // |v|^2 beyond which a replica counts as unstable
 constexpr int BATCH_LB_MAX_NODES = 256;  // nodes per work item of the LB kernels, at most
 constexpr int BATCH_LB_MAX_THREADS = BATCH_LB_MAX_NODES + 32;
+// Touched-node bits and corner records (per-tick schedule, FP32) where the
+// replicas with m = 1 have this many nodes, at least four per corner of their
+// particles.  Measured, us per tick with / without: 863,360 nodes and few
+// particles 66.3 / 73.6, 444,608 39.7 / 41.8, 222,144 30.2 / 26.4, 44,480 17.9
+// / 15.2; 523,072 nodes with half of them corners 64.5 / 54.3.
+constexpr int64_t BATCH_SPARSE_NODES = 400000;
 constexpr int BATCH_ITEM_WORDS = 8;  // words of a bit per node of an item (at most 256 nodes)
 
 // Per-replica constants, one entry per replica in device memory.
@@ -857,7 +863,7 @@ struct lbmd_batch {
     bool particles_tuned = false;
     int2 *work = nullptr;
     std::vector<int64_t> work_off, work_len;
-    // FP32: touched-node bits; the replicas with m = 1 come first in every work
+    // touched-node bits (or null: see BATCH_SPARSE_NODES); the replicas with m = 1 come first in every work
     // table (m1_len items), with their slots, and whether their node records
     // hold every node (dense) or the particles' corners only
     uint32_t *touched = nullptr;
@@ -1093,7 +1099,7 @@ cudaError_t launch_lb_tables(lbmd_batch *b, int64_t table, bool step) {
     if (a.n_items == 0) return cudaSuccess;
     const int th = lb_threads(b->nodes_per_block);
     const size_t smem = lb_smem_bytes<T>(b->nodes_per_block, true);
-    const bool sparse = step && transfers_by_corner<T>();  // (tuning steps everything alike)
+    const bool sparse = step && b->touched;  // (tuning steps everything alike)
     if (sparse) a.touched = b->touched;
     if (b->co.gamma_bulk == 0.0 && b->co.gamma_ghost == 0.0)
         batch_collide_kernel<T, true>
@@ -1581,7 +1587,13 @@ lbmd_status lbmd_batch_create(const lbmd_batch_params *p, lbmd_batch **out) {
             return s;
         }
     }
-    if (b->precision == LBMD_FP32) {
+    int64_t m1_nodes = 0, m1_corners = 0;
+    for (int r = 0; r < R; ++r) {
+        if (b->n_sub[r] != 1) continue;
+        m1_nodes += (int64_t)b->nx[r] * b->ny[r] * b->nz[r];
+        m1_corners += 8ll * b->cap[r];
+    }
+    if (b->precision == LBMD_FP32 && m1_nodes >= BATCH_SPARSE_NODES && 4 * m1_corners <= m1_nodes) {
         for (int r = 0; r < R; ++r) {
             b->n_words += ((int64_t)b->nx[r] * b->ny[r] * b->nz[r] + 31) / 32;
             if (b->n_sub[r] != 1) continue;

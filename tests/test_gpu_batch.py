@@ -237,11 +237,12 @@ def test_full_batched_configuration_sampled(precision, schedule):
 
 
 def test_replicas_with_an_lb_step_every_md_step_follow_fast_particles():
-    # m = 1 replicas keep the node records of their particles' corners only:
-    # particles that cross cells every step, added between runs, without
-    # particles at all, and under both schedules in turn, against one replica
-    # per batch under the schedule that makes every record
-    dims, n, m = [(12, 9, 7), (5, 33, 6), (8, 8, 8), (16, 4, 10)], [60, 1, 0, 25], [1, 1, 1, 2]
+    # m = 1 replicas with many nodes keep the node records of their particles'
+    # corners only: particles that cross cells every step, added between runs,
+    # a replica without particles, and both schedules in turn, against one
+    # replica per batch under the schedule that makes every record (the last
+    # replica alone is large enough to be kept that way too)
+    dims, n, m = [(12, 9, 7), (5, 33, 6), (8, 8, 8), (16, 4, 10), (90, 71, 67)], [60, 1, 0, 25, 50], [1, 1, 1, 2, 1]
     pos = [inputs.uniform_positions(max(k, 1), d, 3 + i)[:k] for i, (k, d) in enumerate(zip(n, dims))]
     vel = [inputs.maxwell_velocities(max(k, 1), 0.05, 3 + i)[:k] for i, (k, d) in enumerate(zip(n, dims))]
     more = [(inputs.uniform_positions(7, d, 50 + i), inputs.maxwell_velocities(7, 0.05, 50 + i))
@@ -265,9 +266,9 @@ def test_replicas_with_an_lb_step_every_md_step_follow_fast_particles():
         return out
 
     g, p = "period_graph", "persistent"
-    mixed = run(range(4), [(g, 3), (p, 2), (g, 4), (p, 1), (g, 5)])
-    graph = run(range(4), [(g, 3), (g, 2), (g, 4), (g, 1), (g, 5)])
-    for r in range(4):
+    mixed = run(range(5), [(g, 3), (p, 2), (g, 4), (p, 1), (g, 5)])
+    graph = run(range(5), [(g, 3), (g, 2), (g, 4), (g, 1), (g, 5)])
+    for r in range(5):
         want = run([r], [(p, 3), (p, 2), (p, 4), (p, 1), (p, 5)])[0]
         for a, b, c in zip(want, mixed[r], graph[r]):
             assert np.array_equal(a, b) and np.array_equal(a, c)
