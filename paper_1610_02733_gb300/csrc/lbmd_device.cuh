@@ -126,6 +126,26 @@ __host__ __device__ __forceinline__ long long to_fixed(double v, int scale) {
     return (long long)(q ^ (unsigned long long)s) - s;
 }
 
+// a b rounded to an integer (half away from zero, of the product's leading 62
+// bits or more); *fits: whether that holds (always for |a b| < 2^61, never for
+// 2^62 and more, infinity or NaN).
+__host__ __device__ __forceinline__ long long product_fixed(double a, double b, bool *fits) {
+    const unsigned long long u = bits_of(a), v = bits_of(b);
+    const int ex = (int)((u >> 52) & 0x7ffu) + (int)((v >> 52) & 0x7ffu);
+#ifdef __CUDA_ARCH__
+    const unsigned long long p = __umul64hi((u << 11) | (1ull << 63), (v << 11) | (1ull << 63));
+#else
+    const unsigned long long p =
+        (unsigned long long)(((unsigned __int128)((u << 11) | (1ull << 63)) * ((v << 11) | (1ull << 63))) >> 64);
+#endif
+    int r = 2 * 1023 + 62 - ex;  // a b = p 2^(ex - 2046 - 62), 2^62 <= p < 2^64
+    *fits = r >= 2;
+    r = r < 1 ? 1 : r > 65 ? 65 : r;
+    const unsigned long long q = r == 65 ? 0ull : ((p >> (r - 1)) + 1ull) >> 1;
+    const long long s = (long long)(u ^ v) >> 63;
+    return (long long)(q ^ (unsigned long long)s) - s;
+}
+
 // the integer v times 2^-scale, rounded to nearest even
 __host__ __device__ __forceinline__ double from_fixed(long long v, int scale) {
     const long long s = v >> 63;
@@ -290,7 +310,11 @@ struct Prec<double> {
     // rounded to nearest; 2^62 and more, and NaN, by the hardware conversion
     // (volatile: kept inside its branch)
     __device__ static __forceinline__ fix to_fix(double v, double s) { return rounded(v * s); }
-    __device__ static __forceinline__ fix to_fix_neg(double d, double ps) { return rounded(d * ps); }
+    __device__ static __forceinline__ fix to_fix_neg(double d, double ps) {
+        bool fits;
+        const fix v = product_fixed(d, ps, &fits);
+        return fits ? v : rounded(d * ps);
+    }
     __device__ static __forceinline__ fix rounded(double v) {
         if (((unsigned)__double2hiint(v) & 0x7fffffffu) >= (unsigned)(1023 + 62) << 20) {
             fix r;

@@ -388,6 +388,8 @@ __global__ void __launch_bounds__(2 * PHASE_THREADS, sizeof(T) == 4 ? 2 : 1)
             kind = a.bond_kind[e];
         }
     }
+    // ideal particles of variant A wait for nobody
+    const bool coupled = CONS || a.variant != LBMD_VARIANT_A;
     const int no_list = CONS == 2 ? __syncthreads_or(a.nb_count[id] < 0) : 0;  // in this block
     const uint32_t step0 = md_step_index(a);
     const T hm = a.half_dt * V.w;  // V.w = 1 / mass
@@ -437,7 +439,7 @@ __global__ void __launch_bounds__(2 * PHASE_THREADS, sizeof(T) == 4 ? 2 : 1)
             }
         }
         // every particle has read the nodes, and its position is known
-        if (!bar.wait()) return;
+        if (coupled && !bar.wait()) return;
         if (CONS) {
             const typename P::real4 R = P::make_pos(fx, fy, fz, 0);
             T g = T(0), dx = T(0), dy = T(0), dz = T(0);
@@ -487,7 +489,7 @@ __global__ void __launch_bounds__(2 * PHASE_THREADS, sizeof(T) == 4 ? 2 : 1)
             P::add_transfer(to, P::to_fix_neg(delta, tx), P::to_fix_neg(delta, ty), P::to_fix_neg(delta, tz));
         }
         // all transfers are in, and the other positions have been read
-        if (s + 1 < count && !bar.wait()) return;
+        if (coupled && s + 1 < count && !bar.wait()) return;
     }
     bar.finish();
     if (!live || lane != 0) return;

@@ -314,8 +314,12 @@ __global__ void __launch_bounds__(256) migrant_spread_kernel(PArgs<T> a, int all
     // during this one)
     if (blockIdx.x == 0 && threadIdx.x == 0) a.migrant_count[par ^ 1] = 0;
     const int32_t *list = a.migrant_slot + (int64_t)par * a.np_cap;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-        spread_particle_atomic(a, all ? (int64_t)t : (int64_t)list[t]);
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (sizeof(T) == 4 && !all) {  // a thread per corner, as in spread_all_kernel
+        for (; t < 8 * (int64_t)n; t += stride) spread_corner_atomic(a, (int64_t)list[t >> 3], (int)t & 7);
+    } else {
+        for (; t < n; t += stride) spread_particle_atomic(a, all ? t : (int64_t)list[t]);
     }
 }
 
@@ -988,8 +992,13 @@ static cudaError_t md_phase_t(lbmd_ctx *ctx, int substep, int count, bool *done)
     const bool atomic = spreads_atomic(ctx);
     // Variant A without conservative forces, from two steps on; a single step
     // has nothing to keep in registers (139x146x135 nodes, 32,748 particles, m =
-    // 1: 192 us a cycle against 189 with the separate kernels).
-    if (ctx->p.variant == LBMD_VARIANT_A && !has_cons(ctx) && count > 1 &&
+    // 1: 192 us a cycle against 189 with the separate kernels).  A few thousand
+    // particles and less are left to the teams below: 48^3 nodes, 500
+    // particles, m = 4, 30.8 us a cycle against 35.2 (FP64, 32^3, m = 5: 54.3
+    // against 69.9); with 5000 particles the two are even, with 19,000 and m = 10
+    // it is 49.2 against 40.2.
+    const bool team_a = 8 * ctx->np <= (int64_t)128 * ctx->sm_count;
+    if (ctx->p.variant == LBMD_VARIANT_A && !has_cons(ctx) && count > 1 && !team_a &&
         (atomic || ctx->p.spread == LBMD_SPREAD_AUTO)) {
         const PArgs<T> a = make_pargs<T>(ctx, substep);
         const unsigned blocks = (unsigned)((ctx->np + 127) / 128);
@@ -999,9 +1008,10 @@ static cudaError_t md_phase_t(lbmd_ctx *ctx, int substep, int count, bool *done)
             frozen_phase_kernel<T, false><<<blocks, 128, 0, ctx->stream>>>(a, count);
         return cudaGetLastError();
     }
-    // Variants B and C, and conservative forces in any variant, while a team
-    // of lanes per particle fits the GPU at once.
-    if (ctx->p.spread == LBMD_SPREAD_AUTO || ctx->p.spread == LBMD_SPREAD_ATOMIC) {
+    // Variants B and C, conservative forces in any variant, and few particles of
+    // variant A, while a team of lanes per particle fits the GPU at once.
+    if ((ctx->p.spread == LBMD_SPREAD_AUTO || ctx->p.spread == LBMD_SPREAD_ATOMIC) &&
+        (ctx->p.variant != LBMD_VARIANT_A || has_cons(ctx) || team_a)) {
         const bool half = ctx->p.integrator == LBMD_INTEGRATOR_HALF_STEP;
         const int cons = ctx->lj_rc > 0.0 ? 2 : has_cons(ctx) ? 1 : 0;
         const int64_t threads = ctx->np * (cons == 2 ? 32 : 8);
@@ -1075,7 +1085,7 @@ static cudaError_t md_substep_t(lbmd_ctx *ctx, int substep) {
         const unsigned gblocks = (unsigned)((rows + gw - 1) / gw);
         spread_rows_kernel<T><<<gblocks, 32 * gw, gather_smem_bytes<T>(ctx, gw), ctx->stream>>>(a, rows);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        migrant_spread_kernel<T><<<ctx->sm_count, 256, 0, ctx->stream>>>(a, 0);
+        migrant_spread_kernel<T><<<2 * ctx->sm_count, 256, 0, ctx->stream>>>(a, 0);
     }
     return cudaGetLastError();
 }

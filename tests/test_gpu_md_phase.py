@@ -28,7 +28,8 @@ def _same(a, b):
 
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
 @pytest.mark.parametrize("integrator", ["start", "half_step"])
-@pytest.mark.parametrize("shape,n,m", [((7, 5, 6), 1, 1), ((40, 6, 5), 129, 4), ((20, 9, 8), 1500, 10)])
+@pytest.mark.parametrize("shape,n,m", [((7, 5, 6), 1, 1), ((40, 6, 5), 129, 4), ((20, 9, 8), 1500, 10),
+                                       ((30, 29, 27), 4000, 3)])
 def test_variant_a_phase(precision, integrator, shape, n, m):
     # slow particles (they stay in their cells) and ones that cross several
     # cells per cycle; captured cycles, single steps, and both in turn
