@@ -41,13 +41,6 @@ struct PairSums {
     }
 };
 
-// MRT collision with forcing and noise at one node; f holds f* on entry and
-// f' on exit -- or, for a deviation storage form, f* - b and f' - b with b the
-// stored rest values (see PopStore): the collision is linear in the moments,
-// and the mass mode takes rho_m (the density, or its part sum_i (f*_i - b_i)),
-// while u, the equilibria and the noise amplitudes take the density rho.  With
-// sum_i w_i = 1 and sum_i w_i e_k(c_i) = 0 for k > 0 the deviations then keep
-// their sum, so the mass is conserved up to the rounding of small numbers.
 // 1/rho and sqrt(rho): IEEE in FP64; in FP32 both from one reciprocal square
 // root (at most a few ulp, far below the FP32 path's tolerance)
 __device__ __forceinline__ void rho_factors(double rho, double &inv, double &sq) {
@@ -119,6 +112,14 @@ __device__ __forceinline__ double centred16x2(uint32_t word, int high, double) {
     return from_fixed((long long)(2u * h) - 65535ll, 0);
 }
 
+// MRT collision with forcing and noise at one node; f holds f* on entry and
+// f' on exit -- or, for a deviation storage form, f* - b and f' - b with b the
+// stored rest values (see PopStore): the collision is linear in the moments,
+// and the mass mode takes rho_m (the density, or its part sum_i (f*_i - b_i)),
+// while u, the equilibria and the noise amplitudes take the density rho.  With
+// sum_i w_i = 1 and sum_i w_i e_k(c_i) = 0 for k > 0 the deviations then keep
+// their sum, so the mass is conserved up to the rounding of small numbers.
+//
 // RELAX_FULL: gamma_bulk = gamma_ghost = 0 (the default reading), so the
 // bulk and ghost modes relax fully, m'_k = m^eq_k exactly, and their moments
 // m_k are not needed.

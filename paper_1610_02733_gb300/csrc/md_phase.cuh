@@ -215,14 +215,14 @@ __device__ __forceinline__ T bond_gain(uint8_t kind, T k, T r0, const Separation
 
 // Bond forces on particle `id` at (R, c), summed over its partners in a fixed
 // order.
-template <bool L2 = false, typename T>
+template <typename T>
 __device__ __forceinline__ void bond_forces(const PArgs<T> &a, int64_t id, const typename Prec<T>::real4 &R,
                                             const CellXYZ &c, T &Fx, T &Fy, T &Fz) {
     Fx = Fy = Fz = T(0);
     const int nbond = a.bond_count[id];
     for (int b = 0; b < nbond; ++b) {
         const int64_t e = id * LBMD_MAX_BONDS_PER_PARTICLE + b;
-        const Separation<T> d = bond_separation<L2>(a, R, c, a.slot_of[a.bond_partner[e]]);
+        const Separation<T> d = bond_separation(a, R, c, a.slot_of[a.bond_partner[e]]);
         const T g = bond_gain(a.bond_kind[e], (T)a.bond_k[e], (T)a.bond_r0[e], d);
         Fx = fma(g, d.x, Fx);
         Fy = fma(g, d.y, Fy);

@@ -132,8 +132,7 @@ __device__ __forceinline__ D4 load_l2(const D4 *p) {
 // record and all records before the first use, so a thread waits on two
 // round trips to memory and has 8 records in flight; fetching them row by
 // row between the divisions of the interpolation left two.
-// L2: read past L1 (the records change during the launch).
-template <bool L2 = false, typename T>
+template <typename T>
 __device__ __forceinline__ void corner_records(const PArgs<T> &a, const CellXYZ &c, typename Prec<T>::node4 n[8]) {
     using N4 = typename Prec<T>::node4;
     uint32_t rows[4];
@@ -165,19 +164,16 @@ __device__ __forceinline__ void corner_records(const PArgs<T> &a, const CellXYZ 
         }
     }
 #pragma unroll
-    for (int k = 0; k < 8; ++k) n[k] = L2 ? load_l2(ptr[k]) : *ptr[k];
+    for (int k = 0; k < 8; ++k) n[k] = *ptr[k];
 }
 
 // The same for a particle in cell c, its records read from memory.
-template <bool L2 = false, typename T>
+template <typename T>
 __device__ __forceinline__ void interp_u(const PArgs<T> &a, const CellXYZ &c, T fx, T fy, T fz, T &ux, T &uy,
                                          T &uz) {
     using P = Prec<T>;
-    uint32_t rows[4];
-    corner_rows(c, a.ny, a.nz, rows);
-    const int x1 = c.x + 1 == a.nx ? 0 : c.x + 1;
     typename P::node4 nn[8];
-    corner_records<L2>(a, c, nn);
+    corner_records(a, c, nn);
     interp_u_from(fx, fy, fz, a.fis, ux, uy, uz, [&](int q, typename P::node4 &n0, typename P::node4 &n1) {
         n0 = nn[2 * q];
         n1 = nn[2 * q + 1];
