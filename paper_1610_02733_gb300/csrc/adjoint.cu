@@ -476,6 +476,7 @@ __global__ void __launch_bounds__(AD_THREADS)
         const T rho = P::rho_of(n), jx = P::from_fix(P::jx_of(n), a.fis), jy = P::from_fix(P::jy_of(n), a.fis),
                 jz = P::from_fix(P::jz_of(n), a.fis);
         const T delta = q.w0 * q.w1 * q.w2, w = delta / rho;
+        bar.arrive();  // while the force is computed
         T ux = T(0), uy = T(0), uz = T(0);
 #pragma unroll
         for (int h = 0; h < 8; ++h) {
@@ -515,7 +516,7 @@ __global__ void __launch_bounds__(AD_THREADS)
         if (live)
             P::add_transfer(&node[q.node], P::to_fix_neg(delta, Fx * a.neg_scale_dt),
                             P::to_fix_neg(delta, Fy * a.neg_scale_dt), P::to_fix_neg(delta, Fz * a.neg_scale_dt));
-        if (s + 1 < a.n_sub && !bar.wait()) return;  // all transfers are in
+        if (s + 1 < a.n_sub && !bar.meet()) return;  // all transfers are in
     }
     bar.finish();
     if (!live || k != 0) return;
@@ -543,6 +544,7 @@ __global__ void __launch_bounds__(AD_THREADS)
         const CellXYZ c = cell_xyz(P::cell_of(R), a.fd_nx, a.fd_ny);
         const AdCorner<T> q(a, c, R.x, R.y, R.z, k);
         const typename P::real4 nb = ad_load(&nbar[q.node]);
+        bar.arrive();  // while the adjoints of the particle are computed
         const T delta = q.w0 * q.w1 * q.w2, im = V.w, dd = dt * delta;
         // F-bar: through v' = v + (dt/m) F, x' = x + dt v + dt^2/(2m) F, the
         // transfers -dt delta_k F and the drag term of the loss
@@ -576,7 +578,7 @@ __global__ void __launch_bounds__(AD_THREADS)
             atomic_addT(n + 2, sk * Fb[1]);
             atomic_addT(n + 3, sk * Fb[2]);
         }
-        if (s > 0 && !bar.wait()) return;  // all of this step's are in
+        if (s > 0 && !bar.meet()) return;  // all of this step's are in
     }
     bar.finish();
     if (!live || k != 0) return;

@@ -422,6 +422,7 @@ __global__ void __launch_bounds__(2 * PHASE_THREADS, sizeof(T) == 4 ? 2 : 1)
         const T w = quotient(delta, P::rho_of(n));
         const T jx = P::from_fix(P::jx_of(n), a.fis), jy = P::from_fix(P::jy_of(n), a.fis),
                 jz = P::from_fix(P::jz_of(n), a.fis);
+        if (coupled) bar.arrive();  // while the force is computed
         T ux = T(0), uy = T(0), uz = T(0);
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
@@ -432,14 +433,21 @@ __global__ void __launch_bounds__(2 * PHASE_THREADS, sizeof(T) == 4 ? 2 : 1)
         }
         coupling_force_id(a, id, step0 + (uint32_t)s, V, ux, uy, uz, Fx, Fy, Fz);
         if (!HALF) kick_drift();
+        // every particle has read the nodes, and the others' positions of the
+        // step before
+        if (coupled && !bar.wait()) return;
         if (CONS) {
             if (live && lane == 0) {
                 if (CONS == 2) check_list_skin(a, p, c, fx, fy, fz);
                 a.pos4[p] = P::make_pos(fx, fy, fz, c.x + (int64_t)a.nx * (c.y + (int64_t)a.ny * c.z));
             }
         }
-        // every particle has read the nodes, and its position is known
-        if (coupled && !bar.wait()) return;
+        if (live && lane < 8) {
+            const T tx = Fx * a.neg_scale_dt, ty = Fy * a.neg_scale_dt, tz = Fz * a.neg_scale_dt;
+            P::add_transfer(to, P::to_fix_neg(delta, tx), P::to_fix_neg(delta, ty), P::to_fix_neg(delta, tz));
+        }
+        // all transfers are in and all positions known
+        if (coupled && (CONS || s + 1 < count) && !bar.meet()) return;
         if (CONS) {
             const typename P::real4 R = P::make_pos(fx, fy, fz, 0);
             T g = T(0), dx = T(0), dy = T(0), dz = T(0);
@@ -484,12 +492,6 @@ __global__ void __launch_bounds__(2 * PHASE_THREADS, sizeof(T) == 4 ? 2 : 1)
         } else {
             kick(Fx, Fy, Fz);
         }
-        if (live && lane < 8) {
-            const T tx = Fx * a.neg_scale_dt, ty = Fy * a.neg_scale_dt, tz = Fz * a.neg_scale_dt;
-            P::add_transfer(to, P::to_fix_neg(delta, tx), P::to_fix_neg(delta, ty), P::to_fix_neg(delta, tz));
-        }
-        // all transfers are in, and the other positions have been read
-        if (coupled && s + 1 < count && !bar.wait()) return;
     }
     bar.finish();
     if (!live || lane != 0) return;

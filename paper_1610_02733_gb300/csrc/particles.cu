@@ -797,7 +797,7 @@ __global__ void __launch_bounds__(REORDER_THREADS)
     for (int64_t b = start; b < a.np; b += stride)
         count_particle<T>(a.pos_in, b + tid, a.np, a.fnx, row_count, a.rank, ccw, W);
     if (blockIdx.x == 0 && tid == 0) *lb_missed = 0;
-    if (!bar.wait()) return;
+    if (!bar.meet()) return;
     const int r0 = min(n_rows, (int)blockIdx.x * per), r1 = min(n_rows, r0 + per), r = r0 + tid;
     int32_t before = block_sum_before(row_count, r0);
     const int32_t first = before + block_exclusive_scan(r < r1 ? __ldcg(row_count + r) : 0, nullptr);
@@ -810,7 +810,7 @@ __global__ void __launch_bounds__(REORDER_THREADS)
         const int cnt = active_row<true>(ccw, nx, fny, nz, W, L, occw, nrow, lane % L, valid);
         if (valid && lane % L == 0) active_count[nrow] = cnt;
     }
-    if (!bar.wait()) return;
+    if (!bar.meet()) return;
     before = block_sum_before(active_count, r0);
     const int32_t mine = r < r1 ? __ldcg(active_count + r) : 0;
     __shared__ int32_t s_base[REORDER_THREADS];
