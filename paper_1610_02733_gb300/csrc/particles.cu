@@ -290,10 +290,6 @@ __global__ void __launch_bounds__(32 * GATHER_WARPS) spread_rows_kernel(PArgs<T>
     }
 }
 
-// Variant B: the migrants of this MD step, spread with atomics once the row
-// gather is done (spread_particle_atomic, particle_step.cuh).  With `all`,
-// every particle is spread this way and the row gather does not run
-// (LBMD_SPREAD_ATOMIC).
 // Every particle's transfers with atomics (LBMD_SPREAD_ATOMIC), FP32: one thread
 // per corner -- 8 times the threads for a kernel whose threads each wait on
 // their loads and then queue 16 atomics (7 -> 4.5 us at 53,000 particles).  FP64,
@@ -305,6 +301,10 @@ __global__ void __launch_bounds__(256) spread_all_kernel(PArgs<T> a) {
     if (t < 2) a.migrant_count[t] = 0;  // the row gather's lists are not in use
     if ((t >> 3) < a.np) spread_corner_atomic(a, t >> 3, (int)t & 7);
 }
+// The migrants of this MD step, spread with atomics once the row gather is done
+// (particle_step.cuh); in FP32 with a thread per corner (256^3 nodes, 10^6
+// particles: the cycle 1670 -> 1655 us).  With `all` (FP64) every particle is
+// spread this way and the row gather does not run (LBMD_SPREAD_ATOMIC).
 template <typename T>
 __global__ void __launch_bounds__(256) migrant_spread_kernel(PArgs<T> a, int all) {
     using P = Prec<T>;
