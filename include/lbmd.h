@@ -296,7 +296,7 @@ lbmd_status lbmd_observables(lbmd_ctx *ctx, lbmd_observables_t *out);
  * Errors: LBMD_ERR_ARG for polls < -1. */
 lbmd_status lbmd_set_moments_wait(lbmd_ctx *ctx, int32_t polls);
 
-/* Rows (collide blocks of up to 256 nodes) whose fused moments timed out and
+/* Rows (pieces of 256, 128, 64 or 32 nodes, the largest that nx fills) whose fused moments timed out and
  * were computed by the follow-up kernel, summed over every LB step since
  * creation (synchronising). */
 lbmd_status lbmd_moments_fallback_rows(lbmd_ctx *ctx, int64_t *rows);

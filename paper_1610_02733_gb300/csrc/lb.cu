@@ -382,14 +382,14 @@ __global__ void __launch_bounds__(256, (collide_min_blocks<T, S, RELAX_FULL, GAU
 
 // The moments the collide kernel left: node rows of plane 0 and of the last
 // FUSE_LAG planes, and the rows whose wait ran out (counted into
-// missed_total); then the LB step counter advances.
+// missed_total, `pieces` for a block); then the LB step counter advances.
 template <typename T, typename S>
 __global__ void __launch_bounds__(256)
     moments_rest_kernel(const S *__restrict__ f, typename Prec<T>::node4 *node, const uint2 *occw,
                         typename Prec<T>::node4 *cact, typename Prec<T>::node4 *cact2, int occ_words, int64_t N,
                         int nx, int ny, int nz, T rho_base, T fs, int e, int32_t *range_flag, const int32_t *missed,
                         const int32_t *missed_list,
-                        unsigned long long *missed_total, unsigned long long *lb_step) {
+                        unsigned long long *missed_total, int pieces, unsigned long long *lb_step) {
     const int gx = (nx + (int)blockDim.x - 1) / (int)blockDim.x;
     const int rows = gx * ny;
     // boundary planes: 0 and max(1, nz - FUSE_LAG) .. nz - 1
@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(256)
                                   t);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        *missed_total += (unsigned long long)*missed;
+        *missed_total += (unsigned long long)*missed * (unsigned)pieces;
         *lb_step += 1ull;
     }
 }
@@ -437,9 +437,14 @@ __global__ void init_equilibrium_kernel(S *f, int64_t N, T rho0) {
     for (int i = 0; i < Q; ++i) PopStore<S, T>::store(f + (int64_t)i * N + r, T(WEIGHT(i)) * rho0, T(WEIGHT(i)) * rho0);
 }
 
-// Node kernels run one thread per node on a (x-blocks, ny, nz) grid.
+// Node kernels run one thread per node on a (x-blocks, ny, nz) grid: a row of up
+// to 256 nodes is one block, rounded up to a power of two.  Two blocks of half
+// that have as many threads, and twice the flags to set and to wait for: two
+// cycles at 96 x 80 x 112 nodes (51,200 particles, variant C, m = 5) 249.6 us
+// with blocks of 64, 239.6 with 128; 250 x 201 x 181 (545,000, variant A) 1153.6
+// with 128, 1150.3 with 256.
 static dim3 node_block(const lbmd_ctx *ctx) {
-    const int bx = ctx->p.nx >= 256 ? 256 : (ctx->p.nx >= 128 ? 128 : (ctx->p.nx >= 64 ? 64 : 32));
+    const int bx = ctx->p.nx > 128 ? 256 : (ctx->p.nx > 64 ? 128 : (ctx->p.nx > 32 ? 64 : 32));
     return dim3(bx, 1, 1);
 }
 static dim3 node_grid(const lbmd_ctx *ctx, dim3 block) {
@@ -510,11 +515,15 @@ static cudaError_t lb_step_t(lbmd_ctx *ctx) {
     else
         launch_collide<T, S, false>(ctx, a, grid, block);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    // the moments the collide kernel left, on the new populations
+    // the moments the collide kernel left, on the new populations (the count of
+    // missed rows is in pieces of 256, 128, 64 or 32 nodes, the largest that nx fills)
+    const int piece = ctx->p.nx >= 256 ? 256 : ctx->p.nx >= 128 ? 128 : ctx->p.nx >= 64 ? 64 : 32;
+    const int pieces = (ctx->p.nx + piece - 1) / piece / (int)grid.x;
     moments_rest_kernel<T, S><<<2 * ctx->sm_count, block, 0, ctx->stream>>>(
         a.fout, a.node, a.occw_new, a.cact_new, a.cact_new2, a.occ_words, ctx->N, ctx->p.nx, ctx->p.ny, ctx->p.nz,
         a.rho_base,
-        a.fs, ctx->fix.e, ctx->range_flag, ctx->lb_missed, ctx->missed_list, ctx->missed_total, ctx->d_lb_step);
+        a.fs, ctx->fix.e, ctx->range_flag, ctx->lb_missed, ctx->missed_list, ctx->missed_total, pieces,
+        ctx->d_lb_step);
     return cudaGetLastError();
 }
 

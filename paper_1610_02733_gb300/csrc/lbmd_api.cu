@@ -192,9 +192,8 @@ lbmd_status lbmd_create(const lbmd_params *p, lbmd_ctx **out) {
     // the tiled MD step's tables and buffers, where the lattice suits it and
     // the spread mode asks for it
     const size_t table_bytes = md_tile_geometry(ctx) && p->spread == LBMD_SPREAD_TILES ? md_tile_table_bytes(ctx) : 0;
-    // blocks of the LB collide (node kernels: rows of up to 256 nodes)
-    const int bx = p->nx >= 256 ? 256 : (p->nx >= 128 ? 128 : (p->nx >= 64 ? 64 : 32));
-    const int64_t n_lb_blocks = (int64_t)((p->nx + bx - 1) / bx) * p->ny * p->nz;
+    // blocks of the LB collide: rows of up to 256 nodes
+    const int64_t n_lb_blocks = (int64_t)((p->nx + 255) / 256) * p->ny * p->nz;
 
     struct Alloc {
         void **ptr;
