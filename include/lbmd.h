@@ -201,8 +201,9 @@ lbmd_status lbmd_add_particles(lbmd_ctx *ctx, int64_t n, const double *pos, cons
 
 /* Append nb harmonic bonds U = (k/2)(|r| - r0)^2 between particle ids
  * pairs[2b], pairs[2b+1] (host array of 2 nb int64, ids must exist; each
- * particle may take part in at most 8 bonds).  Conservative force of Eq. (4),
- * synchronising.  Errors: LBMD_ERR_CAPACITY, LBMD_ERR_ARG. */
+ * particle may take part in at most 8 bonds; k and r0 any finite numbers).
+ * Conservative force of Eq. (4), synchronising.  Errors: LBMD_ERR_CAPACITY,
+ * LBMD_ERR_ARG. */
 lbmd_status lbmd_add_bonds(lbmd_ctx *ctx, int64_t nb, const int64_t *pairs, double k, double r0);
 
 /* Kinds of bonds (per bond, fixed when it is added). */

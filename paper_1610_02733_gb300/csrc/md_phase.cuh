@@ -196,7 +196,9 @@ __device__ __forceinline__ Separation<T> bond_separation(const PArgs<T> &a, cons
 //   FENE     U = -(k/2) R0^2 ln(1 - (r/R0)^2)  g = k / (1 - (r/R0)^2), R0 = r0
 // (Kremer-Grest springs, Sec. 4); a FENE bond at r >= R0 gives NaN.  The
 // harmonic one, stiff and near r0, takes r - r0 = (r^2 - r0^2) / (r + r0) with the
-// squares' and sums' rounding errors carried along.
+// squares' and sums' rounding errors carried along -- for r0 > 0, where r + r0
+// does not cancel, and while r0^2 stays in FP32's range; elsewhere r - r0 as it
+// stands, which does not cancel there (r is at most a few thousand).
 template <typename T>
 __device__ __forceinline__ T bond_gain(uint8_t kind, T k, T r0, const Separation<T> &d) {
     const T px = d.x * d.x, py = d.y * d.y, pz = d.z * d.z;
@@ -204,13 +206,14 @@ __device__ __forceinline__ T bond_gain(uint8_t kind, T k, T r0, const Separation
         const T x = fma(d.z, d.z, fma(d.y, d.y, px)) / (r0 * r0);
         return x < T(1) ? k / (T(1) - x) : quiet_nan<T>();
     }
+    const T r = sqrt(fma(d.z, d.z, fma(d.y, d.y, px)));
+    if (!(r0 > T(0x1p-40) && r0 < T(0x1p40))) return r > T(0) ? k * (r - r0) / r : T(0);
     const T p0 = r0 * r0;
     T e1, e2, e3;
     const T s = two_sum(two_sum(two_sum(px, -p0, e1), py, e2), pz, e3);
     const T small = fma(T(2) * d.x, d.lx, fma(T(2) * d.y, d.ly, (T(2) * d.z) * d.lz));
     const T squares = (fma(d.x, d.x, -px) + fma(d.y, d.y, -py)) + (fma(d.z, d.z, -pz) - fma(r0, r0, -p0));
     const T e = s + ((((e1 + e2) + e3) + squares) + small);  // r^2 - r0^2
-    const T r = sqrt(fma(d.z, d.z, fma(d.y, d.y, px)));
     return r > T(0) ? k * e / (r * (r + r0)) : T(0);
 }
 
