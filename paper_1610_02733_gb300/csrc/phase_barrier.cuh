@@ -24,6 +24,8 @@ template <bool CLUSTER>
 struct PhaseBarrier {
     GridBarrier g;
     uint32_t target = 0;
+    // (The cluster instructions without .aligned: lanes that took different
+    // branches just before need not have met again.)
     // The block's accesses so far are done, as far as the blocks that pass the
     // wait can see.  Work between the two hides a part of the barrier: two cycles
     // of 2,560 beads with Lennard-Jones forces 280 -> 275 us, a gradient of 200 MD
@@ -32,7 +34,7 @@ struct PhaseBarrier {
         if (gridDim.x == 1) {
             __syncthreads();
         } else if (CLUSTER) {
-            asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+            asm volatile("barrier.cluster.arrive.release;" ::: "memory");
         } else {
             target += gridDim.x;
             __syncthreads();
@@ -42,7 +44,7 @@ struct PhaseBarrier {
     __device__ __forceinline__ bool wait() {
         if (gridDim.x == 1) return true;
         if (CLUSTER) {
-            asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+            asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
             return true;
         }
         bool ok = true;
