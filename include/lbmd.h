@@ -297,6 +297,18 @@ lbmd_status lbmd_observables(lbmd_ctx *ctx, lbmd_observables_t *out);
  * Errors: LBMD_ERR_ARG for polls < -1. */
 lbmd_status lbmd_set_moments_wait(lbmd_ctx *ctx, int32_t polls);
 
+/* Where the blocks of one launch wait for one another (the MD steps of a cycle
+ * and the re-ordering of small and middle systems in one launch each), a
+ * block waits at most `polls` polls.  They take microseconds; the default limit
+ * (polls = -1, 2^22 polls) is seconds, and is reached only if the blocks of a
+ * launch do not run together.  Then the launch ends, the context's state is
+ * invalid for good, and md_substep, lb_step, run_cycles, get_particles_device,
+ * synchronize and the synchronising accessors return LBMD_ERR_CUDA once the
+ * failure is known (destroy the context).  polls = 0 makes every such wait
+ * give up: it exists to exercise the report.  (Up to 16 blocks wait in hardware,
+ * without a limit.)  Errors: LBMD_ERR_ARG for polls < -1. */
+lbmd_status lbmd_set_barrier_wait(lbmd_ctx *ctx, int32_t polls);
+
 /* Rows (pieces of 256, 128, 64 or 32 nodes, the largest that nx fills) whose fused moments timed out and
  * were computed by the follow-up kernel, summed over every LB step since
  * creation (synchronising). */
@@ -557,6 +569,9 @@ lbmd_status lbmd_adjoint_forward(lbmd_adjoint *a, double zeta, const double *pos
 /* dL/dzeta and dL/dR0 (host array of 3 N_p doubles) of the last forward pass;
  * LBMD_ERR_SEQUENCE before any forward pass.  Synchronising. */
 lbmd_status lbmd_adjoint_backward(lbmd_adjoint *a, double *dloss_dzeta, double *dloss_dpos0);
+/* As lbmd_set_barrier_wait, for the launches of the two passes.  A pass whose
+ * wait gave up returns LBMD_ERR_CUDA; the next forward pass starts over. */
+lbmd_status lbmd_adjoint_set_barrier_wait(lbmd_adjoint *a, int32_t polls);
 const char *lbmd_adjoint_last_error(lbmd_adjoint *a);
 
 /* The cudaStream_t the context enqueues on. */

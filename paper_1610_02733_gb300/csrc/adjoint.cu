@@ -639,6 +639,7 @@ struct lbmd_adjoint {
     double *staging = nullptr;               // host-conversion scratch, 8 K m np doubles or more
     int64_t staging_len = 0;
     uint32_t *phase_words = nullptr;         // grid barrier of the phases (2 words), then its error flag
+    int barrier_polls = LBMD_DEFAULT_BARRIER_POLLS;  // limit of its waits
     int64_t phase_threads = 0;               // threads of a phase resident at once
     int phase_cluster = 1;                   // largest cluster of its blocks
     std::string err;
@@ -741,6 +742,10 @@ bool in_phases(const lbmd_adjoint *ad) {
     return ad->p.n_particles > 0 && 8ll * ad->p.n_particles <= ad->phase_threads;
 }
 
+GridBarrier phase_barrier(const lbmd_adjoint *ad) {
+    return GridBarrier{ad->phase_words, reinterpret_cast<int32_t *>(ad->phase_words + 2), nullptr, ad->barrier_polls};
+}
+
 template <typename T>
 cudaError_t launch_ad(const lbmd_adjoint *ad, const void *cluster_kernel, const void *grid_kernel, void **args) {
     return launch_phase(cluster_kernel, grid_kernel, nb(8ll * ad->p.n_particles, AD_THREADS), AD_THREADS,
@@ -785,7 +790,7 @@ cudaError_t run_md(lbmd_adjoint *ad, int c, bool record) {
         N4 *node = static_cast<N4 *>(ad->node);
         T *drag = static_cast<T *>(ad->drag) + (size_t)c * m * np;
         uint32_t step0 = (uint32_t)(c * m);
-        GridBarrier words{ad->phase_words, reinterpret_cast<int32_t *>(ad->phase_words + 2)};
+        GridBarrier words = phase_barrier(ad);
         void *args[] = {&args_a, &pos_in, &vel_in, &pos_out, &vel_out, &node, &drag, &rec, &step0, &words};
         return launch_ad<T>(ad, (const void *)ad_md_phase<T, true>, (const void *)ad_md_phase<T, false>, args);
     }
@@ -811,13 +816,16 @@ cudaError_t run_md(lbmd_adjoint *ad, int c, bool record) {
 }
 
 // A wait of a phase that gave up (see PhaseBarrier) since the last check;
-// synchronises.
+// synchronises.  The words and the flag start over: lbmd_adjoint_forward
+// recomputes everything from its arguments.
 cudaError_t check_phases(lbmd_adjoint *ad) {
     int32_t gave_up = 0;
     cudaError_t e = cudaMemcpyAsync(&gave_up, ad->phase_words + 2, sizeof(gave_up), cudaMemcpyDeviceToHost, ad->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ad->stream);
-    if (e == cudaSuccess && gave_up) e = cudaErrorLaunchTimeout;
-    return e;
+    if (e != cudaSuccess || !gave_up) return e;
+    e = cudaMemsetAsync(ad->phase_words, 0, 3 * sizeof(uint32_t), ad->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ad->stream);
+    return e != cudaSuccess ? e : cudaErrorLaunchTimeout;
 }
 
 template <typename T>
@@ -900,7 +908,7 @@ cudaError_t backward_t(lbmd_adjoint *ad, double *dzeta, double *dpos) {
             R4 *nbar = static_cast<R4 *>(ad->nbar[o]), *Rbar = static_cast<R4 *>(ad->Rbar),
                *vbar = static_cast<R4 *>(ad->vbar);
             T *zb = static_cast<T *>(ad->zbar) + (size_t)c * m * np;
-            GridBarrier words{ad->phase_words, reinterpret_cast<int32_t *>(ad->phase_words + 2)};
+            GridBarrier words = phase_barrier(ad);
             void *args[] = {&args_a, &rec, &nbar, &Rbar, &vbar, &zb, &words};
             e = launch_ad<T>(ad, (const void *)ad_adjoint_phase<T, true>, (const void *)ad_adjoint_phase<T, false>, args);
             if (e != cudaSuccess) return e;
@@ -1013,6 +1021,9 @@ lbmd_status lbmd_adjoint_create(const lbmd_adjoint_params *p, lbmd_adjoint **out
         }
     }
     cudaError_t e = cudaMemsetAsync(a->phase_words, 0, 3 * sizeof(uint32_t), a->stream);
+    // cells in range wherever a phase that ended early has not written
+    if (e == cudaSuccess) e = cudaMemsetAsync(a->pchk, 0, (K + 1) * 2 * np * r4, a->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(a->rec, 0, m * np * 12 * r4, a->stream);
     if (e == cudaSuccess) e = p->precision == LBMD_FP64 ? setup_phases<double>(a) : setup_phases<float>(a);
     if (e != cudaSuccess) {
         free_ad(a);
@@ -1039,6 +1050,7 @@ lbmd_status lbmd_adjoint_forward(lbmd_adjoint *a, double zeta, const double *pos
     for (int64_t q = 0; q < 3 * (int64_t)a->p.n_particles; ++q)
         if (!ad_finite(pos0[q]) || !ad_finite(vel0[q])) return afail(a, LBMD_ERR_ARG, "non-finite particle data");
     a->zeta = zeta;
+    a->have_forward = false;  // until the checkpoints are those of this call
     cudaError_t e = a->p.precision == LBMD_FP64 ? forward_t<double>(a, pos0, vel0, loss)
                                                 : forward_t<float>(a, pos0, vel0, loss);
     if (e != cudaSuccess) return afail(a, LBMD_ERR_CUDA, std::string("adjoint forward: ") + cudaGetErrorString(e));
@@ -1052,7 +1064,17 @@ lbmd_status lbmd_adjoint_backward(lbmd_adjoint *a, double *dloss_dzeta, double *
     if (!a->have_forward) return afail(a, LBMD_ERR_SEQUENCE, "backward before forward");
     cudaError_t e = a->p.precision == LBMD_FP64 ? backward_t<double>(a, dloss_dzeta, dloss_dpos0)
                                                 : backward_t<float>(a, dloss_dzeta, dloss_dpos0);
-    if (e != cudaSuccess) return afail(a, LBMD_ERR_CUDA, std::string("adjoint backward: ") + cudaGetErrorString(e));
+    if (e != cudaSuccess) {
+        a->have_forward = false;  // it writes the checkpoints again
+        return afail(a, LBMD_ERR_CUDA, std::string("adjoint backward: ") + cudaGetErrorString(e));
+    }
+    return LBMD_OK;
+}
+
+lbmd_status lbmd_adjoint_set_barrier_wait(lbmd_adjoint *a, int32_t polls) {
+    if (!a) return LBMD_ERR_ARG;
+    if (polls < -1) return afail(a, LBMD_ERR_ARG, "polls must be >= -1");
+    a->barrier_polls = polls < 0 ? LBMD_DEFAULT_BARRIER_POLLS : polls;
     return LBMD_OK;
 }
 

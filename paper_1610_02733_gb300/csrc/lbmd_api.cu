@@ -33,6 +33,16 @@ lbmd_status cuda_fail(lbmd_ctx *ctx, cudaError_t e, const char *where) {
         if (e_ != cudaSuccess) return cuda_fail((ctx), e_, #call); \
     } while (0)
 
+lbmd_status wait_failed(lbmd_ctx *ctx) {
+    return fail(ctx, LBMD_ERR_CUDA, "a kernel's bounded wait (bulk copies or grid barrier) gave up: results are invalid");
+}
+// A kernel whose wait gave up leaves the context's state unfinished: told by the
+// calls that advance it, and by the accessors once they have synchronised.
+#define CHECK_WAITS(ctx)                                                                            \
+    do {                                                                                            \
+        if (*static_cast<volatile int32_t *>((ctx)->host_error)) return wait_failed(ctx);           \
+    } while (0)
+
 // bytes of one real of the node field and particle records (FP32 for the
 // reduced-precision population forms)
 size_t real_size(const lbmd_ctx *ctx) { return ctx->p.precision == LBMD_FP64 ? 8 : 4; }
@@ -68,6 +78,7 @@ void free_all(lbmd_ctx *ctx) {
     }
     if (ctx->obs_ready) cudaEventDestroy(ctx->obs_ready);
     if (ctx->obs_host) cudaFreeHost(ctx->obs_host);
+    if (ctx->host_error) cudaFreeHost(ctx->host_error);
     if (ctx->up_stream) cudaStreamDestroy(ctx->up_stream);
     if (ctx->down_stream) cudaStreamDestroy(ctx->down_stream);
     for (int i = 0; i < 16; ++i)
@@ -150,6 +161,7 @@ lbmd_status lbmd_create(const lbmd_params *p, lbmd_ctx **out) {
     ctx->dt = 1.0 / (double)p->n_sub;
     ctx->fix = fix;
     ctx->fuse_spin = LBMD_DEFAULT_FUSE_SPIN;
+    ctx->barrier_polls = LBMD_DEFAULT_BARRIER_POLLS;
     lb_coefficients(p->nu, p->nu_bulk, p->gamma_ghost, p->kT, ctx->co);
     for (int d = 0; d < 3; ++d) ctx->co.body_force[d] = p->body_force[d];
 
@@ -263,7 +275,8 @@ lbmd_status lbmd_create(const lbmd_params *p, lbmd_ctx **out) {
             return s;
         }
     }
-    cudaError_t e = cudaSuccess;
+    cudaError_t e = cudaHostAlloc((void **)&ctx->host_error, sizeof(int32_t), cudaHostAllocMapped);
+    if (e == cudaSuccess) *ctx->host_error = 0;
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_lb_step, 0, sizeof(unsigned long long), ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->missed_total, 0, sizeof(unsigned long long), ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->range_flag, 0, sizeof(int32_t), ctx->stream);
@@ -345,6 +358,8 @@ static lbmd_status ensure_nb_lists(lbmd_ctx *ctx) {
     ctx->nb_invalid = static_cast<int32_t *>(bufs[2]);
     ctx->nb_ref4 = bufs[3];
     ctx->nb_end = static_cast<uint8_t *>(bufs[4]);
+    // every entry a slot in range from the start, whatever a build leaves out
+    for (int k : {0, 1, 4}) CK(ctx, cudaMemsetAsync(bufs[k], 0, bytes[k], ctx->stream));
     return LBMD_OK;
 }
 
@@ -508,6 +523,7 @@ lbmd_status lbmd_set_particles(lbmd_ctx *ctx, const double *pos, const double *v
 lbmd_status lbmd_md_substep(lbmd_ctx *ctx) {
     LBMD_TRACE("lbmd_md_substep");
     if (!ctx) return LBMD_ERR_ARG;
+    CHECK_WAITS(ctx);
     if (ctx->sub_done >= ctx->p.n_sub) return fail(ctx, LBMD_ERR_SEQUENCE, "n_sub MD steps already done");
     CK(ctx, launch_md_steps(ctx, ctx->sub_done, 1));
     ctx->sub_done += 1;
@@ -518,6 +534,7 @@ lbmd_status lbmd_md_substep(lbmd_ctx *ctx) {
 lbmd_status lbmd_lb_step(lbmd_ctx *ctx) {
     LBMD_TRACE("lbmd_lb_step");
     if (!ctx) return LBMD_ERR_ARG;
+    CHECK_WAITS(ctx);
     if (ctx->sub_done != ctx->p.n_sub) return fail(ctx, LBMD_ERR_SEQUENCE, "LB step before n_sub MD steps");
     CK(ctx, launch_lb_step(ctx));
     ctx->sub_done = 0;
@@ -528,6 +545,7 @@ lbmd_status lbmd_lb_step(lbmd_ctx *ctx) {
 lbmd_status lbmd_run_cycles(lbmd_ctx *ctx, int64_t n) {
     LBMD_TRACE("lbmd_run_cycles");
     if (!ctx || n < 0) return LBMD_ERR_ARG;
+    CHECK_WAITS(ctx);
     if (ctx->sub_done != 0) return fail(ctx, LBMD_ERR_SEQUENCE, "run_cycles must start at a cycle boundary");
     for (int64_t c = 0; c < n; ++c) {
         // the launches of a cycle depend on the buffer state it starts from
@@ -584,7 +602,7 @@ lbmd_status lbmd_observables(lbmd_ctx *ctx, lbmd_observables_t *out) {
     CK(ctx, cudaMemcpyAsync(h, ctx->red_out, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
     CK(ctx, cudaStreamSynchronize(ctx->stream));
     if (h[9] != 0.0)
-        return fail(ctx, LBMD_ERR_CUDA, "a kernel's bounded wait (bulk copies or grid barrier) gave up: results are invalid");
+        return wait_failed(ctx);
     out->mass = h[0];
     for (int d = 0; d < 3; ++d) {
         out->p_fluid[d] = h[1 + d];
@@ -609,6 +627,17 @@ lbmd_status lbmd_set_moments_wait(lbmd_ctx *ctx, int32_t polls) {
     const int v = polls < 0 ? LBMD_DEFAULT_FUSE_SPIN : polls;
     if (v != ctx->fuse_spin) {
         ctx->fuse_spin = v;
+        drop_cycle_graphs(ctx);  // the captured launches carry the old limit
+    }
+    return LBMD_OK;
+}
+
+lbmd_status lbmd_set_barrier_wait(lbmd_ctx *ctx, int32_t polls) {
+    if (!ctx) return LBMD_ERR_ARG;
+    if (polls < -1) return fail(ctx, LBMD_ERR_ARG, "polls must be >= -1");
+    const int v = polls < 0 ? LBMD_DEFAULT_BARRIER_POLLS : polls;
+    if (v != ctx->barrier_polls) {
+        ctx->barrier_polls = v;
         drop_cycle_graphs(ctx);  // the captured launches carry the old limit
     }
     return LBMD_OK;
@@ -649,6 +678,7 @@ lbmd_status lbmd_get_populations(lbmd_ctx *ctx, double *out) {
         CK(ctx, cudaMemcpyAsync(out + s, ctx->staging, c * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
         CK(ctx, cudaStreamSynchronize(ctx->stream));
     }
+    CHECK_WAITS(ctx);
     return LBMD_OK;
 }
 
@@ -682,6 +712,7 @@ static lbmd_status node_out(lbmd_ctx *ctx, double *out, bool transfer) {
                                 ctx->stream));
         CK(ctx, cudaStreamSynchronize(ctx->stream));
     }
+    CHECK_WAITS(ctx);
     return LBMD_OK;
 }
 
@@ -708,6 +739,7 @@ lbmd_status lbmd_get_particles(lbmd_ctx *ctx, double *pos, double *vel) {
     if (pos) CK(ctx, cudaMemcpyAsync(pos, dpos, 3 * n * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     if (vel) CK(ctx, cudaMemcpyAsync(vel, dvel, 3 * n * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     CK(ctx, cudaStreamSynchronize(ctx->stream));
+    CHECK_WAITS(ctx);
     return LBMD_OK;
 }
 
@@ -750,7 +782,7 @@ lbmd_status finalise_observables(lbmd_ctx *ctx, int s) {
     out->lb_step = ctx->obs_lb[s];
     out->md_step = ctx->obs_md[s];
     if (h[9] != 0.0)
-        return fail(ctx, LBMD_ERR_CUDA, "a kernel's bounded wait (bulk copies or grid barrier) gave up: results are invalid");
+        return wait_failed(ctx);
     for (int c = 0; c < 8; ++c)
         if (!is_finite_d(h[c])) return fail(ctx, LBMD_ERR_NONFINITE, "non-finite observable");
     if (h[8] != 0.0)
@@ -840,7 +872,10 @@ lbmd_status lbmd_synchronize(lbmd_ctx *ctx) {
     LBMD_TRACE("lbmd_synchronize");
     if (!ctx) return LBMD_ERR_ARG;
     CK(ctx, cudaStreamSynchronize(ctx->stream));
-    if (!ctx->async_ready) return LBMD_OK;
+    if (!ctx->async_ready) {
+        CHECK_WAITS(ctx);
+        return LBMD_OK;
+    }
     CK(ctx, cudaStreamSynchronize(ctx->up_stream));
     CK(ctx, cudaStreamSynchronize(ctx->down_stream));
     lbmd_status st = LBMD_OK;
@@ -850,11 +885,13 @@ lbmd_status lbmd_synchronize(lbmd_ctx *ctx) {
         const lbmd_status r = finalise_observables(ctx, s);
         if (st == LBMD_OK) st = r;
     }
+    CHECK_WAITS(ctx);
     return st;
 }
 
 lbmd_status lbmd_get_particles_device(lbmd_ctx *ctx, double *pos, double *vel) {
     if (!ctx) return LBMD_ERR_ARG;
+    CHECK_WAITS(ctx);
     CK(ctx, launch_particles_to_double(ctx, pos, vel));
     return LBMD_OK;
 }
@@ -956,6 +993,7 @@ lbmd_status lbmd_save_state(lbmd_ctx *ctx, void *buf, int64_t bytes) {
     const int b = ctx->pcur, M = LBMD_MAX_BONDS_PER_PARTICLE;
     const size_t rb = (size_t)ctx->np * 4 * real_size(ctx), np = (size_t)ctx->np;
     CK(ctx, cudaStreamSynchronize(ctx->stream));
+    CHECK_WAITS(ctx);
     CK(ctx, cudaMemcpy(o, ctx->f[ctx->cur], (size_t)19 * ctx->N * pop_size(ctx), cudaMemcpyDeviceToHost));
     o += L.pops;
     if (np) {

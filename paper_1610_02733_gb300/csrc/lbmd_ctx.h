@@ -154,6 +154,7 @@ struct lbmd_ctx {
     int fuse_spin;         // polls of a collide block's wait (0: no fused moments)
     int sm_count;
     uint32_t *phase_bar;    // grid barrier of the MD phase (arrivals, finished blocks)
+    int barrier_polls;      // limit of its waits
     int64_t phase_threads;  // threads of it resident at once
     int phase_cluster;      // largest cluster of its blocks
     bool in_buckets;        // the particles are where the last re-ordering bucketed them
@@ -179,7 +180,8 @@ struct lbmd_ctx {
     // range guard of the fixed-point momentum: set (sticky) by the kernels
     // that write a node record whose momentum reaches half the range
     int32_t *range_flag;
-    int32_t *dev_error;  // set by a kernel whose bounded wait gave up
+    int32_t *dev_error;   // set by a kernel whose bounded wait gave up
+    int32_t *host_error;  // the same in mapped host memory
     FixUnit fix;
     int red_blocks;
     unsigned long long *d_lb_step;  // LB step counter read by the kernels
@@ -249,6 +251,9 @@ inline void *vel_now(const lbmd_ctx *c) { return c->vel4[c->pv]; }
 // before it leaves its row's fused moments to the follow-up kernel (64 ns per
 // poll: about 67 ms, far above the few microseconds the lag needs).
 constexpr int LBMD_DEFAULT_FUSE_SPIN = 1 << 20;
+// Default poll limit of a grid barrier (phase_barrier.cuh): seconds, against the
+// microseconds a barrier takes.
+constexpr int LBMD_DEFAULT_BARRIER_POLLS = 1 << 22;
 
 // Deviation storage: the density of the stored rest values, sum_i b_i with
 // b_i = w_i rho0 formed in T as the kernels form it (0 for the plain forms,

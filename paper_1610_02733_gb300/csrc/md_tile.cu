@@ -231,7 +231,7 @@ struct TileArgs {
     int32_t *late_rows, *late_count;             // rows whose wait ran out (two lists by MD-step parity)
     int late_cap;
     int tiles_y, n_tiles;
-    int32_t *dev_error;  // set if a copy wait gave up
+    int32_t *dev_error, *host_error;  // set if a copy wait gave up
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -261,11 +261,13 @@ __device__ __forceinline__ void bulk_to_shared(void *dst, const void *src, uint3
 // Wait for phase `parity` of bar, at most TILE_SPIN polls; on a timeout the
 // error flag is set and the copies still in flight get a second bounded wait
 // before the block goes on (its results are then flagged invalid).
-__device__ __forceinline__ void mbar_wait(unsigned long long *bar, uint32_t parity, int32_t *dev_error) {
+__device__ __forceinline__ void mbar_wait(unsigned long long *bar, uint32_t parity, int32_t *dev_error,
+                                          int32_t *host_error) {
     int polls = 0;
     while (!mbar_try_wait(bar, parity)) {
         if (++polls > TILE_SPIN) {
             atomicOr(dev_error, 1);
+            *(volatile int32_t *)host_error = 1;
             for (int p2 = 0; p2 < TILE_SPIN && !mbar_try_wait(bar, parity); ++p2) {
             }
             return;
@@ -303,7 +305,8 @@ __device__ __forceinline__ int warp_excl_scan(int lane, int v, int &excl) {
 // the rows (arow) and the particle buckets (row_start).
 __global__ void __launch_bounds__(256) tile_table_kernel(const int32_t *arow, const int32_t *row_start, int ny,
                                                          int nz, int tiles_y, int n_tiles, int rec_cap, int acc_cap,
-                                                         TileTable *table) {
+                                                         TileTable *table, const int32_t *dev_error) {
+    if (*dev_error) return;  // the offsets may be those of two orderings
     const int lane = threadIdx.x & 31;
     const int T = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (T >= n_tiles) return;  // whole warps
@@ -442,6 +445,8 @@ __global__ void __launch_bounds__(TILE_THREADS, 3) md_tile_kernel(PArgs<T> a, Ti
     N4 *s_rec = reinterpret_cast<N4 *>(tile_smem);
     unsigned char *s_acc = tile_smem + (size_t)REC_CAP * sizeof(N4);
 
+    // after a wait that gave up, the tables need not fit the words and buckets
+    if (__syncthreads_or(threadIdx.x == 0 && *(volatile const int32_t *)t.dev_error != 0)) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tile = blockIdx.x;
     const TileGeo G(tile, t.tiles_y, a.ny, a.nz);
@@ -463,7 +468,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 3) md_tile_kernel(PArgs<T> a, Ti
             words[row][w] = a.occw[(size_t)g * a.occ_words + w];
         }
     }
-    if (tid == 0) mbar_wait(&mbar[0], 0u, t.dev_error);
+    if (tid == 0) mbar_wait(&mbar[0], 0u, t.dev_error, t.host_error);
     __syncthreads();
 
     // (2) the records (bulk copies), each thread's particle, the sums cleared
@@ -488,7 +493,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 3) md_tile_kernel(PArgs<T> a, Ti
             for (int k = lane; k < n; k += 32) t.cact_out[f + k] = a.cact[f + k];
         }
     }
-    if (staged && n_rec > 0 && tid == 0) mbar_wait(&mbar[1], 0u, t.dev_error);
+    if (staged && n_rec > 0 && tid == 0) mbar_wait(&mbar[1], 0u, t.dev_error, t.host_error);
     __syncthreads();
 
     // (3) the MD step of the tile's particles
@@ -611,7 +616,10 @@ __global__ void __launch_bounds__(TILE_THREADS, 3) md_tile_kernel(PArgs<T> a, Ti
             const int g = (G.y0 + (tb.bij[o] & 0xff)) + a.ny * (G.z0 + (tb.bij[o] >> 8));
             const int k = atomicAdd(t.late_count + a.mig_par, 1);
             if (k < t.late_cap) t.late_rows[(int64_t)a.mig_par * t.late_cap + k] = g;
-            else atomicOr(t.dev_error, 2);
+            else {
+                atomicOr(t.dev_error, 2);
+                *(volatile int32_t *)t.host_error = 1;
+            }
         }
         if (staged) {
             const int src = tb.osrc[o], a0 = tb.aoff[o];
@@ -639,6 +647,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) md_tile_finish_kernel(PArgs<T> a, TileArgs<T> t, const int32_t *arow,
                                                              int64_t edge_cap) {
     using Acc = TileAcc<T>;
+    if (*t.dev_error) return;
     const int par = a.mig_par;
     const int n_fix = a.nz + a.ny - 1;
     const int n_late = min(t.late_count[par], t.late_cap);
@@ -723,7 +732,7 @@ cudaError_t md_tile_build_table(lbmd_ctx *ctx, int set) {
         ctx->arow[set], ctx->row_start, ctx->p.ny, ctx->p.nz, tiles_y, n_tiles,
         f64 ? lbmd::TileCap<double>::REC : lbmd::TileCap<float>::REC,
         f64 ? lbmd::TileCap<double>::ACC : lbmd::TileCap<float>::ACC,
-        static_cast<lbmd::TileTable *>(ctx->tile_table[set]));
+        static_cast<lbmd::TileTable *>(ctx->tile_table[set]), ctx->dev_error);
     return cudaGetLastError();
 }
 
@@ -747,6 +756,7 @@ cudaError_t md_tile_step(lbmd_ctx *ctx, const lbmd::PArgs<T> &a) {
     t.tiles_y = (ctx->p.ny + lbmd::TILE_Y - 1) / lbmd::TILE_Y;
     t.n_tiles = md_tile_count(ctx);
     t.dev_error = ctx->dev_error;
+    t.host_error = ctx->host_error;
     lbmd::md_tile_kernel<T>
         <<<t.n_tiles, lbmd::TILE_THREADS, lbmd::tile_dyn_smem<T>(), ctx->stream>>>(a, t, ctx->cact_cap);
     cudaError_t e = cudaGetLastError();

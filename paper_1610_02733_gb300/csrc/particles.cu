@@ -204,10 +204,12 @@ __global__ void __launch_bounds__(32 * GATHER_WARPS) spread_rows_kernel(PArgs<T>
     const int ym = y == 0 ? a.ny - 1 : y - 1, zm = z == 0 ? a.nz - 1 : z - 1;
     const int c0 = y + a.ny * z, c1 = ym + a.ny * z, c2 = y + a.ny * zm, c3 = ym + a.ny * zm;
     const int lo0 = a.row_start[c0], lo1 = a.row_start[c1], lo2 = a.row_start[c2], lo3 = a.row_start[c3];
-    const int e1 = a.row_start[c0 + 1] - lo0;
-    const int e2 = e1 + a.row_start[c1 + 1] - lo1;
-    const int e3 = e2 + a.row_start[c2 + 1] - lo2;
-    const int total = e3 + a.row_start[c3 + 1] - lo3;
+    // (a re-ordering that the limit of a barrier ended may leave the starts of
+    // two orderings: no row's count is taken as negative)
+    const int e1 = max(a.row_start[c0 + 1] - lo0, 0);
+    const int e2 = e1 + max(a.row_start[c1 + 1] - lo1, 0);
+    const int e3 = e2 + max(a.row_start[c2 + 1] - lo2, 0);
+    const int total = e3 + max(a.row_start[c3 + 1] - lo3, 0);
     const uint2 *wrow = a.occw + (size_t)nrow * W;
     const int base = (int)wrow[0].y;
     for (int w = lane; w < W; w += 32) {
@@ -462,7 +464,7 @@ __global__ void __launch_bounds__(32 * NB_WARPS) nb_build_kernel(PArgs<T> a, T r
             const int ky = (r0 + lane) % ny_rows, kz = (r0 + lane) / ny_rows;
             const int row = (y0 + ky) % a.ny + a.ny * ((z0 + kz) % a.nz);
             lo = a.row_start[row];
-            cnt = a.row_start[row + 1] - lo;
+            cnt = max(a.row_start[row + 1] - lo, 0);  // (as in spread_rows_kernel)
         }
         int incl = cnt;
 #pragma unroll
@@ -763,7 +765,9 @@ __global__ void __launch_bounds__(1024) active_finalize_kernel(const int32_t *ro
 // the numbering of the nodes, between two grid barriers.  Block b takes the
 // rows [b per, (b + 1) per); for the scans it adds up the counts of all rows
 // before its own (at most 38,912 values out of L2).  row_count and ccw are zero
-// before and after.  As seven launches and two memsets the same took 23 us at
+// before and after -- unless the limit of a barrier ends the kernel: the counts
+// then stay as they are, and no later launch gets past its first barrier to use
+// them.  As seven launches and two memsets the same took 23 us at
 // 64^3 nodes, where each of them is a launch's latency; this takes 9.
 constexpr int REORDER_THREADS = 256;
 
@@ -1017,7 +1021,7 @@ static cudaError_t md_phase_t(lbmd_ctx *ctx, int substep, int count, bool *done)
         const int64_t threads = ctx->np * (cons == 2 ? 32 : 8);
         if (threads <= ctx->phase_threads) {
             PArgs<T> a = make_pargs<T>(ctx, substep);
-            GridBarrier words{ctx->phase_bar, ctx->dev_error};
+            GridBarrier words{ctx->phase_bar, ctx->dev_error, ctx->host_error, ctx->barrier_polls};
             void *args[] = {&a, &count, &words};
             // one block per SM if that takes at most twice the threads each
             const int per = threads > (int64_t)PHASE_THREADS * ctx->sm_count ? 2 * PHASE_THREADS : PHASE_THREADS;
@@ -1205,7 +1209,7 @@ static cudaError_t reorder_t(lbmd_ctx *ctx) {
     uint2 *occw = active_words_next(ctx);
     int32_t *arow = ctx->arow[(ctx->lb_step + 1) & 1];
     FastDiv fny = make_fastdiv((uint32_t)ctx->p.ny);
-    GridBarrier words{ctx->phase_bar, ctx->dev_error};
+    GridBarrier words{ctx->phase_bar, ctx->dev_error, ctx->host_error, ctx->barrier_polls};
     void *args[] = {&a,    &ctx->row_count, &ctx->active_count, &ctx->row_start, &ctx->ccw, &occw, &arow,
                     &ctx->lb_missed, &fny, &nz, &W, &L, &per, &words};
     const cudaError_t e = cudaLaunchCooperativeKernel((const void *)reorder_kernel<T>, dim3(blocks),

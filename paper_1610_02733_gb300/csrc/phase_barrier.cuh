@@ -14,12 +14,24 @@ namespace lbmd {
 // during the launch (1.2 us / 1.8 us at 128 blocks of 256 threads; a count that
 // the last block clears beside a generation word took 2.2 / 2.9 us).  The last
 // block to finish clears the word for the next launch.  The wait is bounded
-// (the blocks arrive within microseconds; 2^22 polls are seconds): a block that
-// gives up sets the context's device error flag, and the kernel ends.
+// (the blocks arrive within microseconds; the default limit is seconds): a
+// block that gives up sets the error flags and ends, and so does every block
+// that finds the flag set.  The words then keep counts that no launch can use,
+// so while the flag is set no wait is passed, in this launch or a later one,
+// until the owner clears the flag and the words.  What a kernel that ends there
+// has not written keeps its former values: the owner's buffers must be safe to
+// read in that state.
 struct GridBarrier {
-    uint32_t *word;  // arrivals, finished blocks
-    int32_t *error;
+    uint32_t *word;       // arrivals, finished blocks
+    int32_t *error;       // device memory
+    int32_t *host_error;  // the same in mapped host memory, or null
+    int polls;            // limit of a wait
 };
+__device__ __forceinline__ int32_t load_flag(const int32_t *p) {
+    int32_t v;
+    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 template <bool CLUSTER>
 struct PhaseBarrier {
     GridBarrier g;
@@ -49,16 +61,22 @@ struct PhaseBarrier {
         }
         bool ok = true;
         if (threadIdx.x == 0) {
+            // a flag of an earlier launch: at the first wait; of this launch: the
+            // block that set it arrives no more
+            int32_t failed = target == gridDim.x ? load_flag(g.error) : 0;
             for (int polls = 0;; ++polls) {
+                if (polls >= g.polls) {
+                    atomicExch(g.error, 1);
+                    if (g.host_error) *(volatile int32_t *)g.host_error = 1;
+                    failed = 1;
+                    break;
+                }
                 uint32_t v;
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(g.word) : "memory");
                 if ((int32_t)(v - target) >= 0) break;
-                if (polls > (1 << 22)) {
-                    atomicExch(g.error, 1);
-                    ok = false;
-                    break;
-                }
+                if ((polls & 1023) == 1023 && (failed = load_flag(g.error)) != 0) break;
             }
+            ok = failed == 0;
         }
         return __syncthreads_and(ok) != 0;
     }

@@ -47,13 +47,14 @@ EXPORTS = (
     "lbmd_get_particles_device", "lbmd_get_counts", "lbmd_stream", "lbmd_last_error", "lbmd_status_string",
     "lbmd_set_particles_async", "lbmd_get_particles_async", "lbmd_observables_async", "lbmd_synchronize",
     "lbmd_particle_sums_static", "lbmd_set_moments_wait", "lbmd_moments_fallback_rows", "lbmd_set_frozen_copy",
+    "lbmd_set_barrier_wait",
     "lbmd_batch_create", "lbmd_batch_destroy", "lbmd_batch_add_particles", "lbmd_batch_run", "lbmd_batch_kinetic",
     "lbmd_batch_kinetic_device",
     "lbmd_batch_unstable", "lbmd_batch_get_populations", "lbmd_batch_set_populations", "lbmd_batch_get_particles",
     "lbmd_batch_get_counts", "lbmd_batch_tuning", "lbmd_batch_set_lb_grid", "lbmd_batch_stream",
     "lbmd_batch_last_error", "lbmd_batch_set_schedule", "lbmd_batch_persistent_tuning",
     "lbmd_adjoint_create", "lbmd_adjoint_destroy", "lbmd_adjoint_forward", "lbmd_adjoint_backward",
-    "lbmd_adjoint_last_error",
+    "lbmd_adjoint_last_error", "lbmd_adjoint_set_barrier_wait",
 )
 
 
@@ -141,6 +142,7 @@ def load():
     L.lbmd_get_counts.argtypes = [P, i64p, i64p, i64p, i64p, ct.POINTER(ct.c_int32)]
     L.lbmd_particle_sums_static.argtypes = [ct.c_void_p, ct.c_void_p, ct.c_int64, ct.c_void_p, ct.c_void_p]
     L.lbmd_set_moments_wait.argtypes = [P, ct.c_int32]
+    L.lbmd_set_barrier_wait.argtypes = [P, ct.c_int32]
     L.lbmd_moments_fallback_rows.argtypes = [P, i64p]
     L.lbmd_set_frozen_copy.argtypes = [P, ct.c_int32]
     L.lbmd_stream.restype = ct.c_void_p
@@ -173,6 +175,7 @@ def load():
     L.lbmd_adjoint_destroy.argtypes = [P]
     L.lbmd_adjoint_forward.argtypes = [P, ct.c_double, P, P, dp]
     L.lbmd_adjoint_backward.argtypes = [P, dp, P]
+    L.lbmd_adjoint_set_barrier_wait.argtypes = [P, i32]
     L.lbmd_adjoint_last_error.restype = ct.c_char_p
     L.lbmd_adjoint_last_error.argtypes = [P]
     for name in EXPORTS:
@@ -473,6 +476,11 @@ class LBMD:
         every row to the follow-up kernel); results do not depend on it."""
         _check(self._h, load().lbmd_set_moments_wait(self._h, int(polls)), "lbmd_set_moments_wait")
 
+    def set_barrier_wait(self, polls: int):
+        """Poll limit of the waits between the blocks of one launch (-1:
+        default; 0: each gives up, which invalidates the context)."""
+        _check(self._h, load().lbmd_set_barrier_wait(self._h, int(polls)), "lbmd_set_barrier_wait")
+
     def set_frozen_copy(self, on: bool):
         """Variant A: read the frozen node velocities from a copy of the
         compact records (True) or the node field (False); same results.  Only
@@ -706,6 +714,11 @@ class Adjoint:
         dpos = np.zeros(3 * max(self.n_particles, 1))
         _acheck(self._h, load().lbmd_adjoint_backward(self._h, ct.byref(dz), _ptr(dpos)), "lbmd_adjoint_backward")
         return dz.value, dpos[:3 * self.n_particles].reshape(-1, 3)
+
+    def set_barrier_wait(self, polls: int):
+        """Poll limit of the waits between the blocks of one launch (-1:
+        default; 0: each gives up, and the pass raises)."""
+        _acheck(self._h, load().lbmd_adjoint_set_barrier_wait(self._h, int(polls)), "lbmd_adjoint_set_barrier_wait")
 
 
 def drag_function(adjoint: Adjoint, vel0):
