@@ -198,22 +198,33 @@ __device__ __forceinline__ Separation<T> bond_separation(const PArgs<T> &a, cons
 // harmonic one, stiff and near r0, takes r - r0 = (r^2 - r0^2) / (r + r0) with the
 // squares' and sums' rounding errors carried along -- for r0 > 0, where r + r0
 // does not cancel, and while r0^2 stays in FP32's range; elsewhere r - r0 as it
-// stands, which does not cancel there (r is at most a few thousand).
+// stands, which does not cancel there (r is at most a few thousand).  That choice
+// is made by bond_form, outside the MD steps of a phase (inside them it cost 0.6 %
+// of a cycle of 4,096 bonded particles).
+constexpr uint8_t BOND_HARMONIC_PLAIN = 2;
 template <typename T>
-__device__ __forceinline__ T bond_gain(uint8_t kind, T k, T r0, const Separation<T> &d) {
+__device__ __forceinline__ uint8_t bond_form(uint8_t kind, T r0) {
+    return kind == LBMD_BOND_HARMONIC && !(r0 > T(0x1p-40) && r0 < T(0x1p40)) ? BOND_HARMONIC_PLAIN : kind;
+}
+template <typename T>
+__device__ __forceinline__ T bond_gain(uint8_t form, T k, T r0, const Separation<T> &d) {
     const T px = d.x * d.x, py = d.y * d.y, pz = d.z * d.z;
-    if (kind == LBMD_BOND_FENE) {
-        const T x = fma(d.z, d.z, fma(d.y, d.y, px)) / (r0 * r0);
+    if (form != LBMD_BOND_HARMONIC) {
+        const T r2 = fma(d.z, d.z, fma(d.y, d.y, px));
+        if (form == BOND_HARMONIC_PLAIN) {
+            const T r = sqrt(r2);
+            return r > T(0) ? k * (r - r0) / r : T(0);
+        }
+        const T x = r2 / (r0 * r0);
         return x < T(1) ? k / (T(1) - x) : quiet_nan<T>();
     }
-    const T r = sqrt(fma(d.z, d.z, fma(d.y, d.y, px)));
-    if (!(r0 > T(0x1p-40) && r0 < T(0x1p40))) return r > T(0) ? k * (r - r0) / r : T(0);
     const T p0 = r0 * r0;
     T e1, e2, e3;
     const T s = two_sum(two_sum(two_sum(px, -p0, e1), py, e2), pz, e3);
     const T small = fma(T(2) * d.x, d.lx, fma(T(2) * d.y, d.ly, (T(2) * d.z) * d.lz));
     const T squares = (fma(d.x, d.x, -px) + fma(d.y, d.y, -py)) + (fma(d.z, d.z, -pz) - fma(r0, r0, -p0));
     const T e = s + ((((e1 + e2) + e3) + squares) + small);  // r^2 - r0^2
+    const T r = sqrt(fma(d.z, d.z, fma(d.y, d.y, px)));
     return r > T(0) ? k * e / (r * (r + r0)) : T(0);
 }
 
@@ -227,7 +238,7 @@ __device__ __forceinline__ void bond_forces(const PArgs<T> &a, int64_t id, const
     for (int b = 0; b < nbond; ++b) {
         const int64_t e = id * LBMD_MAX_BONDS_PER_PARTICLE + b;
         const Separation<T> d = bond_separation(a, R, c, a.slot_of[a.bond_partner[e]]);
-        const T g = bond_gain(a.bond_kind[e], (T)a.bond_k[e], (T)a.bond_r0[e], d);
+        const T r0 = (T)a.bond_r0[e], g = bond_gain(bond_form(a.bond_kind[e], r0), (T)a.bond_k[e], r0, d);
         Fx = fma(g, d.x, Fx);
         Fy = fma(g, d.y, Fy);
         Fz = fma(g, d.z, Fz);
@@ -378,7 +389,7 @@ __global__ void __launch_bounds__(2 * PHASE_THREADS, sizeof(T) == 4 ? 2 : 1)
     }
     int32_t partner = -1;
     T bond_k = T(0), bond_r0 = T(0);
-    uint8_t kind = 0;
+    uint8_t form = 0;
     int nbond = 0;
     if (CONS) {
         const typename P::real4 B = a.fcons4[p];
@@ -391,7 +402,7 @@ __global__ void __launch_bounds__(2 * PHASE_THREADS, sizeof(T) == 4 ? 2 : 1)
             partner = a.slot_of[a.bond_partner[e]];
             bond_k = (T)a.bond_k[e];
             bond_r0 = (T)a.bond_r0[e];
-            kind = a.bond_kind[e];
+            form = bond_form(a.bond_kind[e], bond_r0);
         }
     }
     // ideal particles of variant A wait for nobody
@@ -462,7 +473,7 @@ __global__ void __launch_bounds__(2 * PHASE_THREADS, sizeof(T) == 4 ? 2 : 1)
                 dx = d.x;
                 dy = d.y;
                 dz = d.z;
-                g = bond_gain(kind, bond_k, bond_r0, d);
+                g = bond_gain(form, bond_k, bond_r0, d);
             }
             Bx = By = Bz = T(0);
             if (CONS == 1) {

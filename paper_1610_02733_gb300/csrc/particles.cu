@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(PAIR_THREADS) pair_kick_kernel(PArgs<T> a) {
     if (lane < a.bond_count[i]) {
         const int64_t e = i * LBMD_MAX_BONDS_PER_PARTICLE + lane;
         const Separation<T> d = bond_separation(a, R, c, a.slot_of[a.bond_partner[e]]);
-        const T g = bond_gain(a.bond_kind[e], (T)a.bond_k[e], (T)a.bond_r0[e], d);
+        const T r0 = (T)a.bond_r0[e], g = bond_gain(bond_form(a.bond_kind[e], r0), (T)a.bond_k[e], r0, d);
         Fx = fma(g, d.x, Fx);
         Fy = fma(g, d.y, Fy);
         Fz = fma(g, d.z, Fz);
