@@ -251,10 +251,9 @@ __device__ __forceinline__ void collide_push_node(const LbArgs<T, S> &a, int x, 
     for (int i = 0; i < Q; ++i) f[i] = St::arith(a.fin + (size_t)i * a.N + r);
     if constexpr (sizeof(T) == 8) {
         typename P::fix J[3];
-        bool done = RELAX_FULL && a.fx.usable && in_fixed_range(f, a.fx.e);
+        FixedMoments o;
+        bool done = RELAX_FULL && a.fx.usable && fixed_moments_in_range(f, a.fx.e, o);
         if (RELAX_FULL && done) {
-            FixedMoments o;
-            fixed_moments(f, a.fx.e, o);
             node_transfer<C>(a, r, x, y, z, record_momentum(o.j[0]), record_momentum(o.j[1]), record_momentum(o.j[2]),
                              J);
             const FluidNoise<GAUSS> noise(a, r, (uint32_t)step);
