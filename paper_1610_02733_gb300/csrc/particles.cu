@@ -1018,13 +1018,21 @@ static cudaError_t md_phase_t(lbmd_ctx *ctx, int substep, int count, bool *done)
         (ctx->p.variant != LBMD_VARIANT_A || has_cons(ctx) || team_a)) {
         const bool half = ctx->p.integrator == LBMD_INTEGRATOR_HALF_STEP;
         const int cons = ctx->lj_rc > 0.0 ? 2 : has_cons(ctx) ? 1 : 0;
-        const int64_t threads = ctx->np * (cons == 2 ? 32 : 8);
-        if (threads <= ctx->phase_threads) {
+        const int64_t threads = ctx->np * (cons == 2 ? 32 : 8), one_block = (int64_t)PHASE_THREADS * ctx->sm_count;
+        // Up to that many particles the teams are the faster, m = 10, us a cycle
+        // with them / with the separate kernels: FP32 64^3 ideal 19,400 particles
+        // 75.9 / 87.3, bonded 96.2 / 121.2; 4,800 Lennard-Jones beads 132 / 147;
+        // FP64 ideal 9,600 204 / 245.  FP64 with conservative forces only up to one
+        // block of the smaller size per SM (the larger ones put twice the FP64 work
+        // on half as many SMs): bonded 4,864 particles 282 / 350, 4,900 443 / 350
+        // (m = 2: 134 / 145, 166 / 146); 1,216 beads 342 / 390, 1,248 548 / 495,
+        // 2,400 570 / 557.
+        if (threads <= (sizeof(T) == 8 && cons ? std::min(one_block, ctx->phase_threads) : ctx->phase_threads)) {
             PArgs<T> a = make_pargs<T>(ctx, substep);
             GridBarrier words{ctx->phase_bar, ctx->dev_error, ctx->host_error, ctx->barrier_polls};
             void *args[] = {&a, &count, &words};
             // one block per SM if that takes at most twice the threads each
-            const int per = threads > (int64_t)PHASE_THREADS * ctx->sm_count ? 2 * PHASE_THREADS : PHASE_THREADS;
+            const int per = threads > one_block ? 2 * PHASE_THREADS : PHASE_THREADS;
             return launch_phase(phase_kernel<T, true>(half, cons), phase_kernel<T, false>(half, cons),
                                 (unsigned)((threads + per - 1) / per), per, ctx->phase_cluster, args, ctx->stream);
         }

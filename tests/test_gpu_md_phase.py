@@ -76,3 +76,20 @@ def test_coupled_phase_with_bonds(precision, integrator, variant):
         g.close()
     _same(out[1], out[0])
     _same(out[2], out[0])
+
+
+@pytest.mark.parametrize("n", [4864, 4900])
+def test_fp64_bonds_at_the_limit_of_the_teams(n):
+    # 8 lanes a particle, one block of 256 per SM: both sides of the line on 152 SMs
+    shape, m, out = (20, 19, 18), 2, []
+    for spread, steps in (("rows", "ee"), ("auto", "gg"), ("auto", "eg")):
+        g = lbmd.LBMD(*shape, kT=1e-3, zeta=1.0, seed=11, max_particles=n, max_bonds=n, precision="fp64", n_sub=m,
+                      spread=spread)
+        g.add_particles(inputs.uniform_positions(n, shape, 6), inputs.maxwell_velocities(n, 1e-3, 6))
+        g.add_bonds([(i, i + 1) for i in range(0, n - 1, 2)], 1e-3, 1.0)
+        for s in steps:
+            g.run_cycles(1) if s == "g" else g.cycle(1)
+        out.append((g.populations(), g.node_field(), *g.particles()))
+        g.close()
+    _same(out[1], out[0])
+    _same(out[2], out[0])
