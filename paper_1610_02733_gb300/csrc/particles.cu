@@ -1198,11 +1198,14 @@ static cudaError_t active_set_t(lbmd_ctx *ctx) {
 }
 
 // Re-ordering and active set of the coming cycle in one launch (reorder_kernel),
-// while a thread of the grid takes at most one row and 8 particles; larger
-// systems take the separate kernels, which fill the GPU.
+// while a thread of the grid takes at most one row and 4 particles; larger
+// systems take the separate kernels, which fill the GPU.  64 x 196 x 196 nodes (38,416
+// rows), m = 2, us a cycle in one launch / separately, FP32: 1,000 particles
+// 137 / 141, 100,000 161 / 163, 200,000 184 / 183, 300,000 204 / 200 (FP64 676 / 678,
+// 745 / 746, 812 / 806, 879 / 873); 96 x 128 x 128, 150,000: 136 / 140 (575 / 578).
 static bool reorder_fits(const lbmd_ctx *ctx) {
     const int64_t threads = (int64_t)ctx->sm_count * REORDER_THREADS;
-    return ctx->np > 0 && (int64_t)ctx->p.ny * ctx->p.nz <= threads && ctx->np <= 8 * threads;
+    return ctx->np > 0 && (int64_t)ctx->p.ny * ctx->p.nz <= threads && ctx->np <= 4 * threads;
 }
 template <typename T>
 static cudaError_t reorder_t(lbmd_ctx *ctx) {
