@@ -54,6 +54,27 @@ struct PArgs {
     int64_t np_cap;
 };
 
+// FP64 quotient a / b in 6 operations of the FP64 pipe: Goldschmidt's division
+// (R. E. Goldschmidt, Applications of Division by Convergence, MIT 1964), which
+// multiplies numerator and denominator by what takes the denominator to one.
+// With y an approximation of 1/b, b y = 1 - h, the factors y and 1 + h + h^2 leave
+// 1 - h^3: the numerator a y (1 + h + h^2) is the quotient to within |h|^3 and two
+// roundings (|h| below 2^-19: 2^-52 of it, at most two units of the last place).
+// Markstein's correction (P. W. Markstein, IBM J. Res. Dev. 34 (1990) 111) adds the
+// residual a - b q, which a fused multiply-add forms exactly, times y, which is
+// off by |h|: the error is half a unit of the last place and 2^-18 of one, so the
+// result is the IEEE quotient or its neighbour.  For b and a / b in the normal
+// range, far from its ends; 0 / b = 0.  (Measured: |h| below 2^-19.9, and 2^20 of
+// 2^20 quotients the IEEE ones.)
+__device__ __forceinline__ double quotient(double a, double b) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+    const double h = fma(-b, y, 1.0), q0 = a * y;
+    const double q = fma(q0, fma(h, h, h), q0);
+    return fma(fma(-b, q, a), y, q);
+}
+__device__ __forceinline__ float quotient(float a, float b) { return a / b; }
+
 // Fluid velocity at a particle with fractional offsets (fx, fy, fz) in its
 // cell, Eq. (5): corners k = ox + 2 oy + 4 oz = 0..7 with weights
 // delta_k = wx wy wz, u(R) = sum_k delta_k j_k / rho_k.  fetch(q, n0, n1)
@@ -61,19 +82,6 @@ struct PArgs {
 // x and x + 1); every caller sums in this one order with explicit fused
 // multiply-adds, so the paths that fetch the records differently agree bit
 // for bit whatever the compiler would contract.
-// FP64 quotient: the reciprocal's approximation (rcp.approx.ftz.f64, about 20
-// bits), one cubic step, then the quotient corrected by its residual -- 6
-// operations of the FP64 pipe, within the last place of the IEEE division.
-__device__ __forceinline__ double quotient(double a, double b) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-    const double h = fma(-b, y, 1.0);
-    y = fma(y, fma(h, h, h), y);
-    const double q = a * y;
-    return fma(fma(-b, q, a), y, q);
-}
-__device__ __forceinline__ float quotient(float a, float b) { return a / b; }
-
 template <typename T>
 __device__ __forceinline__ void add_corner(T weight, T rho, T jx, T jy, T jz, T &ux, T &uy, T &uz) {
     const T w = quotient(weight, rho);

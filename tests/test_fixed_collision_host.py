@@ -40,3 +40,10 @@ def test_error_and_range(program, rho0):
         assert worst <= 12, (rel, worst)
         # 19 rounding errors of rms 5e-18 a node, 80 nodes: 2.5e-18; five times that
         assert abs(mass) <= 1.25e-17, (rel, mass)
+
+
+def test_reciprocal_and_root(program):
+    # 1/rho and sqrt(rho) over every density rho0 in 2^-60 .. 2^60 admits: half a
+    # unit of the last place for the final rounding, and little else
+    inv, root = [float(v) for v in subprocess.check_output([program, "factors"], text=True).split()]
+    assert 0 < inv <= 0.51 and 0 < root <= 0.51, (inv, root)
