@@ -128,10 +128,11 @@ __host__ __device__ __forceinline__ long long to_fixed(double v, int scale) {
 
 // a b rounded to an integer (half away from zero, of the product's leading 62
 // bits or more); *fits: whether that holds (always for |a b| < 2^61, never for
-// 2^62 and more, infinity or NaN).
+// 2^62 and more, or with a factor that is infinite or NaN, also where the other
+// is 0).
 __host__ __device__ __forceinline__ long long product_fixed(double a, double b, bool *fits) {
     const unsigned long long u = bits_of(a), v = bits_of(b);
-    const int ex = (int)((u >> 52) & 0x7ffu) + (int)((v >> 52) & 0x7ffu);
+    const int eu = (int)((u >> 52) & 0x7ffu), ev = (int)((v >> 52) & 0x7ffu), ex = eu + ev;
 #ifdef __CUDA_ARCH__
     const unsigned long long p = __umul64hi((u << 11) | (1ull << 63), (v << 11) | (1ull << 63));
 #else
@@ -139,7 +140,7 @@ __host__ __device__ __forceinline__ long long product_fixed(double a, double b, 
         (unsigned long long)(((unsigned __int128)((u << 11) | (1ull << 63)) * ((v << 11) | (1ull << 63))) >> 64);
 #endif
     int r = 2 * 1023 + 62 - ex;  // a b = p 2^(ex - 2046 - 62), 2^62 <= p < 2^64
-    *fits = r >= 2;
+    *fits = r >= 2 && (eu > ev ? eu : ev) < 0x7ff;
     r = r < 1 ? 1 : r > 65 ? 65 : r;
     const unsigned long long q = r == 65 ? 0ull : ((p >> (r - 1)) + 1ull) >> 1;
     const long long s = (long long)(u ^ v) >> 63;

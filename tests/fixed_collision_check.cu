@@ -173,7 +173,46 @@ static void factors(int lo, int hi, int count) {
     std::printf("%.6f %.6f\n", wi, ws);
 }
 
+// product_fixed against quadruple precision (half away from zero, of at least 62
+// leading bits), and the products it may not call fitting.  Prints the number of
+// wrong answers of each kind.
+static void products(int count) {
+    std::mt19937_64 gen(7);
+    std::uniform_real_distribution<double> U(-1, 1);
+    long wrong = 0, outside = 0, unfit = 0;
+    for (int t = 0; t < count; ++t) {
+        const double a = std::ldexp(U(gen), -(int)(gen() % 80)), b = std::ldexp(U(gen), (int)(gen() % 70));
+        const double z = t % 50 ? a : 0.0;
+        bool fits;
+        const long long v = product_fixed(z, b, &fits);
+        const Quad x = (Quad)z * (Quad)b;
+        const double mag = std::fabs((double)x);
+        if (mag < std::ldexp(1.0, 61) && !fits) ++outside;
+        if (fits) {
+            const Quad d = (Quad)v - x, half = (Quad)0.5 + (Quad)mag * (Quad)std::ldexp(1.0, -62);
+            if (d > half || d < -half) ++wrong;
+        }
+    }
+    const double inf = HUGE_VAL, nan = std::nan(""), tiny = 4.9e-324, big = std::ldexp(1.0, 31);
+    for (double s : {1.0, -1.0})
+        for (double b : {inf, nan, -inf})
+            for (double a : {0.0, -0.0, tiny, 2.2e-308, 1e-300, 0.5, 1.0, big, inf, nan}) {
+                bool f1, f2;
+                product_fixed(s * a, b, &f1);
+                product_fixed(b, s * a, &f2);
+                unfit += f1 + f2;
+            }
+    bool fits;
+    product_fixed(big, big, &fits);
+    unfit += fits;
+    std::printf("%ld %ld %ld\n", wrong, outside, unfit);
+}
+
 int main(int argc, char **argv) {
+    if (argc > 1 && argv[1][0] == 'p') {
+        products(2000000);
+        return 0;
+    }
     if (argc > 1 && argv[1][0] == 'f') {
         factors(-65, 64, 2000000);
         return 0;

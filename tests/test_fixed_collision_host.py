@@ -47,3 +47,9 @@ def test_reciprocal_and_root(program):
     # unit of the last place for the final rounding, and little else
     inv, root = [float(v) for v in subprocess.check_output([program, "factors"], text=True).split()]
     assert 0 < inv <= 0.51 and 0 < root <= 0.51, (inv, root)
+
+
+def test_product_as_an_integer(program):
+    # rounded right wherever it says it fits, fitting below 2^61, and never
+    # fitting with a factor that is not finite, whatever the other one
+    assert subprocess.check_output([program, "products"], text=True).split() == ["0", "0", "0"]
