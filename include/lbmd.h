@@ -111,11 +111,13 @@ enum { LBMD_INTEGRATOR_START = 0, LBMD_INTEGRATOR_HALF_STEP = 1 };
  * bonds or Lennard-Jones forces, nx <= 512, ny and nz >= 6; otherwise ROWS is
  * used; measured slower than ROWS at 0.06 particles per node).  AUTO: ATOMIC
  * while there are fewer than LBMD_SPREAD_ATOMIC_PER_ROW particles per lattice
- * row (y, z) on average (10 in FP64), ROWS above (measured crossover: 256^3
- * nodes, m = 10, us per cycle ATOMIC / ROWS: 6.1 per row 1065 / 1211, 9.9 per
- * row 1384 / 1432, 15.3 per row 1780 / 1672; 128^3: 15.3 per row 360 / 381,
- * 30.5 per row 548 / 491).  The transfers are
- * fixed-point integers, so all of them give bitwise the same results. */
+ * row (y, z) on average, ROWS above (measured crossover, FP32, m = 10, us per
+ * cycle ATOMIC / ROWS: 256 x 192 x 192 nodes 12 per row 820 / 840, 15 per row
+ * 950 / 936; 192 x 160 x 160 12 per row 546 / 553, 14 per row 590 / 584; 128^3
+ * 12 per row 329 / 342, 16 per row 378 / 373), in FP64 always (128^3: 10 per row
+ * 1111 / 1355, 64 per row 3853 / 4148, 128 per row 7046 / 7387; other boxes,
+ * variants, integrators and bonds alike).  The transfers are fixed-point
+ * integers, so all of them give bitwise the same results. */
 enum { LBMD_SPREAD_AUTO = 0, LBMD_SPREAD_ROWS = 1, LBMD_SPREAD_ATOMIC = 2, LBMD_SPREAD_TILES = 3 };
 /* Distribution of the random numbers of the thermal noise (fluid modes,
  * Sec. 2) and of the particles' random force (Eq. (4)); both have zero mean

@@ -11,8 +11,8 @@
 // forcing part of the collision (apply_transfer), once per LB step.
 //
 // The post-stream moments rho* and j* of the freshly streamed populations
-// (the node field the MD steps of the next LB cycle read and, in variant B,
-// update, plus the compact record of every active node) are fused into
+// (the node field the MD steps of the next LB cycle read and, in variants B and
+// C, update, plus the compact record of every active node) are fused into
 // lb_collide_push: a block computes them for the node row two planes back,
 // once the 27 blocks around that row have pushed (per-block flags tagged with
 // the LB step); moments_rest_kernel covers the rows the dataflow cannot
@@ -67,8 +67,7 @@ __device__ __forceinline__ typename Prec<T>::node4 guarded_record(const NodeSums
 }
 
 // Post-stream moments rho*, j* (Eqs. (1), (2)) of node (x, y, t): the node
-// record and, for an active node of the coming cycle (variant B), its
-// compact record.  The populations are read through L2 (ld.global.cg): they
+// record and, for an active node of the coming cycle, its compact record.  The populations are read through L2 (ld.global.cg): they
 // were written by other blocks of the same kernel.
 template <typename T, typename S>
 __device__ __forceinline__ void node_moments_at(const S *f, typename Prec<T>::node4 *node, const uint2 *occw,
@@ -561,8 +560,7 @@ static cudaError_t init_equilibrium_t(lbmd_ctx *ctx) {
                                               : FN<float, float>(__VA_ARGS__))
 
 // One LB update: re-order the particles by row and build the active nodes of
-// the coming cycle (variant B; the particles do not move during the LB
-// step), then collide and stream with the post-stream moments fused in
+// the coming cycle (the particles do not move during the LB step), then collide and stream with the post-stream moments fused in
 // (node field and the new active nodes' compact records).
 cudaError_t launch_lb_step(lbmd_ctx *ctx) {
     cudaError_t e = launch_reorder(ctx);

@@ -1,7 +1,9 @@
 // lb_core.cuh -- the MRT collision with thermal noise and forcing at one
 // node (Sec. 2 collision operator, Sec. 3 forcing term), shared by the
-// single-box LB kernel (lb.cu) and the batched replicas (batch.cu), so that
-// both run one instruction sequence.
+// single-box LB kernel (lb.cu), the batched replicas (batch.cu) and the adjoint's
+// forward pass (adjoint.cu), which run one instruction sequence -- but for the
+// single box in FP64, whose nodes mostly take the integer form of lb_fixed.cuh
+// (the same collision, other roundings).
 #pragma once
 
 #include "lbmd_device.cuh"

@@ -512,9 +512,10 @@ struct PopStore<bf16_sr, float> {
     static constexpr bool stochastic = true;
 };
 
-// Hydrodynamic moments rho = sum f_i, j = sum f_i c_i (Eqs. (1), (2)).  One
-// fixed summation order, shared by every kernel that needs them, so the
-// values are bitwise identical wherever they are recomputed.
+// Hydrodynamic moments rho = sum f_i, j = sum f_i c_i (Eqs. (1), (2)) in one
+// fixed summation order, so the values are bitwise identical wherever they are
+// recomputed.  (The single box in FP64 sums most nodes as integers: node_sums in
+// lb_fixed.cuh, in the same way wherever it recomputes them.)
 template <typename T>
 __device__ __forceinline__ void node_moments(const T f[Q], T &rho, T &jx, T &jy, T &jz) {
     T s[9], d[9];  // sums and differences of opposite velocities

@@ -21,8 +21,7 @@
 // (y, z) of their cell (counting sort: count, scan, scatter), so that a warp
 // handles particles whose corner nodes lie in a few neighbouring rows.
 //
-// active_*: variant B, after each re-ordering: the corners of the particles'
-// cells become the active nodes, numbered row by row into a compact array of
+// active_*: after each re-ordering: the corners of the particles' cells become the active nodes, numbered row by row into a compact array of
 // node records (filled by the post-stream moments of the LB step).  Between
 // LB updates the MD kernels read and update an active node through its
 // compact record, which is about as large as the touched part of the lattice
@@ -671,7 +670,7 @@ __global__ void __launch_bounds__(256) sort_scatter_kernel(ScatterArgs<T> a, con
 }
 
 // ---------------------------------------------------------------------------
-// Active nodes (variants A and B), rebuilt after each re-ordering.
+// Active nodes, rebuilt after each re-ordering.
 // ---------------------------------------------------------------------------
 // Level 0: node x of row (y, z) is active when a particle's cell has it as a
 // corner, i.e. when cell x or x - 1 (periodic) of one of the four cell rows
@@ -983,8 +982,8 @@ static PArgs<T> make_pargs(lbmd_ctx *ctx, int substep) {
 static bool spreads_atomic(const lbmd_ctx *ctx) {
     return ctx->p.spread == LBMD_SPREAD_ATOMIC ||
            (ctx->p.spread == LBMD_SPREAD_AUTO &&
-            // (the FP64 atomics, a thread per particle, cross over earlier)
-            ctx->np < (int64_t)(ctx->p.precision == LBMD_FP64 ? 10 : LBMD_SPREAD_ATOMIC_PER_ROW) * ctx->p.ny * ctx->p.nz);
+            // (FP64: the faster at every density; the figures stand at LBMD_SPREAD_AUTO)
+            (ctx->p.precision == LBMD_FP64 || ctx->np < (int64_t)LBMD_SPREAD_ATOMIC_PER_ROW * ctx->p.ny * ctx->p.nz));
 }
 
 // `count` MD steps from `substep` on in one launch, where the system allows it.
