@@ -311,8 +311,8 @@ __device__ __forceinline__ void collide_push_node(const LbArgs<T, S> &a, int x, 
 }
 
 // Resident blocks per SM the compiler plans registers for.  FP32 storage: 6 (40
-// registers; two cycles at 256^3 with 10^6 particles 3396 us, 5 blocks 3461,
-// 7 blocks, with spills, 3482).  Rounded-to-nearest 16-bit storage with full
+// registers; two cycles at 256^3 with 10^6 particles 3341 us, 5 blocks 3406,
+// 7 blocks, with spills, 3425).  Rounded-to-nearest 16-bit storage with full
 // relaxation and uniform noise: 7 (3183 us, 6 blocks 3287); the stochastic
 // rounding form measured slower at 7.  Variant C 5.  FP64: 2 with the
 // collision in integers (128 registers), 3 in its FP64 form.

@@ -78,7 +78,7 @@ void free_all(lbmd_ctx *ctx) {
     }
     if (ctx->obs_ready) cudaEventDestroy(ctx->obs_ready);
     if (ctx->obs_host) cudaFreeHost(ctx->obs_host);
-    if (ctx->host_error) cudaFreeHost(ctx->host_error);
+    if (ctx->host_error && ctx->host_error != &ctx->host_word) cudaFreeHost(ctx->host_error);
     if (ctx->up_stream) cudaStreamDestroy(ctx->up_stream);
     if (ctx->down_stream) cudaStreamDestroy(ctx->down_stream);
     for (int i = 0; i < 16; ++i)
@@ -275,7 +275,15 @@ lbmd_status lbmd_create(const lbmd_params *p, lbmd_ctx **out) {
             return s;
         }
     }
-    cudaError_t e = cudaHostAlloc((void **)&ctx->host_error, sizeof(int32_t), cudaHostAllocMapped);
+    // the host's copy of the error flag: a GPU that shares the host's page tables
+    // writes it in place; elsewhere a pinned page, which takes 110 us to allocate
+    cudaError_t e = cudaSuccess;
+    int pageable = 0;
+    cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, dev);
+    if (pageable)
+        ctx->host_error = &ctx->host_word;
+    else
+        e = cudaHostAlloc((void **)&ctx->host_error, sizeof(int32_t), cudaHostAllocMapped);
     if (e == cudaSuccess) *ctx->host_error = 0;
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_lb_step, 0, sizeof(unsigned long long), ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->missed_total, 0, sizeof(unsigned long long), ctx->stream);

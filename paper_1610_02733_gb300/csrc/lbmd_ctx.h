@@ -181,7 +181,8 @@ struct lbmd_ctx {
     // that write a node record whose momentum reaches half the range
     int32_t *range_flag;
     int32_t *dev_error;   // set by a kernel whose bounded wait gave up
-    int32_t *host_error;  // the same in mapped host memory
+    int32_t *host_error;  // the same in host memory the GPU writes: host_word, or pinned memory
+    int32_t host_word;
     FixUnit fix;
     int red_blocks;
     unsigned long long *d_lb_step;  // LB step counter read by the kernels

@@ -54,7 +54,8 @@ namespace lbmd {
 // pair kernel otherwise), transfer around the start position.
 // The variant is a run-time flag (one instruction sequence for both
 // variants, as in the LB kernel).  Bound by the latency of the scattered
-// corner loads (16 B records, 33 % of the issue slots busy): 8 records in
+// corner loads (16 B records; 34 % of the issue slots busy, 12 cycles of waiting on
+// a load per instruction, DRAM at 31 %): 8 records in
 // flight per thread (corner_records) need 64 registers, and 8 blocks of 128
 // threads of them per SM measured faster (42 us at 256^3 nodes and 10^6
 // particles, FP32) than 4 of 256 (44 us), 6 of 128 (45 us) or 5 of 256 with
