@@ -770,7 +770,8 @@ cudaError_t setup_phases(lbmd_adjoint *ad) {
 
 // one cycle's MD steps from the checkpoint of cycle c (node field from the
 // checkpointed populations), optionally recording every MD step; the particles
-// end in the checkpoint of cycle c + 1, where its recomputation leaves the same
+// end in the checkpoint of cycle c + 1 (the run that records finds them there
+// already, or writes the same)
 template <typename T>
 cudaError_t run_md(lbmd_adjoint *ad, int c, bool record) {
     using R4 = typename Prec<T>::real4;
@@ -810,6 +811,7 @@ cudaError_t run_md(lbmd_adjoint *ad, int c, bool record) {
                                                             static_cast<N4 *>(ad->node));
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
+    if (record) return cudaSuccess;
     if ((e = cudaMemcpyAsync(next, ad->pos, np * sizeof(R4), cudaMemcpyDeviceToDevice, ad->stream)) != cudaSuccess)
         return e;
     return cudaMemcpyAsync(next + np, ad->vel, np * sizeof(R4), cudaMemcpyDeviceToDevice, ad->stream);
