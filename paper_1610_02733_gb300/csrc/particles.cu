@@ -1146,24 +1146,20 @@ static cudaError_t sort_t(lbmd_ctx *ctx) {
     const int W = active_words(ctx->p.nx);
     cudaError_t e = cudaMemsetAsync(ctx->row_count, 0, (size_t)rows * sizeof(int32_t), ctx->stream);
     if (e != cudaSuccess) return e;
-    if (ctx->np > 0 &&
-        (e = cudaMemsetAsync(ctx->ccw, 0, (size_t)rows * W * sizeof(uint32_t), ctx->stream)) != cudaSuccess)
-        return e;
-    if (ctx->np > 0) {
-        const ScatterArgs<T> a = scatter_args<T>(ctx);
-        const unsigned blocks = (unsigned)((ctx->np + 255) / 256);
-        sort_count_kernel<T><<<blocks, 256, 0, ctx->stream>>>(a.pos_in, ctx->np, a.fnx, ctx->row_count, ctx->sort_rank,
-                                                                ctx->ccw, W);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        const int n_chunks = (int)((rows + 1023) / 1024);
-        sort_chunk_scan_kernel<<<n_chunks, 1024, 0, ctx->stream>>>(ctx->row_count, rows, ctx->chunk_total);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        sort_finalize_kernel<<<n_chunks, 1024, 0, ctx->stream>>>(ctx->row_count, ctx->chunk_total, rows,
-                                                                 ctx->row_start, (int32_t)ctx->np);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        sort_scatter_kernel<T><<<blocks, 256, 0, ctx->stream>>>(a, ctx->row_start);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
+    if ((e = cudaMemsetAsync(ctx->ccw, 0, (size_t)rows * W * sizeof(uint32_t), ctx->stream)) != cudaSuccess) return e;
+    const ScatterArgs<T> a = scatter_args<T>(ctx);
+    const unsigned blocks = (unsigned)((ctx->np + 255) / 256);
+    sort_count_kernel<T><<<blocks, 256, 0, ctx->stream>>>(a.pos_in, ctx->np, a.fnx, ctx->row_count, ctx->sort_rank,
+                                                            ctx->ccw, W);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const int n_chunks = (int)((rows + 1023) / 1024);
+    sort_chunk_scan_kernel<<<n_chunks, 1024, 0, ctx->stream>>>(ctx->row_count, rows, ctx->chunk_total);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    sort_finalize_kernel<<<n_chunks, 1024, 0, ctx->stream>>>(ctx->row_count, ctx->chunk_total, rows, ctx->row_start,
+                                                             (int32_t)ctx->np);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    sort_scatter_kernel<T><<<blocks, 256, 0, ctx->stream>>>(a, ctx->row_start);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     ctx->pcur ^= 1;
     ctx->pv ^= 1;
     return cudaSuccess;
@@ -1175,11 +1171,6 @@ static cudaError_t active_set_t(lbmd_ctx *ctx) {
     const int W = active_words(ctx->p.nx);
     uint2 *occw = active_words_next(ctx);  // built for the coming LB cycle
     int32_t *arow = ctx->arow[(ctx->lb_step + 1) & 1];
-    if (ctx->np == 0) {
-        cudaError_t e = cudaMemsetAsync(occw, 0, (size_t)rows * W * sizeof(uint2), ctx->stream);
-        if (e != cudaSuccess) return e;
-        return cudaMemsetAsync(arow, 0, (size_t)(rows + 1) * sizeof(int32_t), ctx->stream);
-    }
     int L = 1;
     while (L < W && L < 32) L <<= 1;
     const int64_t warps = (rows + (32 / L) - 1) / (32 / L);
@@ -1205,7 +1196,7 @@ static cudaError_t active_set_t(lbmd_ctx *ctx) {
 // 745 / 746, 812 / 806, 879 / 873); 96 x 128 x 128, 150,000: 136 / 140 (575 / 578).
 static bool reorder_fits(const lbmd_ctx *ctx) {
     const int64_t threads = (int64_t)ctx->sm_count * REORDER_THREADS;
-    return ctx->np > 0 && (int64_t)ctx->p.ny * ctx->p.nz <= threads && ctx->np <= 4 * threads;
+    return (int64_t)ctx->p.ny * ctx->p.nz <= threads && ctx->np <= 4 * threads;
 }
 template <typename T>
 static cudaError_t reorder_t(lbmd_ctx *ctx) {
@@ -1264,6 +1255,8 @@ static cudaError_t launch_sort_particles(lbmd_ctx *ctx);
 cudaError_t launch_reorder(lbmd_ctx *ctx) {
     const bool dbl = ctx->p.precision == LBMD_FP64;
     cudaError_t e;
+    // without particles both sets are empty, as lbmd_create left them
+    if (ctx->np == 0) return cudaMemsetAsync(ctx->lb_missed, 0, sizeof(int32_t), ctx->stream);
     if (lbmd::reorder_fits(ctx)) {
         ctx->in_buckets = true;
         if ((e = dbl ? lbmd::reorder_t<double>(ctx) : lbmd::reorder_t<float>(ctx)) != cudaSuccess) return e;

@@ -3,6 +3,7 @@ with the row gather, whatever the particles do meanwhile."""
 import numpy as np
 import pytest
 
+from gpu_common import assert_pops_close, assert_vec_close, pair
 from paper_1610_02733_gb300 import inputs, lbmd
 
 pytestmark = pytest.mark.gpu
@@ -93,3 +94,22 @@ def test_fp64_bonds_at_the_limit_of_the_teams(n):
         g.close()
     _same(out[1], out[0])
     _same(out[2], out[0])
+
+
+@pytest.mark.parametrize("variant", ["A", "B", "C"])
+@pytest.mark.parametrize("empty", [1, 2, 3])
+def test_particles_added_after_empty_cycles(variant, empty):
+    # both active sets are empty until the first particle, whichever the cycle
+    # that it comes in takes
+    o, g = pair((14, 9, 10), variant=variant, n_sub=3, kT=1e-4, zeta=0.7, seed=5, max_particles=60,
+                body_force=(1e-4, 0.0, 0.0))
+    o.cycle(empty)
+    g.run_cycles(empty)
+    pos, vel = inputs.uniform_positions(60, (14, 9, 10), 2), inputs.maxwell_velocities(60, 1e-3, 2)
+    for s in (o, g):
+        s.add_particles(pos, vel)
+        s.cycle(2)
+    assert_pops_close(g.populations(), o.populations(), "fp32")
+    assert_vec_close(g.particles()[1], o.particles()[1], "fp32", "velocities")
+    g.close()
+    o.close()
