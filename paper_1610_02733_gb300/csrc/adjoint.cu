@@ -821,6 +821,7 @@ cudaError_t run_md(lbmd_adjoint *ad, int c, bool record) {
 // synchronises.  The words and the flag start over: lbmd_adjoint_forward
 // recomputes everything from its arguments.
 cudaError_t check_phases(lbmd_adjoint *ad) {
+    if (!in_phases(ad)) return cudaStreamSynchronize(ad->stream);
     int32_t gave_up = 0;
     cudaError_t e = cudaMemcpyAsync(&gave_up, ad->phase_words + 2, sizeof(gave_up), cudaMemcpyDeviceToHost, ad->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ad->stream);
